@@ -706,7 +706,7 @@ def run_gpu(args):
     ms_prof, _ = timed(step, args.steps)
     dwt.dwt_profile_enable(False)
     fams = {}
-    for name in ("interp_fwd", "interp_top", "interp_inv", "interp_inv_fwd", "effdim_classes", "effdim_finalize"):
+    for name in ("interp_fwd", "interp_top", "interp_inv", "interp_inv_fwd", "effdim_reduce"):
         n, tot = dwt.dwt_profile_query(name)
         if n:
             fams[name] = (n, tot)

@@ -503,7 +503,7 @@ long long dwt_alloc_count(void);
  * "p2_hi_inv"; p = 2 interpolation "interp_fwd", "interp_top", "interp_inv",
  * "interp_inv_fwd" (two low passes in one launch); tensor-core tiles
  * "tc_lo14"; generic passes "pass_lo", "pass_mid", "pass_hi"; variance classes
- * "effdim_bins", "effdim_classes", "effdim_finalize"; index maps "points",
+ * "effdim_bins", "effdim_reduce"; index maps "points",
  * "k_to_h", "h2k_recon", "h2k_copy"; plan build "dp_init", "dp_step",
  * "dp_check", "dp_prefix", "dp_recon", "dp_weights", "dp_small",
  * "tile_tables"; test functions "eval_product", "eval_exp".

@@ -175,6 +175,9 @@ static inline EffOut eff_packed(double* var, int* dim, int nb) {
     o.dstride = 2;
     return o;
 }
+// class partials part [batch][2 nb][nchunk] -> the outputs of o (one launch)
+int effdim_reduce(const double* part, long long nchunk, int nb, int batch, double thr, const EffOut& o,
+                  cudaStream_t st);
 int run_effdim(dwt_plan_s* P, const void* coef, int batch, long long ld, dwt_dtype t, const EffOut& o, double thr,
                cudaStream_t st);
 // tensor-core low pass (p = 2, low 14 digits): one job of ntiles tiles of

@@ -576,7 +576,7 @@ int p2_interpolate(dwt_plan_s* Pl, const float* f, float* c, float* coef, int ba
         return DWT_EUNSUPPORTED;
     }
     const long long ntile = N >> LT;
-    int rc = ensure_workspace(Pl, (size_t)batch * (ntile + 1) * nb2 * sizeof(double), st);
+    int rc = ensure_workspace(Pl, (size_t)batch * ntile * nb2 * sizeof(double), st);
     if (rc) return rc;
     double* part = (double*)Pl->d_ws;
     const long long fbytes = N * 4;

@@ -841,7 +841,7 @@ int p2i_interpolate(dwt_plan_s* Pl, const float* f, float* c, float* coef, int b
         return DWT_ETIMEOUT;
     }
     const long long ntile = N >> kTopLT;
-    int rc = ensure_workspace(Pl, (size_t)batch * (ntile + 1) * nb2 * sizeof(double), st);
+    int rc = ensure_workspace(Pl, (size_t)batch * ntile * nb2 * sizeof(double), st);
     if (rc) return rc;
     double* part = (double*)Pl->d_ws;
     int G = (int)std::max(1ll, kL2GroupP2i / (N * 4));

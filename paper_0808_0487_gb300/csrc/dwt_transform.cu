@@ -27,6 +27,10 @@ int p2_transform(dwt_plan_s* Pl, const void* in, void* out, int batch, long long
 int p2_interpolate(dwt_plan_s* Pl, const float* f, float* c, float* coef, int batch, long long ld, const float* W,
                    bool tc, double** part_out, long long* ntile_out, cudaStream_t st);
 
+bool p2_small_ok(int m);
+int p2_small_interpolate(dwt_plan_s* Pl, const float* f, float* c, float* coef, int batch, long long ld,
+                         bool weighted, double thr, const EffOut& o, cudaStream_t st);
+
 static bool aligned16(const void* p, long long ld, int elem) {
     return ((uintptr_t)p & 15) == 0 && ((ld * elem) & 15) == 0;
 }
@@ -520,64 +524,6 @@ __global__ void __launch_bounds__(256) k_effdim_bins(const T* coef, long long ld
     reduce_bins(bins, nb2, blockDim.x >> 5, part + fn * nb2 * nchunk + chunk, nchunk);
 }
 
-// partials part[fn][class][tile] -> per-class totals: one block per (class,
-// function); thread t sums tiles t, t+256, ... in order, then a fixed tree.
-__global__ void __launch_bounds__(256) k_effdim_classes(const double* __restrict__ part, long long nchunk, int nb2,
-                                                        double* csum) {
-    __shared__ double red[256];
-    const int bi = blockIdx.x;
-    const long long fn = blockIdx.y;
-    const double* pp = part + (fn * nb2 + bi) * nchunk;
-    double acc = 0.0;
-    long long t = threadIdx.x;
-    for (; t + 3 * 256 < nchunk; t += 4 * 256) {   // four loads in flight, added in order
-        const double a0 = pp[t], a1 = pp[t + 256], a2 = pp[t + 512], a3 = pp[t + 768];
-        acc += a0;
-        acc += a1;
-        acc += a2;
-        acc += a3;
-    }
-    for (; t < nchunk; t += 256) acc += pp[t];
-    red[threadIdx.x] = acc;
-    __syncthreads();
-    for (int o = 128; o > 0; o >>= 1) {
-        if ((int)threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) csum[fn * nb2 + bi] = red[0];
-}
-
-// per-class totals -> cumulative truncation / superposition variances and dimensions
-__global__ void __launch_bounds__(32) k_effdim_finalize(const double* __restrict__ csum, int nb, double thr, EffOut o,
-                                                         int batch) {
-    // one warp per function: the class totals come into shared memory together,
-    // then lane 0 forms the cumulative sums in class order
-    __shared__ double c[2 * 256];
-    const int fn = blockIdx.x;
-    if (fn >= batch) return;
-    const double* cs_ = csum + (long long)fn * 2 * nb;
-    for (int i = threadIdx.x; i < 2 * nb; i += 32) c[i] = cs_[i];
-    __syncwarp();
-    if (threadIdx.x != 0) return;
-    double tot = 0.0;
-    for (int d = 0; d < nb; ++d) tot += c[d];
-    double ct = 0.0, cs = 0.0;
-    int dt = 0, ds = 0;
-    bool ft = false, fs = false;
-    for (int d = 0; d < nb; ++d) {
-        ct += c[d];
-        cs += c[nb + d];
-        if (o.vt) o.vt[(long long)fn * o.vstride + d] = ct;
-        if (o.vs) o.vs[(long long)fn * o.vstride + d] = cs;
-        if (tot > 0.0) {
-            if (!ft && ct >= thr * tot) { dt = d; ft = true; }
-            if (!fs && cs >= thr * tot) { ds = d; fs = true; }
-        }
-    }
-    if (o.dt) o.dt[(long long)fn * o.dstride] = dt;
-    if (o.ds) o.ds[(long long)fn * o.dstride] = ds;
-}
-
 // ---------------------------------------------------------------------------
 // host side
 static Tw make_tw(int p) {
@@ -948,23 +894,7 @@ static int bins_warps(size_t tile_bytes, int nb2, size_t budget = 227 * 1024, in
 
 static int finalize(dwt_plan_s* Pl, const double* part, long long nchunk, int batch, double thr, const EffOut& o,
                     cudaStream_t st) {
-    if (!o.vt && !o.vs && !o.dt && !o.ds) return DWT_OK;
-    const int nb = Pl->s + 1, nb2 = 2 * nb;
-    // per-class totals go right after the partials in the workspace
-    double* csum = const_cast<double*>(part) + (size_t)batch * nb2 * nchunk;
-    for (int f0 = 0; f0 < batch; f0 += 65535) {
-        const int nf = std::min(65535, batch - f0);
-        LaunchScope ls("effdim_classes", st);
-        k_effdim_classes<<<dim3((unsigned)nb2, (unsigned)nf), 256, 0, st>>>(part + (size_t)f0 * nb2 * nchunk, nchunk,
-                                                                            nb2, csum + (size_t)f0 * nb2);
-    }
-    DWT_CK_LAUNCH("k_effdim_classes");
-    {
-        LaunchScope ls("effdim_finalize", st);
-        k_effdim_finalize<<<batch, 32, 0, st>>>(csum, nb, thr, o, batch);
-    }
-    DWT_CK_LAUNCH("k_effdim_finalize");
-    return DWT_OK;
+    return effdim_reduce(part, nchunk, Pl->s + 1, batch, thr, o, st);
 }
 
 template <int P, typename T, typename TI>
@@ -986,7 +916,7 @@ static int interpolate_t(dwt_plan_s* Pl, const void* f, void* c, void* coef, int
         return DWT_EUNSUPPORTED;
     }
     const size_t smem = ((tile_bytes + 15) & ~(size_t)15) + (size_t)nw * nb2 * 32 * 4;
-    int rc = ensure_workspace(Pl, (size_t)batch * (ntile + 1) * nb2 * sizeof(double), st);
+    int rc = ensure_workspace(Pl, (size_t)batch * ntile * nb2 * sizeof(double), st);
     if (rc) return rc;
     double* part = (double*)Pl->d_ws;
     auto kmid_first = k_mid<P, T, TI, KM>;   // single pass: reads f directly
@@ -1067,6 +997,9 @@ int run_interpolate(dwt_plan_s* Pl, const void* f, void* c, void* coef, int batc
         if (rc) return rc;
         return finalize(Pl, part, ntile, batch, thr, eff_packed(var, dim, Pl->s + 1), st);
     }
+    if (Pl->p == 2 && p2_small_ok(Pl->m))
+        return p2_small_interpolate(Pl, (const float*)f, (float*)c, (float*)coef, batch, ld,
+                                    weight == DWT_WEIGHT_INV_SQ_WAVENUMBER, thr, eff_packed(var, dim, Pl->s + 1), st);
     switch (Pl->p) {
         case 2: return interpolate_t<2, float, float>(Pl, f, c, coef, batch, ld, weight, var, dim, thr, st);
         case 3:
@@ -1114,7 +1047,7 @@ static int effdim_t(dwt_plan_s* Pl, const void* coef, int batch, long long ld, c
         return DWT_EUNSUPPORTED;
     }
     const size_t smem = (size_t)nw * nb2 * 32 * 4;
-    int rc = ensure_workspace(Pl, (size_t)batch * (nchunk + 1) * nb2 * sizeof(double), st);
+    int rc = ensure_workspace(Pl, (size_t)batch * nchunk * nb2 * sizeof(double), st);
     if (rc) return rc;
     double* part = (double*)Pl->d_ws;
     auto kern = k_effdim_bins<T>;
