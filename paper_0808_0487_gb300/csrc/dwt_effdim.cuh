@@ -30,12 +30,12 @@ __device__ __forceinline__ void effdim_outputs(double* c, int* first, int nb, do
         }
     }
     __syncthreads();
-    const double tot = c[nb - 1], lim = thr * tot;
     for (int i = t; i < 2 * nb; i += blockDim.x) {
         const int k = i >= nb, d = i - k * nb;
+        const double tot = c[nb - 1];
         if (!k && o.vt) o.vt[fn * o.vstride + d] = c[i];
         if (k && o.vs) o.vs[fn * o.vstride + d] = c[i];
-        if (tot > 0.0 && c[i] >= lim) atomicMin(first + k, d);
+        if (tot > 0.0 && c[i] >= thr * tot) atomicMin(first + k, d);
     }
     __syncthreads();
     if (t == 0) {

@@ -73,10 +73,10 @@ def test_small_interpolate(dwt, dev, orc, m, s, pad, weight, inplace):
             assert all(abs(x[d] / vt[-1] - 0.95) < 1e-6 for d in range(lo, hi))
 
 
-# one CTA or a cluster per function (2^18, 2^19 points at s = 255 lie on the two
+# one CTA or a cluster per function (s = 255: 2^15 and 2^16 points lie on the two
 # sides of the line), fewer partials than lanes, odd counts; classes that add
 # nothing leave the dimension at threshold 1 where the last contribution is
-@pytest.mark.parametrize("p,m,s", [(2, 13, 3), (2, 18, 255), (2, 19, 255), (3, 13, 8), (2, 22, 31)])
+@pytest.mark.parametrize("p,m,s", [(2, 13, 3), (2, 15, 255), (2, 16, 255), (3, 13, 8), (2, 22, 31)])
 def test_effdim_reduction(dwt, dev, orc, p, m, s):
     N, B = p ** m, 2
     plan = dwt.dwt_plan(p, m, s, S.small_net(p, m, s, index=60 + m))
