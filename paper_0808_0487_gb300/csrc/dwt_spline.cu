@@ -28,7 +28,7 @@
 #include <algorithm>
 #include <vector>
 
-#include "dwt_internal.cuh"
+#include "dwt_effdim.cuh"
 
 namespace dwt {
 
@@ -141,43 +141,38 @@ __global__ void __launch_bounds__(256) k_spline_dots(const double* __restrict__ 
     }
 }
 
-// sums over tiles in tile order, then the cumulative variances and dimensions
-// (least d with variance >= thr * total, 0 when the total is 0)
-__global__ void k_spline_finalize(const double* __restrict__ part, long long ntile, int s, int batch, double N2,
-                                  double thr, double* var_trc, double* var_sup, int* dim) {
-    const int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b >= batch) return;
-    const int nt = 2 * s;
-    double vt[kSplineMaxS + 1], vs[kSplineMaxS + 1];
-    vt[0] = vs[0] = 0.0;
-    for (int d = 1; d <= s; ++d) {
-        double x = 0.0, y = 0.0;
-        const double* pr = part + ((long long)b * nt + (d - 1)) * ntile;
-        const double* pe = part + ((long long)b * nt + (s + d - 1)) * ntile;
-        for (long long i = 0; i < ntile; ++i) {
-            x += pr[i];
-            y += pe[i];
-        }
-        vt[d] = N2 * x;
-        vs[d] = vs[d - 1] + N2 * y;
+// sums over tiles, then the cumulative variances and dimensions (least d with
+// variance >= thr * total, 0 when the total is 0): one CTA per function.  The
+// FP64 additions of its 2 s ntile partials bound it (p = 2, m = 20, s = 16, 32
+// functions: 553 us with one thread per function, 9 us so).
+constexpr int kFinThreads = 512;
+__global__ void __launch_bounds__(kFinThreads) k_spline_finalize(const double* __restrict__ part, int ntile, int s,
+                                                                 int lg, double N2, double thr, double* var_trc,
+                                                                 double* var_sup, int* dim) {
+    __shared__ double x[2 * kSplineMaxS];
+    __shared__ double v[2][kSplineMaxS + 1];
+    __shared__ int first[2];
+    const long long b = blockIdx.x;
+    const int t = threadIdx.x;
+    sum_rows(part + b * 2 * s * ntile, 2 * s, ntile, lg, 0, 1, x);
+    if (t < 2) first[t] = s;
+    __syncthreads();
+    if (t == 0) {
+        double acc = v[1][0] = 0.0;
+        for (int d = 1; d <= s; ++d) v[1][d] = acc += N2 * x[s + d - 1];
+    } else if (t >= 32 && t <= 32 + s) {
+        v[0][t - 32] = t == 32 ? 0.0 : N2 * x[t - 33];
     }
-    for (int d = 0; d <= s; ++d) {
-        if (var_trc) var_trc[(long long)b * (s + 1) + d] = vt[d];
-        if (var_sup) var_sup[(long long)b * (s + 1) + d] = vs[d];
+    __syncthreads();
+    if (t <= s) {
+        if (var_trc) var_trc[b * (s + 1) + t] = v[0][t];
+        if (var_sup) var_sup[b * (s + 1) + t] = v[1][t];
+        const double lim = thr * v[0][s];
+        if (v[0][t] >= lim) atomicMin(first, t);
+        if (v[1][t] >= lim) atomicMin(first + 1, t);
     }
-    if (dim) {
-        const double tot = vt[s];
-        int dt = 0, ds = 0;
-        if (tot > 0.0) {
-            dt = ds = s;
-            for (int d = s; d >= 0; --d) {
-                if (vt[d] >= thr * tot) dt = d;
-                if (vs[d] >= thr * tot) ds = d;
-            }
-        }
-        dim[2 * b] = dt;
-        dim[2 * b + 1] = ds;
-    }
+    __syncthreads();
+    if (t < 2 && dim) dim[2 * b + t] = v[0][s] > 0.0 ? first[t] : 0;
 }
 
 // kernel data at the shifted points: Kd[w] = prod_j (1 + gamma_j K'(x_{j,w} (+) delta_j, 0)),
@@ -684,8 +679,8 @@ int run_spline(dwt_plan_s* P, const double* f, void* c, int batch, long long ld,
     }
     if (want_var) {
         LaunchScope ls("spline_finalize", st);
-        k_spline_finalize<<<(batch + 127) / 128, 128, 0, st>>>(part, ntile, s, batch, (double)N * (double)N, thr,
-                                                               var_trc, var_sup, dim);
+        k_spline_finalize<<<batch, kFinThreads, 0, st>>>(part, (int)ntile, s, sum_rows_lanes(2 * s, ntile, kFinThreads),
+                                                         (double)N * (double)N, thr, var_trc, var_sup, dim);
     }
     DWT_CK_LAUNCH("k_spline_finalize");
     cleanup();
