@@ -1,0 +1,339 @@
+// dwt_p2d.cu -- the p = 2 transform in FP64 (Algorithms 1 and 2) with its
+// additions in 96-bit integers.
+//
+// This GPU starts one FP64 addition of a warp every 19 cycles per SM but one
+// 96-bit integer addition (three 32-bit ones with carries) every cycle, and the
+// p = 2 transform is additions only.  A pass over a tile therefore turns its
+// samples into fixed point once, runs all its stages exactly, and rounds once
+// to FP64 on the way out.
+//
+// Precision.  The elements that a pass combines (a contiguous tile, or the rows
+// of one column) share the exponent E of their largest.  Their 53-bit
+// significands are placed so that the b stages cannot overflow 95 bits and a
+// sign, which leaves 42 - b >= 30 bits below the largest one's last place:
+// elements down to 2^-30 of it enter exactly, smaller ones within 2^-83 of it.
+// Every result is the exact sum of those, rounded once, where FP64 stages round
+// b times at 2^-53 of the partial sums.  A tile with an infinity or a NaN runs
+// the FP64 stages; results below the normal range go through one FP64 scaling.
+//
+// Tiles are 2^12 elements for 256 threads, 16 elements (48 words) each:
+//   layout A  e = t + 256 r               bits 8..11 of the tile index in thread
+//   layout C  e = 16 t + r                bits 0..3
+//   layout B  e = (t & 15) + 16 r + 256 (t >> 4)    bits 4..7
+// in that order, so that both ends move 128-byte runs.  The low pass takes the
+// 12 low digits of a contiguous tile; a high pass of b digits has 2^b rows
+// (2^d0 apart) of 2^(12-b) consecutive columns, its digits the top b bits of
+// the tile index.
+#include <algorithm>
+
+#include "dwt_internal.cuh"
+
+namespace dwt {
+
+namespace {
+
+constexpr int kLT = 12;              // tile: 2^12 elements
+constexpr int kNT = 256;             // threads, 16 elements each
+constexpr int kPlane = (1 << kLT) + (1 << (kLT - 4));   // words of one limb's plane, one pad word per 16
+
+struct DArgs {
+    const double* in;
+    double* out;
+    long long ld_in, ld_out;
+    long long S;        // row distance (high pass)
+    int exp_shift;      // exponent of the factor: -m in the last pass of a forward transform
+};
+
+__device__ __forceinline__ int plane_pos(int e) { return e + (e >> 4); }
+
+struct W96 {
+    uint32_t a, b, c;   // low, middle, high word
+};
+
+__device__ __forceinline__ void bfly96(W96& x, W96& y) {
+    W96 s, d;
+    asm("add.cc.u32 %0, %3, %6;\n addc.cc.u32 %1, %4, %7;\n addc.u32 %2, %5, %8;"
+        : "=r"(s.a), "=r"(s.b), "=r"(s.c)
+        : "r"(x.a), "r"(x.b), "r"(x.c), "r"(y.a), "r"(y.b), "r"(y.c));
+    asm("sub.cc.u32 %0, %3, %6;\n subc.cc.u32 %1, %4, %7;\n subc.u32 %2, %5, %8;"
+        : "=r"(d.a), "=r"(d.b), "=r"(d.c)
+        : "r"(x.a), "r"(x.b), "r"(x.c), "r"(y.a), "r"(y.b), "r"(y.c));
+    x = s;
+    y = d;
+}
+
+// negate when mask is all ones
+__device__ __forceinline__ W96 negate_if(W96 v, uint32_t mask) {
+    W96 r;
+    asm("sub.cc.u32 %0, %3, %6;\n subc.cc.u32 %1, %4, %6;\n subc.u32 %2, %5, %6;"
+        : "=r"(r.a), "=r"(r.b), "=r"(r.c)
+        : "r"(v.a ^ mask), "r"(v.b ^ mask), "r"(v.c ^ mask), "r"(mask));
+    return r;
+}
+
+__device__ __forceinline__ int exponent_of(uint32_t hi) { return (int)((hi >> 20) & 0x7ffu); }
+
+// significand of a double at 2^g below the largest exponent E (>= 1) of its group
+__device__ __forceinline__ W96 to_fixed(uint32_t hi, uint32_t lo, int E, int g) {
+    const int ex = exponent_of(hi);
+    uint32_t mh = hi & 0xfffffu;
+    if (ex) mh |= 0x100000u;
+    const int d = min(E - max(ex, 1), 95);
+    // significand << g, g = 30 .. 38: up to 91 bits; right by d in two steps
+    W96 v;
+    if (g >= 32) {
+        v.a = 0;
+        v.b = lo << (g - 32);
+        v.c = __funnelshift_l(lo, mh, g - 32);
+    } else {
+        v.a = lo << g;
+        v.b = __funnelshift_l(lo, mh, g);
+        v.c = mh >> (32 - g);
+    }
+    if (d >= 64) {
+        v.a = v.c;
+        v.b = v.c = 0;
+    } else if (d >= 32) {
+        v.a = v.b;
+        v.b = v.c;
+        v.c = 0;
+    }
+    const int r = d & 31;
+    v.a = __funnelshift_r(v.a, v.b, r);
+    v.b = __funnelshift_r(v.b, v.c, r);
+    v.c >>= r;
+    return negate_if(v, (uint32_t)((int)hi >> 31));
+}
+
+// fixed point -> nearest double (ties to even), times 2^shift
+__device__ __forceinline__ double from_fixed(W96 v, int E, int g, int shift) {
+    const uint32_t sign = (uint32_t)((int)v.c >> 31);
+    v = negate_if(v, sign);
+    int e = 95 + E - 52 - g + shift;   // exponent field of bit 95
+    if (v.c == 0) {
+        v.c = v.b;
+        v.b = v.a;
+        v.a = 0;
+        e -= 32;
+    }
+    if (v.c == 0) {
+        v.c = v.b;
+        v.b = 0;
+        e -= 32;
+    }
+    const int lz = __clz((int)v.c);   // 32 when the value is zero
+    if (lz == 32) return 0.0;
+    e -= lz;
+    v.c = __funnelshift_l(v.b, v.c, lz);
+    v.b = __funnelshift_l(v.a, v.b, lz);
+    v.a <<= lz;
+    // 53 bits of c:b, the rest rounds
+    uint32_t uh = v.c >> 11, ul = __funnelshift_r(v.b, v.c, 11);
+    const uint32_t rem = (v.b & 0x7ffu) | (v.a ? 1u : 0u);
+    const uint32_t up = rem + (ul & 1u) > 0x400u ? 1u : 0u;
+    const bool tiny = e < 1, huge = e >= 0x7ff;
+    const int ef = tiny ? e + 128 : e;   // the implicit bit adds one to the field
+    uint32_t rl, rh;
+    asm("add.cc.u32 %0, %2, %3;\n addc.u32 %1, %4, %5;"
+        : "=r"(rl), "=r"(rh)
+        : "r"(ul), "r"(up), "r"(uh), "r"((uint32_t)(ef - 1) << 20));
+    if (huge) {
+        rh = 0x7ff00000u;
+        rl = 0;
+    }
+    double x = __hiloint2double((int)(rh | (sign & 0x80000000u)), (int)rl);
+    if (tiny) x = ef < 1 ? 0.0 : x * 0x1p-128;
+    return x;
+}
+
+// stages of register bits LO .. 3
+template <int LO> __device__ __forceinline__ void stages(W96* v) {
+#pragma unroll
+    for (int i = 3; i >= LO; --i) {
+#pragma unroll
+        for (int r = 0; r < 16; ++r)
+            if (!(r & (1 << i))) bfly96(v[r], v[r | (1 << i)]);
+    }
+}
+
+__device__ __forceinline__ int e_a(int t, int r) { return t + kNT * r; }
+__device__ __forceinline__ int e_c(int t, int r) { return 16 * t + r; }
+__device__ __forceinline__ int e_b(int t, int r) { return (t & 15) + 16 * r + 256 * (t >> 4); }
+
+template <int (*EL)(int, int)> __device__ __forceinline__ void put(uint32_t* p, const W96* v, int t) {
+#pragma unroll
+    for (int r = 0; r < 16; ++r) {
+        const int q = plane_pos(EL(t, r));
+        p[q] = v[r].a;
+        p[q + kPlane] = v[r].b;
+        p[q + 2 * kPlane] = v[r].c;
+    }
+}
+template <int (*EL)(int, int)> __device__ __forceinline__ void get(const uint32_t* p, W96* v, int t) {
+#pragma unroll
+    for (int r = 0; r < 16; ++r) {
+        const int q = plane_pos(EL(t, r));
+        v[r].a = p[q];
+        v[r].b = p[q + kPlane];
+        v[r].c = p[q + 2 * kPlane];
+    }
+}
+
+// One pass over 2^12-element tiles, B of the tile index's bits (the top ones)
+// transformed: B = 12 the low pass, B < 12 a high pass with 2^(12-B) columns.
+template <int B>
+__global__ void __launch_bounds__(kNT, 3) k2d_pass(DArgs a) {
+    constexpr int LC = kLT - B;          // column bits
+    constexpr int G = 42 - B;            // bits below the largest element's last place
+    extern __shared__ __align__(16) unsigned char smraw[];
+    uint32_t* plane = reinterpret_cast<uint32_t*>(smraw);
+    int* emax = reinterpret_cast<int*>(plane + 3 * kPlane);   // per column
+    const int t = threadIdx.x;
+    const long long tile = blockIdx.x;
+    const long long nlo = a.S >> LC;     // tiles side by side below the pass's digits
+    const long long base = B == kLT ? tile << kLT : ((tile % nlo) << LC) + (tile / nlo) * (a.S << B);
+    const double* src = a.in + blockIdx.y * a.ld_in + base;
+    double* dst = a.out + blockIdx.y * a.ld_out + base;
+    auto off = [&](int e) { return B == kLT ? (long long)e : (long long)(e & ((1 << LC) - 1)) + a.S * (long long)(e >> LC); };
+    double x[16];
+#pragma unroll
+    for (int r = 0; r < 16; ++r) x[r] = src[off(e_a(t, r))];
+    if constexpr (B <= 3) {
+        // a few stages, all in thread: FP64
+#pragma unroll
+        for (int i = 3; i >= 4 - B; --i)
+#pragma unroll
+            for (int r = 0; r < 16; ++r)
+                if (!(r & (1 << i))) {
+                    const double p = x[r], q = x[r | (1 << i)];
+                    x[r] = p + q;
+                    x[r | (1 << i)] = p - q;
+                }
+        const double sc = __hiloint2double((1023 + a.exp_shift) << 20, 0);
+#pragma unroll
+        for (int r = 0; r < 16; ++r) dst[off(e_a(t, r))] = a.exp_shift ? x[r] * sc : x[r];
+    } else {
+        int mx = 1;
+#pragma unroll
+        for (int r = 0; r < 16; ++r) mx = max(mx, exponent_of((uint32_t)__double2hiint(x[r])));
+        if (t < (1 << LC)) emax[t] = 1;
+        if (__syncthreads_or(mx == 0x7ff)) {
+            // an infinity or a NaN: FP64 stages through shared memory
+            double* y = reinterpret_cast<double*>(smraw);
+#pragma unroll
+            for (int r = 0; r < 16; ++r) y[e_a(t, r)] = x[r];
+            for (int i = kLT - 1; i >= LC; --i) {
+                __syncthreads();
+                for (int q = t; q < (1 << (kLT - 1)); q += kNT) {
+                    const int e0 = ((q >> i) << (i + 1)) | (q & ((1 << i) - 1)), e1 = e0 | (1 << i);
+                    const double p = y[e0], s = y[e1];
+                    y[e0] = p + s;
+                    y[e1] = p - s;
+                }
+            }
+            __syncthreads();
+            const double sc = __hiloint2double((1023 + a.exp_shift) << 20, 0);
+            for (int e = t; e < (1 << kLT); e += kNT) dst[off(e)] = y[e] * sc;
+            return;
+        }
+        if constexpr (LC == 0) {
+            mx = __reduce_max_sync(0xffffffffu, mx);
+            if ((t & 31) == 0) atomicMax(emax, mx);
+        } else {
+            atomicMax(emax + (t & ((1 << LC) - 1)), mx);   // LC <= 8: a thread's elements share a column
+        }
+        __syncthreads();
+        W96 v[16];
+        {
+            const int E = emax[t & ((1 << LC) - 1)];
+#pragma unroll
+            for (int r = 0; r < 16; ++r)
+                v[r] = to_fixed((uint32_t)__double2hiint(x[r]), (uint32_t)__double2loint(x[r]), E, G);
+        }
+        stages<0>(v);
+        if constexpr (B == 4) {
+            const int E = emax[t];
+#pragma unroll
+            for (int r = 0; r < 16; ++r) dst[off(e_a(t, r))] = from_fixed(v[r], E, G, a.exp_shift);
+        } else {
+            put<e_a>(plane, v, t);
+            __syncthreads();
+            if constexpr (B > 8) {
+                get<e_c>(plane, v, t);
+                stages<LC>(v);
+                put<e_c>(plane, v, t);
+                __syncthreads();
+            }
+            get<e_b>(plane, v, t);
+            stages<(LC > 4 ? LC - 4 : 0)>(v);
+#pragma unroll
+            for (int r = 0; r < 16; ++r) {
+                const int e = e_b(t, r);
+                dst[off(e)] = from_fixed(v[r], emax[e & ((1 << LC) - 1)], G, a.exp_shift);
+            }
+        }
+    }
+}
+
+template <int B> int launch_b(const DArgs& a, long long N, int nf, const char* fam, cudaStream_t st) {
+    auto k = k2d_pass<B>;
+    int rc = smem_limit_max(k);
+    if (rc) return rc;
+    const size_t smem = B <= 3 ? 0 : (size_t)3 * kPlane * 4 + ((size_t)4 << (kLT - B));
+    {
+        LaunchScope ls(fam, st);
+        k<<<dim3((unsigned)(N >> kLT), (unsigned)nf), kNT, smem, st>>>(a);
+    }
+    DWT_CK_LAUNCH("k2d_pass");
+    return DWT_OK;
+}
+
+int launch(int B, const DArgs& a, long long N, int nf, const char* fam, cudaStream_t st) {
+    switch (B) {
+        case 1: return launch_b<1>(a, N, nf, fam, st);
+        case 2: return launch_b<2>(a, N, nf, fam, st);
+        case 3: return launch_b<3>(a, N, nf, fam, st);
+        case 4: return launch_b<4>(a, N, nf, fam, st);
+        case 5: return launch_b<5>(a, N, nf, fam, st);
+        case 6: return launch_b<6>(a, N, nf, fam, st);
+        case 7: return launch_b<7>(a, N, nf, fam, st);
+        case 8: return launch_b<8>(a, N, nf, fam, st);
+        case 9: return launch_b<9>(a, N, nf, fam, st);
+        case 12: return launch_b<12>(a, N, nf, fam, st);
+        default: set_error("FP64 pass digits"); return DWT_EUNSUPPORTED;
+    }
+}
+
+const long long kL2GroupD = 48ll << 20;   // bytes of functions kept in L2 between the passes
+
+}  // namespace
+
+bool p2d_ok(int m) { return m >= kLT; }
+
+// dwt_forward / dwt_inverse for p = 2, FP64, m >= 12: the 12 low digits, then
+// the others in passes of at most 9 (rows of 64 bytes at least), as even as
+// possible.
+int p2d_transform(dwt_plan_s* Pl, const double* in, double* out, int batch, long long ld_in, long long ld_out,
+                  int sgn, cudaStream_t st) {
+    const int m = Pl->m, high = m - kLT, nh = (high + 8) / 9;
+    const long long N = Pl->N;
+    const int G = (int)std::min(65535ll, std::max(1ll, kL2GroupD / (N * 8)));
+    for (int f0 = 0; f0 < batch; f0 += G) {
+        const int nf = std::min(G, batch - f0);
+        DArgs a{in + (long long)f0 * ld_in, out + (long long)f0 * ld_out, ld_in, ld_out, 1, 0};
+        if (nh == 0 && sgn < 0) a.exp_shift = -m;
+        int rc = launch(kLT, a, N, nf, "pass_lo", st);
+        if (rc) return rc;
+        int d = kLT;
+        for (int k = 0; k < nh; ++k) {
+            const int b = high / nh + (k < high % nh ? 1 : 0);
+            DArgs h{out + (long long)f0 * ld_out, out + (long long)f0 * ld_out, ld_out, ld_out, 1ll << d, 0};
+            if (k == nh - 1 && sgn < 0) h.exp_shift = -m;
+            if ((rc = launch(b, h, N, nf, k == nh - 1 ? "pass_hi" : "pass_mid", st))) return rc;
+            d += b;
+        }
+    }
+    return DWT_OK;
+}
+
+}  // namespace dwt

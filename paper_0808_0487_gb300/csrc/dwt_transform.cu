@@ -27,6 +27,9 @@ int p2_transform(dwt_plan_s* Pl, const void* in, void* out, int batch, long long
 int p2_interpolate(dwt_plan_s* Pl, const float* f, float* c, float* coef, int batch, long long ld, const float* W,
                    bool tc, double** part_out, long long* ntile_out, cudaStream_t st);
 
+bool p2d_ok(int m);
+int p2d_transform(dwt_plan_s* Pl, const double* in, double* out, int batch, long long ld_in, long long ld_out,
+                  int sgn, cudaStream_t st);
 bool p2_small_ok(int m);
 int p2_small_interpolate(dwt_plan_s* Pl, const float* f, float* c, float* coef, int batch, long long ld,
                          bool weighted, double thr, const EffOut& o, cudaStream_t st);
@@ -837,6 +840,11 @@ int run_transform_grouped(const std::vector<GroupJob>& jobs, dwt_dtype in_t, dwt
             }
             continue;
         }
+        if (p == 2 && in_t == DWT_F64 && p2d_ok(j.plan->m)) {
+            const int rc = p2d_transform(j.plan, (const double*)j.in, (double*)j.out, j.batch, j.ld_in, j.ld_out, sgn, st);
+            if (rc) return rc;
+            continue;
+        }
         generic.push_back(j);
     }
     for (int L = 12; L <= 14; ++L)
@@ -866,6 +874,8 @@ int run_transform(dwt_plan_s* Pl, const void* in, void* out, int batch, long lon
     if (Pl->p == 2 && (in_t == DWT_F32 || in_t == DWT_I32) && p2_fast_ok(Pl->m) && aligned16(in, ld_in, 4) &&
         aligned16(out, ld_out, 4))
         return p2_transform(Pl, in, out, batch, ld_in, ld_out, in_t, sgn, st);
+    if (Pl->p == 2 && in_t == DWT_F64 && p2d_ok(Pl->m))
+        return p2d_transform(Pl, (const double*)in, (double*)out, batch, ld_in, ld_out, sgn, st);
     switch (Pl->p) {
         case 2: return transform_p<2>(Pl, in, out, batch, ld_in, ld_out, in_t, out_t, sgn, st);
         case 3: return transform_p<3>(Pl, in, out, batch, ld_in, ld_out, in_t, out_t, sgn, st);
