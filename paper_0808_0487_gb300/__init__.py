@@ -12,6 +12,8 @@ There is no fallback: if the library is missing, every call raises.
 """
 import ctypes
 import os
+import struct
+import sys
 
 import numpy as np
 
@@ -146,6 +148,11 @@ def _ptr(x):
 
 def _stream(s):
     if s is None:
+        # torch's current stream of its current device; once torch has initialised CUDA
+        # the raw handle costs a tenth of the Stream object that current_stream() makes
+        torch = sys.modules.get("torch")
+        if torch is not None and torch.cuda.is_initialized():
+            return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
         try:
             import torch
             if torch.cuda.is_available():
@@ -291,22 +298,21 @@ class _Job(ctypes.Structure):
     _fields_ = [("plan", _VP), ("in_", _VP), ("out", _VP), ("batch", _I), ("ld_in", _LL), ("ld_out", _LL)]
 
 
+_JOB = struct.Struct("@PPPi4xqq")   # the layout of _Job
+
+
 def _jobs(jobs):
-    arr = (_Job * len(jobs))()
-    for i, (plan, inp, out, batch, ld_in, ld_out) in enumerate(jobs):
-        arr[i] = _Job(plan.handle, _ptr(inp), _ptr(out), batch, ld_in, ld_out)
-    return arr
+    return b"".join([_JOB.pack(plan.handle or 0, _ptr(inp) or 0, _ptr(out) or 0, batch, ld_in, ld_out)
+                     for plan, inp, out, batch, ld_in, ld_out in jobs])
 
 
 def dwt_forward_grouped(jobs, in_t, out_t, stream=None):
     """jobs: list of (plan, in, out, batch, ld_in, ld_out); see dwt_forward_grouped in include/dwt.h."""
-    arr = _jobs(jobs)
-    return _check(lib().dwt_forward_grouped(ctypes.cast(arr, _VP), len(jobs), in_t, out_t, _stream(stream)))
+    return _check(lib().dwt_forward_grouped(_jobs(jobs), len(jobs), in_t, out_t, _stream(stream)))
 
 
 def dwt_inverse_grouped(jobs, in_t, out_t, stream=None):
-    arr = _jobs(jobs)
-    return _check(lib().dwt_inverse_grouped(ctypes.cast(arr, _VP), len(jobs), in_t, out_t, _stream(stream)))
+    return _check(lib().dwt_inverse_grouped(_jobs(jobs), len(jobs), in_t, out_t, _stream(stream)))
 
 
 def dwt_forward_digits(plan, inp, out, batch, ld_in, ld_out, in_t, out_t, d0, nd, stream=None):

@@ -84,17 +84,27 @@ template <typename T> struct LoGroup {
     long long first;
 };
 
+// Lists of up to kLoInline jobs travel in the launch's parameters (no
+// allocation, no copy), longer ones lie in device memory.
+constexpr int kLoInline = 32;
+template <typename T> struct LoList {
+    int n;
+    const LoGroup<T>* far;   // n > kLoInline
+    LoGroup<T> near[kLoInline];
+};
+
 template <typename T, int L>
 __global__ void __launch_bounds__(1 << (L - 6), (L == 14 ? 3 : 4))
-    k2_lo_grouped(const LoGroup<T>* __restrict__ jobs, int njobs) {
+    k2_lo_grouped(const __grid_constant__ LoList<T> list) {
+    const LoGroup<T>* jobs = list.n > kLoInline ? list.far : list.near;
     const long long b = blockIdx.x;
-    int lo = 0, hi = njobs - 1;   // the last job starting at or before b
+    int lo = 0, hi = list.n - 1;   // the last job starting at or before b
     while (lo < hi) {
         const int mid = (lo + hi + 1) >> 1;
         if (jobs[mid].first <= b) lo = mid;
         else hi = mid - 1;
     }
-    const LoJob<T>& j = jobs[lo].j;
+    const LoJob<T> j = jobs[lo].j;
     const long long fn = b - jobs[lo].first;
     lo_body<T, L>(j.in + fn * j.ld_in, j.out + fn * j.ld_out, j.scale, j.do_scale, j.stream_out != 0);
 }
@@ -363,9 +373,16 @@ static int lo_grouped_t(int L, const std::vector<GroupJob>& jobs, int sgn, cudaS
         set_error("grouped low pass: %lld blocks exceed one launch", blocks);
         return DWT_EINVAL;
     }
+    LoList<T> list;
+    list.n = (int)h.size();
     LoGroup<T>* d = nullptr;
-    if (dmalloc((void**)&d, sizeof(LoGroup<T>) * h.size(), st)) return DWT_ENOMEM;
-    DWT_CK(cudaMemcpyAsync(d, h.data(), sizeof(LoGroup<T>) * h.size(), cudaMemcpyHostToDevice, st));
+    if (list.n > kLoInline) {
+        if (dmalloc((void**)&d, sizeof(LoGroup<T>) * h.size(), st)) return DWT_ENOMEM;
+        DWT_CK(cudaMemcpyAsync(d, h.data(), sizeof(LoGroup<T>) * h.size(), cudaMemcpyHostToDevice, st));
+    } else {
+        std::copy(h.begin(), h.end(), list.near);
+    }
+    list.far = d;
     const size_t smem = (((size_t)1 << L) + ((size_t)1 << (L - 4))) * sizeof(T);
     int rc = DWT_OK;
 #define DWT_LOG(LL)                                                                       \
@@ -373,7 +390,7 @@ static int lo_grouped_t(int L, const std::vector<GroupJob>& jobs, int sgn, cudaS
         auto k = k2_lo_grouped<T, LL>;                                                    \
         if ((rc = attr_smem(k, smem))) break;                                             \
         LaunchScope ls("grouped_lo", st);                                                 \
-        k<<<(unsigned)blocks, 1 << (LL - 6), smem, st>>>(d, (int)h.size());               \
+        k<<<(unsigned)blocks, 1 << (LL - 6), smem, st>>>(list);                           \
         break;                                                                            \
     }
     switch (L) {
