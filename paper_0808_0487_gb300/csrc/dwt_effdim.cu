@@ -19,6 +19,7 @@ template <int CL>
 __global__ void __launch_bounds__(kRedThreads) k_effdim_reduce(const double* __restrict__ part, long long nchunk,
                                                                int nb, int lg, double thr, EffOut o, long long f0) {
     namespace cg = cooperative_groups;
+    chain_begin();
     __shared__ double c[2 * 256];
     __shared__ int first[2];
     const int nb2 = 2 * nb;
@@ -48,11 +49,13 @@ static int launch_reduce(const double* part, long long nchunk, int nb, int batch
         cfg.gridDim = dim3(CL, (unsigned)std::min(65535, batch - f0));
         cfg.blockDim = dim3(kRedThreads);
         cfg.stream = st;
-        cudaLaunchAttribute at[1];
-        at[0].id = cudaLaunchAttributeClusterDimension;
-        at[0].val.clusterDim = {CL, 1, 1};
+        cudaLaunchAttribute at[2];   // as launch_chain, in clusters
+        at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at[0].val.programmaticStreamSerializationAllowed = 1;
+        at[1].id = cudaLaunchAttributeClusterDimension;
+        at[1].val.clusterDim = {CL, 1, 1};
         cfg.attrs = at;
-        cfg.numAttrs = CL > 1 ? 1 : 0;
+        cfg.numAttrs = CL > 1 ? 2 : 1;
         DWT_CK(cudaLaunchKernelEx(&cfg, k_effdim_reduce<CL>, part, nchunk, nb, lg, thr, o, (long long)f0));
     }
     DWT_CK_LAUNCH("k_effdim_reduce");

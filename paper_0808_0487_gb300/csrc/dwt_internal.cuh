@@ -40,6 +40,33 @@ struct LaunchScope {
     ~LaunchScope() { launch_end(fam, st); }
 };
 
+// A kernel of a chain on one stream: it may be launched as the previous
+// kernel's blocks end (programmatic stream serialisation) and starts with
+// chain_begin(), which waits until that kernel has completed and its writes are
+// visible; everything after it is ordered as between ordinary launches.  The
+// launch latency overlaps the previous kernel's last blocks: p = 2, m = 24, 32
+// functions, 65 kernels: 3.06 -> 2.87 ms per call; m = 20, 32 functions, 6
+// kernels: 118 -> 104 us.  (Letting the next kernel start when this one's last
+// blocks have started is slower: its waiting blocks take their slots.)
+template <typename... KA, typename... A>
+static inline void launch_chain(void (*kern)(KA...), dim3 grid, unsigned threads, size_t smem, cudaStream_t st,
+                                const A&... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, kern, KA(args)...);   // a failure is read by DWT_CK_LAUNCH
+}
+__device__ __forceinline__ void chain_begin() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 // ---------------------------------------------------------------------------
 // the plan
 struct PassGeom {

@@ -67,6 +67,7 @@ template <typename T, int L>
 __global__ void __launch_bounds__(1 << (L - 6), (L == 14 ? 3 : 4))
     k2_lo(LoJob<T> j0, LoJob<T> j1, unsigned tiles0) {
     static_assert(L >= 12 && L <= 14, "low-pass tile 2^12 .. 2^14");
+    chain_begin();
     const bool second = blockIdx.x >= tiles0;
     if ((int)blockIdx.y >= (second ? j1.nf : j0.nf)) return;
     const long long tile = second ? blockIdx.x - tiles0 : blockIdx.x;
@@ -96,6 +97,7 @@ template <typename T> struct LoList {
 template <typename T, int L>
 __global__ void __launch_bounds__(1 << (L - 6), (L == 14 ? 3 : 4))
     k2_lo_grouped(const __grid_constant__ LoList<T> list) {
+    chain_begin();
     const LoGroup<T>* jobs = list.n > kLoInline ? list.far : list.near;
     const long long b = blockIdx.x;
     int lo = 0, hi = list.n - 1;   // the last job starting at or before b
@@ -134,6 +136,7 @@ __global__ void __launch_bounds__(1 << (LT - 6), FUSED ? 4 : 1) k2_hi(HiArgs a) 
     using G = HiGeom<LT, B>;
     using V = typename P2<T>::t;
     constexpr int NT = G::NT, P1 = G::P1;
+    chain_begin();
     extern __shared__ __align__(16) unsigned char smraw[];
     T* sm = reinterpret_cast<T*>(smraw);
     const int t = threadIdx.x;
@@ -342,7 +345,7 @@ static int launch_lo2(int L, const LoJob<T>& a, const LoJob<T>* b, long long N, 
         auto k = k2_lo<T, LL>;                                                             \
         if ((rc = attr_smem(k, smem))) return rc;                                          \
         LaunchScope ls(fam, st);                                                           \
-        k<<<grid, 1 << (LL - 6), smem, st>>>(a, jb, tiles);                                \
+        launch_chain(k, grid, 1u << (LL - 6), smem, st, a, jb, tiles);                     \
         break;                                                                             \
     }
     switch (L) {
@@ -390,7 +393,7 @@ static int lo_grouped_t(int L, const std::vector<GroupJob>& jobs, int sgn, cudaS
         auto k = k2_lo_grouped<T, LL>;                                                    \
         if ((rc = attr_smem(k, smem))) break;                                             \
         LaunchScope ls("grouped_lo", st);                                                 \
-        k<<<(unsigned)blocks, 1 << (LL - 6), smem, st>>>(list);                           \
+        launch_chain(k, dim3((unsigned)blocks), 1u << (LL - 6), smem, st, list);           \
         break;                                                                            \
     }
     switch (L) {
@@ -432,7 +435,7 @@ static int launch_hi_one(HiArgs a, int nf, size_t bins_bytes, const char* fam, c
     dim3 grid((unsigned)a.ntile, (unsigned)nf);
     {
         LaunchScope ls(fam, st);
-        k<<<grid, G::NT, smem, st>>>(a);
+        launch_chain(k, grid, G::NT, smem, st, a);
     }
     DWT_CK_LAUNCH("k2_hi");
     return DWT_OK;

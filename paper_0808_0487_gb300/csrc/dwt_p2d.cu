@@ -189,6 +189,7 @@ __global__ void __launch_bounds__(kNT, 3) k2d_pass(DArgs a) {
     uint32_t* plane = reinterpret_cast<uint32_t*>(smraw);
     int* emax = reinterpret_cast<int*>(plane + 3 * kPlane);   // per column
     const int t = threadIdx.x;
+    chain_begin();
     const long long tile = blockIdx.x;
     const long long nlo = a.S >> LC;     // tiles side by side below the pass's digits
     const long long base = B == kLT ? tile << kLT : ((tile % nlo) << LC) + (tile / nlo) * (a.S << B);
@@ -282,7 +283,7 @@ template <int B> int launch_b(const DArgs& a, long long N, int nf, const char* f
     const size_t smem = B <= 3 ? 0 : (size_t)3 * kPlane * 4 + ((size_t)4 << (kLT - B));
     {
         LaunchScope ls(fam, st);
-        k<<<dim3((unsigned)(N >> kLT), (unsigned)nf), kNT, smem, st>>>(a);
+        launch_chain(k, dim3((unsigned)(N >> kLT), (unsigned)nf), kNT, smem, st, a);
     }
     DWT_CK_LAUNCH("k2d_pass");
     return DWT_OK;

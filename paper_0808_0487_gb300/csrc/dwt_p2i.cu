@@ -203,6 +203,7 @@ __global__ void __launch_bounds__(kTopNT, kTopMinBlocks) k2i_top(const __grid_co
     const int x0 = (int)(tile * WC);
     const uint64_t keep = policy_evict_last();
     const long long to = tile << kTopLT;
+    chain_begin();
     // compact tables: the tile's 16-bit codes (32 KB, contiguous) come into
     // shared memory with the data tile; full tables are read into registers
     const uint4* qsm = COMPACT ? reinterpret_cast<const uint4*>(reinterpret_cast<const unsigned char*>(sm) + a.codes_off)
@@ -407,6 +408,7 @@ __global__ void __launch_bounds__(kHiNT, 3) k2i_hi(const __grid_constant__ CUten
     const int fn = blockIdx.y;
     const int x0 = (int)((long long)blockIdx.x * WC);
     const uint64_t first = policy_evict_first();
+    chain_begin();
     if (t == 0) {
         mbar_init1(smem_u32(&bar));
         mbar_expect_tx(smem_u32(&bar), TG::TILE_BYTES);
@@ -514,6 +516,7 @@ __global__ void __launch_bounds__(1 << (L - 6), 3) k2i_lo(LoJobI j0, LoJobI j1, 
     extern __shared__ __align__(16) unsigned char smraw[];
     float* sm = reinterpret_cast<float*>(smraw);
     const int t = threadIdx.x;
+    chain_begin();
     const bool second = njobs == 2 && (blockIdx.x & 1);
     const long long tile = njobs == 2 ? (blockIdx.x >> 1) : blockIdx.x;
     const LoJobI& J = second ? j1 : j0;
@@ -609,7 +612,7 @@ static int launch_top_one(const CUtensorMap& tm, const TopArgs& a, int nf, int s
         LaunchScope ls("interp_top", st);
         TopArgs a2 = a;
         a2.codes_off = (int)top_region(s, (size_t)HiGeom<kTopLT, B>::SMEM_ELEMS * 4);
-        k<<<grid, kTopNT, top_smem<B>(s, COMPACT), st>>>(tm, a2);
+        launch_chain(k, grid, kTopNT, top_smem<B>(s, COMPACT), st, tm, a2);
     }
     DWT_CK_LAUNCH("k2i_top");
     return DWT_OK;
@@ -648,7 +651,7 @@ static int launch_lo_i(const LoJobI& a, const LoJobI* b, long long N, const char
     if (rc) return rc;
     {
         LaunchScope ls(fam, st);
-        k<<<grid, 1 << (L - 6), smem, st>>>(a, b ? *b : a, b ? 2 : 1);
+        launch_chain(k, grid, 1u << (L - 6), smem, st, a, b ? *b : a, b ? 2 : 1);
     }
     DWT_CK_LAUNCH("k2i_lo");
     return DWT_OK;
@@ -668,7 +671,7 @@ static int launch_hi_b(float* base, long long ld, int nf, float scale, int do_sc
     dim3 grid((unsigned)((1u << kRowLog) / TopGeom<B, kHiLT>::WC), (unsigned)nf);
     {
         LaunchScope ls(do_scale ? "p2_hi_fwd" : "p2_hi_inv", st);
-        k<<<grid, kHiNT, smem, st>>>(tm, scale, do_scale, err);
+        launch_chain(k, grid, kHiNT, smem, st, tm, scale, do_scale, err);
     }
     DWT_CK_LAUNCH("k2i_hi");
     return DWT_OK;

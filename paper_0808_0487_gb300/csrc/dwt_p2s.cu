@@ -149,6 +149,7 @@ __global__ void __launch_bounds__(Small<M>::NT) k2_small(SmallArgs a) {
     int* first = reinterpret_cast<int*>(tot + 2 * a.nb);
     float* bins = reinterpret_cast<float*>(first + 4);
     const int t = threadIdx.x, nb2 = 2 * a.nb;
+    chain_begin();
     const long long fn = blockIdx.x;
     const float* src = a.f + fn * a.ld;
     float* dst = a.c + fn * a.ld;
@@ -242,7 +243,7 @@ template <int M> int launch_small(const SmallArgs& a, int batch, cudaStream_t st
                         (size_t)a.nwb * 2 * a.nb * 128;
     {
         LaunchScope ls("interp_small", st);
-        k<<<(unsigned)batch, G::NT, smem, st>>>(a);
+        launch_chain(k, dim3((unsigned)batch), G::NT, smem, st, a);
     }
     DWT_CK_LAUNCH("k2_small");
     return DWT_OK;

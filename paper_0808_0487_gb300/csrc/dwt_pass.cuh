@@ -330,6 +330,7 @@ __device__ __forceinline__ void pass_body(const PassArgs& a, const Tw& tw, long 
 
 template <int P, typename T, typename TI, int SGN, int KM>
 __global__ void __maxnreg__(pass_maxnreg<P>()) k_pass(PassArgs a, const __grid_constant__ Tw tw) {
+    chain_begin();
     pass_body<P, T, TI, SGN, KM>(a, tw, blockIdx.x, blockIdx.y);
 }
 
@@ -354,6 +355,7 @@ struct GroupList {
 
 template <int P, typename T, typename TI, int SGN, int KM>
 __global__ void __maxnreg__(pass_maxnreg<P>()) k_pass_grouped(const __grid_constant__ GroupList list) {
+    chain_begin();
     const GroupPass* jobs = list.n > kGroupInline ? list.far : list.near;
     const long long b = blockIdx.x;
     int lo = 0, hi = list.n - 1;   // the last job starting at or before b
@@ -408,6 +410,7 @@ __device__ __forceinline__ void reduce_bins(const float* bins, int nb2, int nwb,
 // inverse groups, the last one writing global memory as in k_pass.
 template <int P, typename T, typename TI, int KM>
 __global__ void __maxnreg__(96) k_mid(MidArgs m, int nwb, const __grid_constant__ Tw tw) {
+    chain_begin();
     const PassArgs& a = m.pa;
     extern __shared__ __align__(16) unsigned char smraw[];
     T* sm = reinterpret_cast<T*>(smraw);
@@ -563,7 +566,7 @@ static int launch_pass_k(const PassGeom& g, const PassArgs& a, const Tw& tw, int
     dim3 grid((unsigned)g.ntile, (unsigned)nf);
     {
         LaunchScope ls(fam, st);
-        kern<<<grid, pass_threads<P, KM>(g), smem, st>>>(a, tw);
+        launch_chain(kern, grid, pass_threads<P, KM>(g), smem, st, a, tw);
     }
     DWT_CK_LAUNCH("k_pass");
     return DWT_OK;
@@ -703,7 +706,7 @@ static int launch_grouped(const std::vector<GroupPass>& h, const Tw& tw, long lo
     list.far = d;
     {
         LaunchScope ls(fam, st);
-        kern<<<(unsigned)blocks, threads, smem, st>>>(list);
+        launch_chain(kern, dim3((unsigned)blocks), threads, smem, st, list);
     }
     dfree(d, st);
     DWT_CK_LAUNCH("k_pass_grouped");
@@ -853,8 +856,8 @@ static int interpolate_t(dwt_plan_s* Pl, const void* f, void* c, void* coef, int
         {
             LaunchScope ls("interp_top", st);
             dim3 grid((unsigned)ntile, (unsigned)nf);
-            if (pp.q == 1) kmid_first<<<grid, nt, smem, st>>>(m, nw, tw);
-            else kmid_next<<<grid, nt, smem, st>>>(m, nw, tw);
+            if (pp.q == 1) launch_chain(kmid_first, grid, nt, smem, st, m, nw, tw);
+            else launch_chain(kmid_next, grid, nt, smem, st, m, nw, tw);
         }
         DWT_CK_LAUNCH("k_mid");
         // inverse passes below the top one, in place on c

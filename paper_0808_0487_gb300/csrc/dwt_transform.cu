@@ -42,6 +42,7 @@ __global__ void __launch_bounds__(256) k_effdim_bins(const T* coef, long long ld
     extern __shared__ __align__(16) unsigned char smraw[];
     float* bins = reinterpret_cast<float*>(smraw);
     const int nb2 = 2 * nb, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    chain_begin();
     for (int i = threadIdx.x; i < (int)(blockDim.x >> 5) * nb2 * 32; i += blockDim.x) bins[i] = 0.f;
     __syncthreads();
     const long long fn = blockIdx.y, chunk = blockIdx.x;
@@ -179,7 +180,7 @@ static int effdim_t(dwt_plan_s* Pl, const void* coef, int batch, long long ld, c
     for (int f0 = 0; f0 < batch; f0 += 65535) {
         const int nf = std::min(65535, batch - f0);
         LaunchScope ls("effdim_bins", st);
-        kern<<<dim3((unsigned)nchunk, (unsigned)nf), nw * 32, smem, st>>>(
+        launch_chain(kern, dim3((unsigned)nchunk, (unsigned)nf), nw * 32, smem, st,
             (const T*)coef + (long long)f0 * ld, ld, Pl->N, Pl->d_cls, nb, nchunk, part + (long long)f0 * nchunk * nb2);
     }
     DWT_CK_LAUNCH("k_effdim_bins");
@@ -210,8 +211,8 @@ static int effdim_scratch_t(dwt_plan_s* Pl, const void* coef, int batch, long lo
         const int nf = std::min(G, batch - f0);
         {
             LaunchScope ls("effdim_bins", st);
-            kern<<<dim3((unsigned)nchunk, (unsigned)nf), nw * 32, smem, st>>>(
-                (const T*)coef + (long long)f0 * ld, ld, Pl->N, Pl->d_cls, nb, nchunk, scratch);
+            launch_chain(kern, dim3((unsigned)nchunk, (unsigned)nf), nw * 32, smem, st,
+            (const T*)coef + (long long)f0 * ld, ld, Pl->N, Pl->d_cls, nb, nchunk, scratch);
         }
         DWT_CK_LAUNCH("k_effdim_bins");
         rc = effdim_reduce(scratch, nchunk, nb, nf, thr, eff_packed(var ? var + (long long)f0 * 2 * nb : nullptr,
