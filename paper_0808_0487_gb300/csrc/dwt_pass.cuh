@@ -180,14 +180,27 @@ template <int P, typename T> struct KMax {
 };
 
 // ---------------------------------------------------------------------------
+// one register group of a pass: k digits from row digit g0 on, in the order
+// they run; the divisions of the task numbering as multiplications
+struct PassGroup {
+    unsigned pg0, nrh;       // p^g0, R / p^(g0+k)
+    unsigned mg_lo, mg_hi;   // floor(2^32 / d) + 1 for d = pg0 and nrh, 0 for d = 1
+    int k, last;
+};
+constexpr int kMaxGroups = 8;   // 64 KB tiles: at most five (p = 5, complex FP64)
+
 struct PassArgs {
     const void* in;
     void* out;
     long long ld_in, ld_out;
-    long long S, SR, nlo;
-    int R, b, Wc, wlog;
+    long long S, SR;
+    unsigned nlo;
+    int R, Wc, wlog;
     double scale;
+    float scalef;
     int do_scale;
+    int direct_out;          // the last group writes global memory
+    PassGroup g[kMaxGroups];
 };
 
 // Register groups of a pass.  A tile has R = p^b rows (row digits 0 .. b-1) of
@@ -204,67 +217,93 @@ struct PassArgs {
 // shared memory and writes to global memory (DST_G) or shared memory.
 template <int P, typename T> __device__ __forceinline__ int sx(int e) { return (P & 1) ? e : spad<T>(e); }
 
+template <typename T> __device__ __forceinline__ T scale_of(const PassArgs& a, T v) {
+    if constexpr (sizeof(T) == sizeof(float) || std::is_same<T, float2>::value) return scale_by<T>(v, a.scalef);
+    else return scale_by<T>(v, a.scale);
+}
+
+// Everything that does not depend on the element is worked out on the host
+// (PassGroup) or once per task, and an element's address is the previous one's
+// plus a stride: with the divisions, products and 64-bit offsets per thread and
+// element that this replaces, p = 3 spent 79 instructions per point on eight
+// digits, of which the sums need 24.
 template <int P, int K, int SGN, typename T, typename TI, bool SRC_G, bool DST_G, bool RHF>
-__device__ __forceinline__ void rgroup(T* sm, const TI* gin, T* gout, int g0, const PassArgs& a, const Tw& tw,
-                                       int ncols) {
+__device__ __forceinline__ void rgroup(T* sm, const TI* gin, T* gout, const PassGroup& g, const PassArgs& a,
+                                       const Tw& tw, int ncols) {
     constexpr int NK = cpow(P, K);
-    unsigned pg0 = 1;
-    for (int i = 0; i < g0; ++i) pg0 *= P;
-    const unsigned pgk = pg0 * NK;
-    const unsigned nrh = (unsigned)a.R / pgk;
+    const unsigned pg0 = g.pg0, pgk = pg0 * NK;
     const unsigned ntask = ((unsigned)a.R / NK) << a.wlog;
-    // q / dv = (q mg) >> 42, exact while q dv < 2^42 (q, dv <= R <= 2^16 here)
-    const unsigned dv = RHF ? nrh : pg0;
-    const unsigned long long mg = (1ull << 42) / dv + 1;
+    // q / dv by a multiplication, exact while q dv < 2^32 (q, dv <= R <= 2^16 here)
+    const unsigned dv = RHF ? g.nrh : pg0, mg = RHF ? g.mg_hi : g.mg_lo;
     const unsigned cmask = (unsigned)a.Wc - 1;
-    const long long step = a.S * (long long)pg0;
+    const int sstep = (int)(pg0 << a.wlog);
+    const long long gstep = a.S * (long long)pg0;
     for (unsigned t = threadIdx.x; t < ntask; t += blockDim.x) {
         const unsigned c = t & cmask, q = t >> a.wlog;
-        const unsigned qd = (unsigned)(((unsigned long long)q * mg) >> 42), qm = q - qd * dv;
+        const unsigned qd = mg ? __umulhi(q, mg) : q, qm = q - qd * dv;
         const unsigned rl = RHF ? qd : qm, rh = RHF ? qm : qd;
         const unsigned r0 = rl + rh * pgk;
         const bool live = (int)c < ncols;
+        const int e0 = (int)((r0 << a.wlog) + c);
         T v[NK];
         if constexpr (SRC_G) {
-            const TI* src = gin + c + a.S * (long long)r0;
+            const TI* src = gin + (c + a.S * (long long)r0);
 #pragma unroll
-            for (int i = 0; i < NK; ++i) v[i] = live ? promote<T, TI>(src[i * step]) : zero_of<T>();
+            for (int i = 0; i < NK; ++i) {
+                v[i] = live ? promote<T, TI>(*src) : zero_of<T>();
+                src += gstep;
+            }
         } else {
+            int e = e0;
 #pragma unroll
-            for (int i = 0; i < NK; ++i) v[i] = sm[sx<P, T>((int)(((r0 + i * pg0) << a.wlog) + c))];
+            for (int i = 0; i < NK; ++i) {
+                v[i] = sm[sx<P, T>(e)];
+                e += sstep;
+            }
         }
         RegStages<P, NK, 1, SGN, T>::run(v, tw);
         if constexpr (DST_G) {
-            if (live) {
-                T* dst = gout + c + a.S * (long long)r0;
+            if (a.do_scale) {
 #pragma unroll
-                for (int i = 0; i < NK; ++i) dst[i * step] = a.do_scale ? scale_by<T>(v[i], a.scale) : v[i];
+                for (int i = 0; i < NK; ++i) v[i] = scale_of<T>(a, v[i]);
+            }
+            if (live) {
+                T* dst = gout + (c + a.S * (long long)r0);
+#pragma unroll
+                for (int i = 0; i < NK; ++i) {
+                    *dst = v[i];
+                    dst += gstep;
+                }
             }
         } else {
+            int e = e0;
 #pragma unroll
-            for (int i = 0; i < NK; ++i) sm[sx<P, T>((int)(((r0 + i * pg0) << a.wlog) + c))] = v[i];
+            for (int i = 0; i < NK; ++i) {
+                sm[sx<P, T>(e)] = v[i];
+                e += sstep;
+            }
         }
     }
 }
 
 // mode bits: 1 read global, 2 write global, 4 rh-first numbering
 template <int P, int SGN, typename T, typename TI, int K>
-__device__ __forceinline__ void rgroup_k(int k, int mode, T* sm, const TI* gin, T* gout, int g0, const PassArgs& a,
-                                         const Tw& tw, int ncols) {
+__device__ __forceinline__ void rgroup_k(int mode, T* sm, const TI* gin, T* gout, const PassGroup& g,
+                                         const PassArgs& a, const Tw& tw, int ncols) {
     if constexpr (K >= 1) {
-        if (k == K) {
+        if (g.k == K) {
             switch (mode) {
-                case 1: rgroup<P, K, SGN, T, TI, true, false, false>(sm, gin, gout, g0, a, tw, ncols); break;
-                case 2: rgroup<P, K, SGN, T, TI, false, true, false>(sm, gin, gout, g0, a, tw, ncols); break;
-                case 3: rgroup<P, K, SGN, T, TI, true, true, false>(sm, gin, gout, g0, a, tw, ncols); break;
+                case 1: rgroup<P, K, SGN, T, TI, true, false, false>(sm, gin, gout, g, a, tw, ncols); break;
+                case 2: rgroup<P, K, SGN, T, TI, false, true, false>(sm, gin, gout, g, a, tw, ncols); break;
+                case 3: rgroup<P, K, SGN, T, TI, true, true, false>(sm, gin, gout, g, a, tw, ncols); break;
                 default:
-                    if constexpr (P & 1) rgroup<P, K, SGN, T, TI, false, false, true>(sm, gin, gout, g0, a, tw, ncols);
-                    else rgroup<P, K, SGN, T, TI, false, false, false>(sm, gin, gout, g0, a, tw, ncols);
+                    if constexpr (P & 1) rgroup<P, K, SGN, T, TI, false, false, true>(sm, gin, gout, g, a, tw, ncols);
+                    else rgroup<P, K, SGN, T, TI, false, false, false>(sm, gin, gout, g, a, tw, ncols);
                     break;
             }
             return;
         }
-        rgroup_k<P, SGN, T, TI, K - 1>(k, mode, sm, gin, gout, g0, a, tw, ncols);
+        rgroup_k<P, SGN, T, TI, K - 1>(mode, sm, gin, gout, g, a, tw, ncols);
     }
 }
 
@@ -285,34 +324,23 @@ template <int P> constexpr int pass_maxnreg() { return P > 13 ? 160 : 96; }
 template <int P> constexpr long long pass_max_threads() { return P > 13 ? 384 : 512; }
 
 template <int P, typename T, typename TI, int SGN, int KM>
-__device__ __forceinline__ void pass_body(const PassArgs& a, const Tw& tw, long long tile, long long fn) {
+__device__ __forceinline__ void pass_body(const PassArgs& a, const Tw& tw, unsigned tile, long long fn) {
     extern __shared__ __align__(16) unsigned char smraw[];
     T* sm = reinterpret_cast<T*>(smraw);
-    const long long lo0 = (tile % a.nlo) << a.wlog;
-    const long long base = lo0 + (tile / a.nlo) * a.SR;
+    const unsigned th = tile / a.nlo;
+    const long long lo0 = (long long)(tile - th * a.nlo) << a.wlog;
+    const long long base = lo0 + th * a.SR;
     const int ncols = (int)min((long long)a.Wc, a.S - lo0);
     const TI* in = reinterpret_cast<const TI*>(a.in) + fn * a.ld_in + base;
     T* out = reinterpret_cast<T*>(a.out) + fn * a.ld_out + base;
-    const int b = a.b;
-    const int k0 = min(KM, b);
-    // the last group: the top of the digits below the first group
-    const int g_last = b == k0 ? 0 : ((b - k0 - 1) / KM) * KM;
-    long long run = 1;
-    if (a.S == 1) {
-        for (int i = 0; i < g_last; ++i) run *= P;
-    } else {
-        run = a.Wc;
-    }
-    const bool direct_out = run * (long long)sizeof(T) >= 64;
-    int g0 = b - k0, k = k0;
-    for (;;) {
-        const bool last = g0 == g_last;
-        const int mode = (g0 + k == b ? 1 : 0) | (last && direct_out ? 2 : 0) | (g0 + k != b && !(last && direct_out) ? 4 : 0);
-        rgroup_k<P, SGN, T, TI, KM>(k, mode, sm, in, out, g0, a, tw, ncols);
-        if (!(last && direct_out)) __syncthreads();
-        if (last) break;
-        g0 = g0 + k == b ? 0 : g0 + k;   // after the top group, bottom-up
-        k = min(KM, b - k0 - g0);
+    const bool direct_out = a.direct_out != 0;
+    for (int i = 0; i < kMaxGroups; ++i) {
+        const PassGroup& g = a.g[i];
+        const bool to_out = g.last && direct_out;
+        rgroup_k<P, SGN, T, TI, KM>((i == 0 ? 1 : 0) | (to_out ? 2 : 0) | (i != 0 && !to_out ? 4 : 0), sm, in, out, g, a,
+                                    tw, ncols);
+        if (!to_out) __syncthreads();
+        if (g.last) break;
     }
     if (!direct_out) {
         const int nel = a.R << a.wlog;
@@ -321,7 +349,7 @@ __device__ __forceinline__ void pass_body(const PassArgs& a, const Tw& tw, long 
             const int r = e >> a.wlog, c = e & cmask;
             if (c < ncols) {
                 T v = sm[sx<P, T>(e)];
-                if (a.do_scale) v = scale_by<T>(v, a.scale);
+                if (a.do_scale) v = scale_of<T>(a, v);
                 out[c + (long long)r * a.S] = v;
             }
         }
@@ -365,8 +393,8 @@ __global__ void __maxnreg__(pass_maxnreg<P>()) k_pass_grouped(const __grid_const
         else hi = mid - 1;
     }
     const GroupPass& g = jobs[lo];
-    const long long local = b - g.first;
-    pass_body<P, T, TI, SGN, KM>(g.a, list.tw, local % g.ntile, local / g.ntile);
+    const unsigned local = (unsigned)(b - g.first), fn = local / (unsigned)g.ntile;
+    pass_body<P, T, TI, SGN, KM>(g.a, list.tw, local - fn * (unsigned)g.ntile, fn);
 }
 
 // ---------------------------------------------------------------------------
@@ -419,36 +447,22 @@ __global__ void __maxnreg__(96) k_mid(MidArgs m, int nwb, const __grid_constant_
     float* bins = reinterpret_cast<float*>(smraw + ((tile_elems * sizeof(T) + 15) & ~(size_t)15));
     const int nb2 = 2 * m.nb;
     const long long fn = blockIdx.y;
-    const long long tile = blockIdx.x;
-    const long long lo0 = (tile % a.nlo) << a.wlog;
-    const long long base = lo0 + (tile / a.nlo) * a.SR;
+    const unsigned tile = blockIdx.x, th = tile / a.nlo;
+    const long long lo0 = (long long)(tile - th * a.nlo) << a.wlog;
+    const long long base = lo0 + th * a.SR;
     const int ncols = (int)min((long long)a.Wc, a.S - lo0);
     const int cmask = a.Wc - 1;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const TI* in = reinterpret_cast<const TI*>(a.in) + fn * a.ld_in + base;
     T* out = reinterpret_cast<T*>(a.out) + fn * a.ld_out + base;
     for (int i = threadIdx.x; i < nwb * nb2 * 32; i += blockDim.x) bins[i] = 0.f;
-    const int b = a.b;
-    const int k0 = min(KM, b);
-    const int g_last = b == k0 ? 0 : ((b - k0 - 1) / KM) * KM;
-    long long run = 1;
-    if (a.S == 1) {
-        for (int i = 0; i < g_last; ++i) run *= P;
-    } else {
-        run = a.Wc;
-    }
-    const bool direct_out = run * (long long)sizeof(T) >= 64;
+    const bool direct_out = a.direct_out != 0;
     // forward stages
-    {
-        int g0 = b - k0, k = k0;
-        for (;;) {
-            const bool first = g0 + k == b;
-            rgroup_k<P, -1, T, TI, KM>(k, first ? 1 : 4, sm, in, out, g0, a, tw, ncols);
-            __syncthreads();
-            if (g0 == g_last) break;
-            g0 = first ? 0 : g0 + k;
-            k = min(KM, b - k0 - g0);
-        }
+    for (int i = 0; i < kMaxGroups; ++i) {
+        const PassGroup& g = a.g[i];
+        rgroup_k<P, -1, T, TI, KM>(i == 0 ? 1 : 4, sm, in, out, g, a, tw, ncols);
+        __syncthreads();
+        if (g.last) break;
     }
     // scale, weight, coefficients, class partials; the weight and class loads
     // of 8 elements per thread are issued together
@@ -474,7 +488,7 @@ __global__ void __maxnreg__(96) k_mid(MidArgs m, int nwb, const __grid_constant_
                 const int r = e >> a.wlog, c = e & cmask;
                 if (e >= nel || c >= ncols) continue;
                 const long long H = base + c + (long long)r * a.S;
-                T v = mulw<T>(scale_by<T>(sm[sx<P, T>(e)], a.scale), wv[j]);
+                T v = mulw<T>(scale_of<T>(a, sm[sx<P, T>(e)]), wv[j]);
                 if (coef) coef[c + (long long)r * a.S] = v;
                 if (H != 0) {
                     const float q = mag2<T>(v);
@@ -488,17 +502,12 @@ __global__ void __maxnreg__(96) k_mid(MidArgs m, int nwb, const __grid_constant_
     __syncthreads();
     reduce_bins(bins, nb2, nwb, m.part + fn * nb2 * m.ntile + tile, m.ntile);
     // inverse stages of the same digits, in the same order
-    {
-        int g0 = b - k0, k = k0;
-        for (;;) {
-            const bool last = g0 == g_last;
-            const bool dst_g = last && direct_out;
-            rgroup_k<P, +1, T, T, KM>(k, dst_g ? 2 : 4, sm, out, out, g0, a, tw, ncols);
-            if (!dst_g) __syncthreads();
-            if (last) break;
-            g0 = g0 + k == b ? 0 : g0 + k;
-            k = min(KM, b - k0 - g0);
-        }
+    for (int i = 0; i < kMaxGroups; ++i) {
+        const PassGroup& g = a.g[i];
+        const bool dst_g = g.last && direct_out;
+        rgroup_k<P, +1, T, T, KM>(dst_g ? 2 : 4, sm, out, out, g, a, tw, ncols);
+        if (!dst_g) __syncthreads();
+        if (g.last) break;
     }
     if (!direct_out) {
         for (int e = threadIdx.x; e < nel; e += blockDim.x) {
@@ -528,7 +537,10 @@ static int set_smem(F* kern, size_t bytes) {
     return smem_limit_max(kern);
 }
 
-static PassArgs pass_args(const PassGeom& g, const void* in, void* out, long long ld_in, long long ld_out) {
+// geometry of one pass with register groups of at most km digits: the top
+// group first, then from the lowest digit up
+static PassArgs pass_args(int p, int km, int elem, const PassGeom& g, const void* in, void* out, long long ld_in,
+                          long long ld_out) {
     PassArgs a;
     a.in = in;
     a.out = out;
@@ -536,14 +548,40 @@ static PassArgs pass_args(const PassGeom& g, const void* in, void* out, long lon
     a.ld_out = ld_out;
     a.S = g.S;
     a.SR = g.S * g.R;
-    a.nlo = g.nlo;
+    a.nlo = (unsigned)g.nlo;
     a.R = g.R;
-    a.b = g.b;
     a.Wc = g.Wc;
     a.wlog = g.wlog;
     a.scale = 1.0;
+    a.scalef = 1.f;
     a.do_scale = 0;
+    const int k0 = std::min(km, g.b);
+    int g0 = g.b - k0, k = k0, g_last = 0;
+    for (int i = 0; i < kMaxGroups; ++i) {
+        PassGroup& x = a.g[i];
+        x.k = k;
+        x.pg0 = (unsigned)ipow_ll(p, g0);
+        x.nrh = (unsigned)(g.R / ipow_ll(p, g0 + k));
+        x.mg_lo = x.pg0 == 1 ? 0u : (unsigned)((1ull << 32) / x.pg0 + 1);
+        x.mg_hi = x.nrh == 1 ? 0u : (unsigned)((1ull << 32) / x.nrh + 1);
+        g_last = g0;
+        const int next = i == 0 ? 0 : g0 + k;
+        x.last = next >= g.b - k0;
+        if (x.last) break;
+        g0 = next;
+        k = std::min(km, g.b - k0 - g0);
+    }
+    // a run of neighbouring elements below the last group (p^g0 rows in the low
+    // pass, Wc columns in the others) of at least 64 bytes
+    const long long run = g.S == 1 ? ipow_ll(p, g_last) : g.Wc;
+    a.direct_out = run * elem >= 64;
     return a;
+}
+
+static void pass_scale(PassArgs& a, double scale) {
+    a.do_scale = 1;
+    a.scale = scale;
+    a.scalef = (float)scale;
 }
 
 static const char* pass_family(int t, int q) { return t == 0 ? "pass_lo" : (t == q - 1 ? "pass_hi" : "pass_mid"); }
@@ -609,14 +647,14 @@ static int transform_pp(dwt_plan_s* Pl, const PassPlan& pp, double scale_by_n, c
             const PassGeom& g = pp.g[t];
             int rc;
             if (t == 0) {
-                PassArgs a = pass_args(g, (const TI*)in + (long long)f0 * ld_in, (T*)out + (long long)f0 * ld_out,
+                PassArgs a = pass_args(P, KMax<P, T>::v, (int)sizeof(T), g, (const TI*)in + (long long)f0 * ld_in, (T*)out + (long long)f0 * ld_out,
                                        ld_in, ld_out);
-                if (scale && pp.q == 1) { a.do_scale = 1; a.scale = scale_by_n; }
+                if (scale && pp.q == 1) pass_scale(a, scale_by_n);
                 rc = launch_pass<P, T, TI, SGN>(g, a, tw, nf, pass_family(t, pp.q), st);
             } else {
-                PassArgs a = pass_args(g, (const T*)out + (long long)f0 * ld_out, (T*)out + (long long)f0 * ld_out,
+                PassArgs a = pass_args(P, KMax<P, T>::v, (int)sizeof(T), g, (const T*)out + (long long)f0 * ld_out, (T*)out + (long long)f0 * ld_out,
                                        ld_out, ld_out);
-                if (scale && t == pp.q - 1) { a.do_scale = 1; a.scale = scale_by_n; }
+                if (scale && t == pp.q - 1) pass_scale(a, scale_by_n);
                 rc = launch_pass<P, T, T, SGN>(g, a, tw, nf, pass_family(t, pp.q), st);
             }
             if (rc) return rc;
@@ -739,17 +777,11 @@ static int grouped_t(const std::vector<GroupJob>& js, cudaStream_t st) {
             const PassGeom& g = pp.g[t];
             GroupPass gp;
             if (t == 0) {
-                gp.a = pass_args(g, j.in, j.out, j.ld_in, j.ld_out);
-                if (scale && pp.q == 1) {
-                    gp.a.do_scale = 1;
-                    gp.a.scale = 1.0 / (double)j.plan->N;
-                }
+                gp.a = pass_args(P, KMax<P, T>::v, (int)sizeof(T), g, j.in, j.out, j.ld_in, j.ld_out);
+                if (scale && pp.q == 1) pass_scale(gp.a, 1.0 / (double)j.plan->N);
             } else {
-                gp.a = pass_args(g, j.out, j.out, j.ld_out, j.ld_out);
-                if (scale && t == pp.q - 1) {
-                    gp.a.do_scale = 1;
-                    gp.a.scale = 1.0 / (double)j.plan->N;
-                }
+                gp.a = pass_args(P, KMax<P, T>::v, (int)sizeof(T), g, j.out, j.out, j.ld_out, j.ld_out);
+                if (scale && t == pp.q - 1) pass_scale(gp.a, 1.0 / (double)j.plan->N);
             }
             gp.ntile = g.ntile;
             gp.first = blocks;
@@ -834,19 +866,20 @@ static int interpolate_t(dwt_plan_s* Pl, const void* f, void* c, void* coef, int
         for (int t = 0; t + 1 < pp.q; ++t) {
             const PassGeom& g = pp.g[t];
             if (t == 0) {
-                PassArgs a = pass_args(g, (const TI*)f + off, (T*)c + off, ld, ld);
+                PassArgs a = pass_args(P, KMax<P, T>::v, (int)sizeof(T), g, (const TI*)f + off, (T*)c + off, ld, ld);
                 rc = launch_pass<P, T, TI, -1>(g, a, tw, nf, "interp_fwd", st);
             } else {
-                PassArgs a = pass_args(g, (const T*)c + off, (T*)c + off, ld, ld);
+                PassArgs a = pass_args(P, KMax<P, T>::v, (int)sizeof(T), g, (const T*)c + off, (T*)c + off, ld, ld);
                 rc = launch_pass<P, T, T, -1>(g, a, tw, nf, "interp_fwd", st);
             }
             if (rc) return rc;
         }
         // fused top pass
         MidArgs m;
-        if (pp.q == 1) m.pa = pass_args(gm, (const TI*)f + off, (T*)c + off, ld, ld);
-        else m.pa = pass_args(gm, (const T*)c + off, (T*)c + off, ld, ld);
+        if (pp.q == 1) m.pa = pass_args(P, KM, (int)sizeof(T), gm, (const TI*)f + off, (T*)c + off, ld, ld);
+        else m.pa = pass_args(P, KM, (int)sizeof(T), gm, (const T*)c + off, (T*)c + off, ld, ld);
         m.pa.scale = 1.0 / (double)Pl->N;
+        m.pa.scalef = (float)m.pa.scale;
         m.W = weight == DWT_WEIGHT_INV_SQ_WAVENUMBER ? Pl->d_W : nullptr;
         m.cls = Pl->d_cls;
         m.coef = coef ? (void*)((T*)coef + off) : nullptr;
@@ -863,7 +896,7 @@ static int interpolate_t(dwt_plan_s* Pl, const void* f, void* c, void* coef, int
         // inverse passes below the top one, in place on c
         for (int t = pp.q - 2; t >= 0; --t) {
             const PassGeom& g = pp.g[t];
-            PassArgs a = pass_args(g, (const T*)c + off, (T*)c + off, ld, ld);
+            PassArgs a = pass_args(P, KMax<P, T>::v, (int)sizeof(T), g, (const T*)c + off, (T*)c + off, ld, ld);
             rc = launch_pass<P, T, T, +1>(g, a, tw, nf, "interp_inv", st);
             if (rc) return rc;
         }
