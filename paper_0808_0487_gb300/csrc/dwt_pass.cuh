@@ -320,7 +320,9 @@ __device__ __forceinline__ void rgroup_k(int mode, T* sm, const TI* gin, T* gout
 // Register cap: 96 x 512 threads fit the register file; a single digit of a
 // prime above 13 holds p complex elements and the p-point sums, so those
 // passes get 160 registers and at most 384 threads.
-template <int P> constexpr int pass_maxnreg() { return P > 13 ? 160 : 96; }
+template <int P, typename T> constexpr int pass_maxnreg() {
+    return P > 13 ? 160 : sizeof(T) == 8 && P == 3 ? 80 : sizeof(T) == 8 && P == 5 ? 72 : 96;
+}
 template <int P> constexpr long long pass_max_threads() { return P > 13 ? 384 : 512; }
 
 template <int P, typename T, typename TI, int SGN, int KM>
@@ -357,7 +359,7 @@ __device__ __forceinline__ void pass_body(const PassArgs& a, const Tw& tw, unsig
 }
 
 template <int P, typename T, typename TI, int SGN, int KM>
-__global__ void __maxnreg__(pass_maxnreg<P>()) k_pass(PassArgs a, const __grid_constant__ Tw tw) {
+__global__ void __maxnreg__((pass_maxnreg<P, T>())) k_pass(PassArgs a, const __grid_constant__ Tw tw) {
     chain_begin();
     pass_body<P, T, TI, SGN, KM>(a, tw, blockIdx.x, blockIdx.y);
 }
@@ -382,7 +384,7 @@ struct GroupList {
 };
 
 template <int P, typename T, typename TI, int SGN, int KM>
-__global__ void __maxnreg__(pass_maxnreg<P>()) k_pass_grouped(const __grid_constant__ GroupList list) {
+__global__ void __maxnreg__(P > 13 ? 160 : 96) k_pass_grouped(const __grid_constant__ GroupList list) {
     chain_begin();
     const GroupPass* jobs = list.n > kGroupInline ? list.far : list.near;
     const long long b = blockIdx.x;
@@ -464,38 +466,53 @@ __global__ void __maxnreg__(96) k_mid(MidArgs m, int nwb, const __grid_constant_
         __syncthreads();
         if (g.last) break;
     }
-    // scale, weight, coefficients, class partials; the weight and class loads
-    // of 8 elements per thread are issued together
+    // scale, weight, coefficients, class partials: lane l of warp w < nwb takes the
+    // elements 32 w + l, + 32 nwb, ... in order, eight at a time with their weight
+    // and class loads in flight together.  Labels fit 32 bits (N <= 2^31).  Two
+    // elements' bins are loaded together and stored together; if both fall in one
+    // bin the second adds to the first's sum.
     if (w < nwb) {
-        float* mybins = bins + (size_t)w * nb2 * 32 + lane;
-        T* coef = m.coef ? reinterpret_cast<T*>(m.coef) + fn * a.ld_out + base : nullptr;
+        float* bt = bins + (size_t)w * nb2 * 32 + lane;
+        float* bs = bt + m.nb * 32;
+        T* coef = m.coef ? reinterpret_cast<T*>(m.coef) + fn * a.ld_out : nullptr;
         const int step = nwb * 32;
+        const unsigned S = (unsigned)a.S, base32 = (unsigned)base;
         for (int e0 = threadIdx.x; e0 < nel; e0 += 8 * step) {
             float wv[8];
-            uchar2 kc[8];
+            unsigned kc[8], H[8];
+            bool ok[8];
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
                 const int e = e0 + j * step;
                 const int r = e >> a.wlog, c = e & cmask;
-                const long long H = base + c + (long long)r * a.S;
-                const bool ok = e < nel && c < ncols;
-                wv[j] = ok && m.W ? __ldg(m.W + H) : 1.f;
-                kc[j] = ok ? __ldg(reinterpret_cast<const uchar2*>(m.cls) + H) : make_uchar2(0, 0);
+                ok[j] = e < nel && c < ncols;
+                H[j] = ok[j] ? base32 + (unsigned)c + (unsigned)r * S : 0u;
+                wv[j] = m.W ? __ldg(m.W + H[j]) : 1.f;
+                kc[j] = __ldg(reinterpret_cast<const unsigned short*>(m.cls) + H[j]);
             }
 #pragma unroll
-            for (int j = 0; j < 8; ++j) {
-                const int e = e0 + j * step;
-                const int r = e >> a.wlog, c = e & cmask;
-                if (e >= nel || c >= ncols) continue;
-                const long long H = base + c + (long long)r * a.S;
-                T v = mulw<T>(scale_of<T>(a, sm[sx<P, T>(e)]), wv[j]);
-                if (coef) coef[c + (long long)r * a.S] = v;
-                if (H != 0) {
-                    const float q = mag2<T>(v);
-                    mybins[(int)kc[j].x * 32] += q;
-                    mybins[(m.nb + (int)kc[j].y) * 32] += q;
+            for (int j = 0; j < 8; j += 2) {
+                float q[2];
+#pragma unroll
+                for (int u = 0; u < 2; ++u) {
+                    q[u] = 0.f;   // the label H = 0 is in no class
+                    if (ok[j + u]) {
+                        T& x = sm[sx<P, T>(e0 + (j + u) * step)];
+                        const T v = mulw<T>(scale_of<T>(a, x), wv[j + u]);
+                        x = v;
+                        if (coef) coef[H[j + u]] = v;
+                        if (H[j + u] != 0) q[u] = mag2<T>(v);
+                    }
                 }
-                sm[sx<P, T>(e)] = v;
+                const int kt0 = (int)(kc[j] & 255u), ks0 = (int)(kc[j] >> 8);
+                const int kt1 = (int)(kc[j + 1] & 255u), ks1 = (int)(kc[j + 1] >> 8);
+                const float xt0 = bt[32 * kt0], xt1 = bt[32 * kt1], xs0 = bs[32 * ks0], xs1 = bs[32 * ks1];
+                const float rt0 = xt0 + q[0], rs0 = xs0 + q[0];
+                const float rt1 = (kt1 == kt0 ? rt0 : xt1) + q[1], rs1 = (ks1 == ks0 ? rs0 : xs1) + q[1];
+                bt[32 * kt0] = rt0;
+                bs[32 * ks0] = rs0;
+                bt[32 * kt1] = rt1;
+                bs[32 * ks1] = rs1;
             }
         }
     }
