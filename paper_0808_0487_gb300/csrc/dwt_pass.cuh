@@ -423,13 +423,25 @@ template <> __device__ __forceinline__ float2 mulw<float2>(float2 v, float w) { 
 // per-lane FP32 class sums of the first nwb warps -> one FP64 value per class
 // and tile, fixed order
 __device__ __forceinline__ void reduce_bins(const float* bins, int nb2, int nwb, double* out, long long stride) {
+    // four classes at a time: their trees overlap
     const int nw = blockDim.x >> 5, w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    for (int bi = w; bi < nb2; bi += nw) {
-        float x = 0.f;
-        for (int ww = 0; ww < nwb; ++ww) x += bins[(ww * nb2 + bi) * 32 + lane];
+    for (int b0 = 4 * w; b0 < nb2; b0 += 4 * nw) {
+        float x[4] = {0.f, 0.f, 0.f, 0.f};
+        for (int ww = 0; ww < nwb; ++ww) {
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-        if (lane == 0) out[bi * stride] = (double)x;
+            for (int k = 0; k < 4; ++k)
+                if (b0 + k < nb2) x[k] += bins[(ww * nb2 + b0 + k) * 32 + lane];
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+#pragma unroll
+            for (int k = 0; k < 4; ++k) x[k] += __shfl_xor_sync(0xffffffffu, x[k], o);
+        }
+        if (lane == 0) {
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                if (b0 + k < nb2) out[(b0 + k) * stride] = (double)x[k];
+        }
     }
 }
 
@@ -457,7 +469,8 @@ __global__ void __maxnreg__(96) k_mid(MidArgs m, int nwb, const __grid_constant_
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const TI* in = reinterpret_cast<const TI*>(a.in) + fn * a.ld_in + base;
     T* out = reinterpret_cast<T*>(a.out) + fn * a.ld_out + base;
-    for (int i = threadIdx.x; i < nwb * nb2 * 32; i += blockDim.x) bins[i] = 0.f;
+    for (int i = threadIdx.x; i < nwb * nb2 * 8; i += blockDim.x)
+        reinterpret_cast<float4*>(bins)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
     const bool direct_out = a.direct_out != 0;
     // forward stages
     for (int i = 0; i < kMaxGroups; ++i) {
@@ -634,8 +647,18 @@ static int launch_pass(const PassGeom& g, const PassArgs& a, const Tw& tw, int n
 }
 
 // L2-sized groups of functions: the passes of one group run back to back so
-// that the intermediate stays in the 126 MB L2 between passes.
-static const long long kL2Group = 48ll << 20;
+// that the intermediate stays in the 126 MB L2 between passes.  Groups of a
+// batch are equally large, so that none ends with launches of few blocks
+// (p = 3, m = 13: interpolation of 4 functions in groups of 3 + 1 100 us, of 4
+// 88 us; forward of 32: 48 MB 299 us, 64 MB 277 us, 96 MB 275 us; p = 5, m = 9,
+// 32 functions: 394, 394 and 406 us).
+static const long long kL2Group = 64ll << 20;
+
+static int functions_per_group(long long bytes, long long fbytes, int batch) {
+    const long long g = std::min(65535ll, std::max(1ll, bytes / fbytes));
+    const long long n = (batch + g - 1) / g;
+    return (int)((batch + n - 1) / n);
+}
 
 template <int P, typename T, typename TI, int SGN>
 static int transform_pp(dwt_plan_s* Pl, const PassPlan& pp, double scale_by_n, const void* in, void* out, int batch,
@@ -655,8 +678,7 @@ static int transform_pp(dwt_plan_s* Pl, const PassPlan& pp, double scale_by_n, c
                         long long ld_in, long long ld_out, cudaStream_t st) {
     static const Tw tw = make_tw(P);
     const long long fbytes = Pl->N * (long long)sizeof(T);
-    int G = (int)std::max(1ll, (Pl->tuned_group_bytes > 0 ? Pl->tuned_group_bytes : kL2Group) / fbytes);
-    G = std::min(G, 65535);
+    const int G = functions_per_group(Pl->tuned_group_bytes > 0 ? Pl->tuned_group_bytes : kL2Group, fbytes, batch);
     const bool scale = SGN < 0 && !std::is_same<T, int>::value;
     for (int f0 = 0; f0 < batch; f0 += G) {
         const int nf = std::min(G, batch - f0);
@@ -874,8 +896,7 @@ static int interpolate_t(dwt_plan_s* Pl, const void* f, void* c, void* coef, int
     rc = set_smem(kmid_next, smem);
     if (rc) return rc;
     const long long fbytes = Pl->N * (long long)sizeof(T);
-    int G = (int)std::max(1ll, kL2Group / fbytes);
-    G = std::min(G, 65535);
+    const int G = functions_per_group(kL2Group, fbytes, batch);
     for (int f0 = 0; f0 < batch; f0 += G) {
         const int nf = std::min(G, batch - f0);
         const long long off = (long long)f0 * ld;

@@ -21,9 +21,11 @@
 // net points, its 1 + 2s DWTs, and keeps W_K = 1 / (p^m K~) and the 2s
 // variance tables (real parts: the kernels are real and symmetric, so their
 // DWTs are real up to rounding).  dwt_spline then transforms each function,
-// multiplies by W_K, transforms back, and contracts |c~|^2 with the tables in
-// a fixed summation order.
+// multiplies by W_K, contracts |c~|^2 with the tables in a fixed summation
+// order, and transforms back.
+#include <cuda_fp16.h>
 #include <math.h>
+#include <string.h>
 
 #include <algorithm>
 #include <vector>
@@ -35,7 +37,7 @@ namespace dwt {
 namespace {
 
 constexpr int kSplineMaxS = 64;
-constexpr int kDotTile = 4096;   // labels per block of the variance contraction
+constexpr int kDotTile = 4096;   // points per block of the hold-out error
 
 // kernel data at point n: K, R_1..R_s, E_1..E_s (rows of `out`, ld N)
 __global__ void k_spline_data(const uint32_t* __restrict__ Y, long long N, int s, int p, int m,
@@ -85,59 +87,247 @@ __global__ void k_spline_tables(const double* __restrict__ tr, int cplx, long lo
     }
 }
 
-// c~ = f~ W_K in place ([batch][N], real or interleaved complex)
-__global__ void k_spline_scale(double* ft, int cplx, long long N, long long total, const double* __restrict__ W) {
+// c~ = f~ W_K in place ([batch][ld], real or interleaved complex): only where no
+// variances are asked for (k_spline_dots scales on its way)
+__global__ void k_spline_scale(double* ft, int cplx, long long N, long long ld, long long total,
+                               const double* __restrict__ W) {
     for (long long x = blockIdx.x * (long long)blockDim.x + threadIdx.x; x < total;
          x += (long long)gridDim.x * blockDim.x) {
-        const double w = W[x % N];
+        const long long b = x / N, H = x - b * N, o = b * ld + H;
+        const double w = W[H];
         if (cplx) {
-            ft[2 * x] *= w;
-            ft[2 * x + 1] *= w;
+            ft[2 * o] *= w;
+            ft[2 * o + 1] *= w;
         } else {
-            ft[x] *= w;
+            ft[o] *= w;
         }
     }
 }
 
-// partial sums of |c~(H)|^2 T_t(H) over one tile of labels, for all 2s tables:
-// part[(b * 2s + t) * ntile + tile]; per thread in label order, then a fixed
-// tree.  Consecutive blocks take the same tile for consecutive functions, so a
-// tile's table rows come from HBM once and from L2 for the other functions.
-__global__ void __launch_bounds__(256) k_spline_dots(const double* __restrict__ ct, int cplx, long long N, int nt,
-                                                     const double* __restrict__ tab, double* part, long long ntile,
-                                                     long long tile0) {
-    __shared__ double red[256];
-    const long long tile = tile0 + blockIdx.y, b = blockIdx.x;
-    const long long h0 = tile * kDotTile;
-    const int t = threadIdx.x;
-    constexpr int PER = kDotTile / 256;
-    double a[PER];
+// ---- the variance contraction ---------------------------------------------
+// part[(b nt + t) ntile + tile] = sum over the tile's labels of |c~_b(H)|^2 T_t(H),
+// and c~ = f~ W_K in place on the way.
+//
+// A batch of 32 functions against 32 tables is a matrix product with the labels
+// as inner dimension, in FP64.  This GPU multiplies 1.7 FP64 numbers per clock
+// and SM, so the product runs on the tensor cores in exact pieces instead: in
+// blocks of 64 labels every operand becomes a 64-bit fixed-point number, scaled
+// by its row's largest exponent so far in the tile, split into eight signed
+// digits of base 256 that FP16 holds exactly; a digit product is below 2^14 and
+// the 8 x 64 products that share a weight sum to less than 2^24, exact in FP32.
+// The 36 digit pairs of weight >= 256^7 are multiplied (the others lie 2^-62
+// below the largest product); the sums join 128-bit integers per pair of
+// function and table, shifted when a row's exponent grows, and become FP64 once
+// per tile.  FP64 rounds every product and every sum at 2^-53.  Rows with an
+// infinity or a NaN in the tile take FP64 sums at the end.
+//
+// p = 2, m = 20, s = 16, 32 functions: 2920 us on the FP64 pipe (one CTA per
+// function and 4096 labels) plus 95 us for the scaling.
+constexpr int kDotThreads = 256;
+constexpr int kDotRows = 32;                  // functions, and tables, per round
+constexpr int kDotK = 64;                     // labels per block
+constexpr int kDotStride = kDotK + 8;         // halves per digit row (16-byte rows on all banks)
+constexpr int kDotPlane = kDotRows * kDotStride;
+constexpr int kDotDigits = 8;
+constexpr int kDotOperand = kDotDigits * kDotPlane;   // halves of one operand
+constexpr size_t kDotSmem = (size_t)2 * kDotOperand * 2 + 4 * kDotRows * 4;
+
+__device__ __forceinline__ int expo(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
+
+// 64-bit fixed point of x against exponent E (>= x's): significand 2^9 at E
+__device__ __forceinline__ unsigned long long to_fix64(double x, int E) {
+    const int ex = expo(x);
+    unsigned long long mnt = (unsigned long long)__double_as_longlong(x) & 0xfffffffffffffull;
+    if (ex) mnt |= 0x10000000000000ull;
+    const int d = E - max(ex, 1);
+    mnt = d > 63 ? 0ull : (mnt << 9) >> d;
+    return __double2hiint(x) < 0 ? 0ull - mnt : mnt;
+}
+
+// the digits of two numbers (label l and l + 32 of a block) into their planes
+__device__ __forceinline__ void put_digits(__half* row, unsigned long long f0, unsigned long long f1, int lane) {
+    // + 128 in every byte with carries: byte - 128 is the signed digit
+    f0 += 0x8080808080808080ull;
+    f1 += 0x8080808080808080ull;
+    const uint32_t lo0 = (uint32_t)f0, hi0 = (uint32_t)(f0 >> 32), lo1 = (uint32_t)f1, hi1 = (uint32_t)(f1 >> 32);
+    const __half2 off = __halves2half2(__ushort_as_half(0xE480), __ushort_as_half(0xE480));   // -(1024 + 128)
 #pragma unroll
-    for (int q = 0; q < PER; ++q) {
-        const long long H = h0 + t + 256 * q;
-        double v = 0.0;
-        if (H < N) {
-            const long long x = b * N + H;
-            v = cplx ? ct[2 * x] * ct[2 * x] + ct[2 * x + 1] * ct[2 * x + 1] : ct[x] * ct[x];
-        }
-        a[q] = v;
+    for (int i = 0; i < kDotDigits; ++i) {
+        // bytes i of both behind 0x64: the FP16 numbers 1024 + byte
+        const uint32_t sel = (uint32_t)(i & 3) | ((uint32_t)(4 + (i & 3)) << 4);
+        const uint32_t two = __byte_perm(i < 4 ? lo0 : hi0, i < 4 ? lo1 : hi1, sel);
+        const uint32_t bits = __byte_perm(two, 0x64u, 0x4140);
+        __half2 h;
+        memcpy(&h, &bits, 4);
+        h = __hadd2(h, off);
+        *reinterpret_cast<__half2*>(row + i * kDotPlane + 2 * lane) = h;
     }
-    for (int tb = 0; tb < nt; ++tb) {
-        const double* T = tab + (long long)tb * N;
-        double acc = 0.0;
+}
+
+__device__ __forceinline__ void ldmatrix4(uint32_t (&r)[4], uint32_t addr) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"(addr));
+}
+__device__ __forceinline__ void ldmatrix2(uint32_t (&r)[2], uint32_t addr) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x2.shared.b16 {%0, %1}, [%2];" : "=r"(r[0]), "=r"(r[1]) : "r"(addr));
+}
+__device__ __forceinline__ void mma_f16(float (&d)[4], const uint32_t (&a)[4], const uint32_t (&b)[2]) {
+    asm volatile(
+        "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
+}
+
+// grid (tiles, groups of 32 functions); warp w converts rows 4 w .. 4 w + 3 of
+// both operands and multiplies functions 16 (w & 1) .. + 15 by tables
+// 8 (w >> 1) .. + 7
+template <bool CPLX>
+__global__ void __launch_bounds__(kDotThreads, 2) k_spline_dots(double* ct, long long N, long long ld, int batch, int nt,
+                                                                const double* __restrict__ tab,
+                                                                const double* __restrict__ W, double* part, int ntile,
+                                                                int labels) {
+    extern __shared__ __align__(16) unsigned char smraw[];
+    __half* A = reinterpret_cast<__half*>(smraw);
+    __half* B = A + kDotOperand;
+    int* grow = reinterpret_cast<int*>(B + kDotOperand);   // [2][32]: growth of the rows' exponents in this block
+    int* bad = grow + 2 * kDotRows;                        // [2][32]: rows with an infinity or a NaN
+    const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+    const int tile = blockIdx.x, f0 = blockIdx.y * kDotRows;
+    const long long h0 = (long long)tile * labels, h1 = min(N, h0 + labels);
+    const int fo = 16 * (w & 1), to = 8 * (w >> 1);
+    const uint32_t sA = (uint32_t)__cvta_generic_to_shared(A), sB = (uint32_t)__cvta_generic_to_shared(B);
+    // ldmatrix row addresses of this lane: A (16 rows x 16 labels), B (8 rows x 16)
+    const uint32_t aoff = sA + 2u * (uint32_t)((fo + (lane & 15)) * kDotStride + 8 * (lane >> 4));
+    const uint32_t boff = sB + 2u * (uint32_t)((to + (lane & 7)) * kDotStride + 8 * ((lane >> 3) & 1));
+    for (int t0 = 0; t0 < nt; t0 += kDotRows) {
+        __syncthreads();
+        if (t < 2 * kDotRows) bad[t] = 0;
+        int Ea[4] = {1, 1, 1, 1}, Et[4] = {1, 1, 1, 1};   // exponents of this warp's rows
+        int ea[2] = {1, 1}, et[2] = {1, 1};               // of the rows of this thread's sums
+        long long hi[4] = {0, 0, 0, 0}, lo[4] = {0, 0, 0, 0};   // sum = hi 2^32 + lo
+        for (long long hb = h0; hb < h1; hb += kDotK) {
+            const long long l0 = hb + lane, l1 = l0 + 32;
+            const bool in0 = l0 < h1, in1 = l1 < h1;
+            double a[4][2], x[4][2];
+            const double w0 = t0 == 0 && in0 ? W[l0] : 1.0, w1 = t0 == 0 && in1 ? W[l1] : 1.0;
 #pragma unroll
-        for (int q = 0; q < PER; ++q) {
-            const long long H = h0 + t + 256 * q;
-            if (H < N) acc += a[q] * T[H];
-        }
-        red[t] = acc;
-        __syncthreads();
-        for (int w = 128; w > 0; w >>= 1) {
-            if (t < w) red[t] += red[t + w];
+            for (int k = 0; k < 4; ++k) {
+                const int f = f0 + 4 * w + k, tb = t0 + 4 * w + k;
+                a[k][0] = a[k][1] = x[k][0] = x[k][1] = 0.0;
+                if (f < batch) {
+                    if constexpr (CPLX) {
+                        double2* row = reinterpret_cast<double2*>(ct) + f * ld;
+                        double2 u = in0 ? row[l0] : make_double2(0.0, 0.0), v = in1 ? row[l1] : make_double2(0.0, 0.0);
+                        if (t0 == 0) {
+                            u = make_double2(u.x * w0, u.y * w0);
+                            v = make_double2(v.x * w1, v.y * w1);
+                            if (in0) row[l0] = u;
+                            if (in1) row[l1] = v;
+                        }
+                        a[k][0] = u.x * u.x + u.y * u.y;
+                        a[k][1] = v.x * v.x + v.y * v.y;
+                    } else {
+                        double* row = ct + f * ld;
+                        double u = in0 ? row[l0] : 0.0, v = in1 ? row[l1] : 0.0;
+                        if (t0 == 0) {
+                            u *= w0;
+                            v *= w1;
+                            if (in0) row[l0] = u;
+                            if (in1) row[l1] = v;
+                        }
+                        a[k][0] = u * u;
+                        a[k][1] = v * v;
+                    }
+                }
+                if (tb < nt) {
+                    const double* row = tab + (long long)tb * N;
+                    if (in0) x[k][0] = row[l0];
+                    if (in1) x[k][1] = row[l1];
+                }
+            }
+            __syncthreads();   // the previous block's digits and growths have been read
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                auto put = [&](double (&v)[2], int& E, int side, __half* plane) {
+                    const int r = 4 * w + k;
+                    int m0 = expo(v[0]), m1 = expo(v[1]);
+                    if (m0 == 0x7ff || m1 == 0x7ff) {
+                        bad[side * kDotRows + r] = 1;
+                        v[0] = v[1] = 0.0;
+                        m0 = m1 = 0;
+                    }
+                    const int top = max((int)__reduce_max_sync(0xffffffffu, max(m0, m1)), E);
+                    if (lane == 0) grow[side * kDotRows + r] = top - E;
+                    E = top;
+                    put_digits(plane + r * kDotStride, to_fix64(v[0], E), to_fix64(v[1], E), lane);
+                };
+                put(a[k], Ea[k], 0, A);
+                put(x[k], Et[k], 1, B);
+            }
             __syncthreads();
+            float acc[kDotDigits][4] = {};
+#pragma unroll 1
+            for (int k = 0; k < kDotK / 16; ++k) {
+                uint32_t fb[kDotDigits][2];
+#pragma unroll
+                for (int j = 0; j < kDotDigits; ++j) ldmatrix2(fb[j], boff + 2u * (uint32_t)(j * kDotPlane + 16 * k));
+#pragma unroll
+                for (int i = 0; i < kDotDigits; ++i) {
+                    uint32_t fa[4];
+                    ldmatrix4(fa, aoff + 2u * (uint32_t)(i * kDotPlane + 16 * k));
+#pragma unroll
+                    for (int j = kDotDigits - 1 - i; j < kDotDigits; ++j) mma_f16(acc[i + j - kDotDigits + 1], fa, fb[j]);
+                }
+            }
+            // this thread's sums: rows fo + lane / 4 (+ 8), tables to + 2 (lane % 4) (+ 1)
+            int ga[2], gt[2];
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                ga[u] = grow[fo + (lane >> 2) + 8 * u];
+                gt[u] = grow[kDotRows + to + 2 * (lane & 3) + u];
+                ea[u] += ga[u];
+                et[u] += gt[u];
+            }
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int g = ga[q >> 1] + gt[q & 1];
+                if (g) {
+                    __int128 v = ((__int128)hi[q] << 32) + lo[q];
+                    v = g > 126 ? (__int128)0 : v >> g;
+                    hi[q] = (long long)(v >> 32);
+                    lo[q] = (long long)((unsigned long long)v & 0xffffffffull);
+                }
+                long long s0 = 0, s1 = 0;
+#pragma unroll
+                for (int c = 3; c >= 0; --c) {
+                    s0 = s0 * 256 + (long long)__float2int_rn(acc[c][q]);
+                    s1 = s1 * 256 + (long long)__float2int_rn(acc[c + 4][q]);
+                }
+                lo[q] += s0;
+                hi[q] += s1;
+            }
         }
-        if (t == 0) part[(b * nt + tb) * ntile + tile] = red[0];
-        __syncthreads();
+        __syncthreads();   // bad is complete, c~ of the tile is written
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int fr = fo + (lane >> 2) + 8 * (q >> 1), tr = to + 2 * (lane & 3) + (q & 1);
+            const int f = f0 + fr, tb = t0 + tr;
+            if (f >= batch || tb >= nt) continue;
+            double v;
+            if (bad[fr] || bad[kDotRows + tr]) {
+                v = 0.0;
+                for (long long H = h0; H < h1; ++H) {
+                    const double* c = ct + (f * ld + H) * (CPLX ? 2 : 1);
+                    const double m2 = CPLX ? c[0] * c[0] + c[1] * c[1] : c[0] * c[0];
+                    v += m2 * tab[(long long)tb * N + H];
+                }
+            } else {
+                // digits of weight 256^7 and up; 2^(E - 1084) is the unit of a row
+                v = scalbn((double)hi[q] * 4294967296.0 + (double)lo[q], 56 + ea[q >> 1] + et[q & 1] - 2168);
+            }
+            part[((long long)f * nt + tb) * ntile + tile] = v;
+        }
     }
 }
 
@@ -640,46 +830,50 @@ int run_spline(dwt_plan_s* P, const double* f, void* c, int batch, long long ld,
     const int s = P->s;
     const bool cplx = P->p != 2;
     const size_t eb = cplx ? 16 : 8;
-    double* ft = nullptr;
+    // f~ and c~ lie in c when there is one (the transforms run in place)
+    double* ft = reinterpret_cast<double*>(c);
+    const long long ldt = c ? ld : N;
     double* part = nullptr;
-    const long long ntile = (N + kDotTile - 1) / kDotTile;
     const bool want_var = var_trc || var_sup || dim;
-    if (dmalloc((void**)&ft, (size_t)batch * N * eb, st) ||
+    const int groups = (batch + kDotRows - 1) / kDotRows;
+    if (groups > 65535) {
+        set_error("dwt_spline: batch too large");
+        return DWT_EINVAL;
+    }
+    // tiles of 1024 labels, shorter ones where those leave SMs without a tile
+    int labels = 1024;
+    while (labels > kDotK && (N + labels - 1) / labels * groups < 2 * 152) labels /= 2;
+    const int ntile = (int)((N + labels - 1) / labels);
+    if ((!c && dmalloc((void**)&ft, (size_t)batch * N * eb, st)) ||
         (want_var && dmalloc((void**)&part, (size_t)batch * 2 * s * ntile * 8, st))) {
-        dfree(ft, st);
+        if (!c) dfree(ft, st);
         return DWT_ENOMEM;
     }
     auto cleanup = [&]() {
-        dfree(ft, st);
+        if (!c) dfree(ft, st);
         dfree(part, st);
     };
-    int rc = run_transform(P, f, ft, batch, ld, N, DWT_F64, cplx ? DWT_C128 : DWT_F64, -1, st);
+    int rc = run_transform(P, f, ft, batch, ld, ldt, DWT_F64, cplx ? DWT_C128 : DWT_F64, -1, st);
     if (rc) { cleanup(); return rc; }
-    {
+    if (want_var) {
+        auto kern = cplx ? k_spline_dots<true> : k_spline_dots<false>;
+        if ((rc = smem_limit_max(kern))) { cleanup(); return rc; }
+        LaunchScope ls("spline_dots", st);
+        kern<<<dim3((unsigned)ntile, (unsigned)groups), kDotThreads, kDotSmem, st>>>(ft, N, ldt, batch, 2 * s, P->d_splT,
+                                                                                     P->d_splW, part, ntile, labels);
+    } else {
         LaunchScope ls("spline_scale", st);
-        k_spline_scale<<<grid_sp((long long)batch * N), 256, 0, st>>>(ft, cplx ? 1 : 0, N, (long long)batch * N,
+        k_spline_scale<<<grid_sp((long long)batch * N), 256, 0, st>>>(ft, cplx ? 1 : 0, N, ldt, (long long)batch * N,
                                                                      P->d_splW);
     }
-    DWT_CK_LAUNCH("k_spline_scale");
-    if (want_var) {
-        for (int b0 = 0; b0 < batch; b0 += 65535) {
-            const int nb = std::min(65535, batch - b0);
-            for (long long t0 = 0; t0 < ntile; t0 += 65535) {
-                LaunchScope ls("spline_dots", st);
-                k_spline_dots<<<dim3((unsigned)nb, (unsigned)std::min(65535ll, ntile - t0)), 256, 0, st>>>(
-                    ft + (size_t)b0 * N * (eb / 8), cplx ? 1 : 0, N, 2 * s, P->d_splT, part + (size_t)b0 * 2 * s * ntile,
-                    ntile, t0);
-            }
-        }
-        DWT_CK_LAUNCH("k_spline_dots");
-    }
+    DWT_CK_LAUNCH("k_spline_dots");
     if (c) {
-        rc = run_transform(P, ft, c, batch, N, ld, cplx ? DWT_C128 : DWT_F64, cplx ? DWT_C128 : DWT_F64, +1, st);
+        rc = run_transform(P, ft, c, batch, ldt, ld, cplx ? DWT_C128 : DWT_F64, cplx ? DWT_C128 : DWT_F64, +1, st);
         if (rc) { cleanup(); return rc; }
     }
     if (want_var) {
         LaunchScope ls("spline_finalize", st);
-        k_spline_finalize<<<batch, kFinThreads, 0, st>>>(part, (int)ntile, s, sum_rows_lanes(2 * s, ntile, kFinThreads),
+        k_spline_finalize<<<batch, kFinThreads, 0, st>>>(part, ntile, s, sum_rows_lanes(2 * s, ntile, kFinThreads),
                                                          (double)N * (double)N, thr, var_trc, var_sup, dim);
     }
     DWT_CK_LAUNCH("k_spline_finalize");

@@ -94,7 +94,6 @@ __device__ __forceinline__ void load_map(uint32_t (*sm)[256], const Map4* g) {
 constexpr int kTL = 12;                    // labels per tile: 2^12
 constexpr int kTT = 256;                   // threads per tile CTA
 constexpr int kRecBytes = 8192 + 512 + 32; // one tile's records
-constexpr int kFwdL = 8;                   // labels per thread of the forward reading
 
 struct TileArgs {
     const Map4* Q;     // Q_j, j = 0 .. s-2
@@ -245,6 +244,46 @@ __device__ __forceinline__ uint32_t representative(const TileArgs& a, uint32_t U
     return U ^ node;
 }
 
+// levels 3 .. 0 inside a group record gw, from (av, ad) at its root: T_j and d
+// of the 16 leaves
+__device__ __forceinline__ void group_down(const uint32_t (&gw)[8], unsigned av, unsigned ad, uint4& tv, uint4& dv) {
+    unsigned v3[2], d3[2], v2[4], d2[4], v1[8], d1[8];
+#pragma unroll
+    for (int x = 0; x < 2; ++x) {
+        const int b = 28 + (x ^ 1);
+        v3[x] = av;
+        d3[x] = ad;
+        a_step(byte_of(gw[b >> 2], b & 3), 3, v3[x], d3[x]);
+    }
+#pragma unroll
+    for (int x = 0; x < 4; ++x) {
+        const int b = 24 + (x ^ 1);
+        v2[x] = v3[x >> 1];
+        d2[x] = d3[x >> 1];
+        a_step(byte_of(gw[b >> 2], b & 3), 2, v2[x], d2[x]);
+    }
+#pragma unroll
+    for (int x = 0; x < 8; ++x) {
+        const int b = 16 + (x ^ 1);
+        v1[x] = v2[x >> 1];
+        d1[x] = d2[x >> 1];
+        a_step(byte_of(gw[b >> 2], b & 3), 1, v1[x], d1[x]);
+    }
+    uint32_t tw[4] = {0u, 0u, 0u, 0u}, dw[4] = {0u, 0u, 0u, 0u};
+#pragma unroll
+    for (int e = 0; e < 16; ++e) {
+        unsigned v0 = v1[e >> 1], d0 = d1[e >> 1];
+        a_step(byte_of(gw[(e ^ 1) >> 2], (e ^ 1) & 3), 0, v0, d0);
+        const unsigned leaf = byte_of(gw[e >> 2], e & 3);
+        const bool keep = leaf <= v0;
+        const unsigned tau = keep ? leaf : v0;
+        tw[e >> 2] |= tau << (8 * (e & 3));
+        dw[e >> 2] |= (keep ? 0u : d0) << (8 * (e & 3));
+    }
+    tv = make_uint4(tw[0], tw[1], tw[2], tw[3]);
+    dv = make_uint4(dw[0], dw[1], dw[2], dw[3]);
+}
+
 // down, for part `part` of `parts` (a power of two <= 16) of tile `tile`: the
 // groups g = part * G .. part * G + G - 1, G = 256 / parts, each by one thread
 // (A down the tile to its 16 leaves, T_j), then the readings of their 16 G
@@ -291,44 +330,15 @@ __device__ __forceinline__ void tile_down(const TileArgs& a, uint32_t tile, int 
         const uint4 glo = *reinterpret_cast<const uint4*>(R0 + (g << 5));
         const uint4 ghi = *reinterpret_cast<const uint4*>(R0 + (g << 5) + 16);
         const uint32_t gw[8] = {glo.x, glo.y, glo.z, glo.w, ghi.x, ghi.y, ghi.z, ghi.w};
-        unsigned v3[2], d3[2], v2[4], d2[4], v1[8], d1[8];
-#pragma unroll
-        for (int x = 0; x < 2; ++x) {
-            const int b = 28 + (x ^ 1);
-            v3[x] = av;
-            d3[x] = ad;
-            a_step(byte_of(gw[b >> 2], b & 3), 3, v3[x], d3[x]);
+        uint4 tv, dv;
+        group_down(gw, av, ad, tv, dv);
+        if (j == 0) {
+            const uint32_t x = __vmaxu4(__vmaxu4(tv.x, tv.y), __vmaxu4(tv.z, tv.w));
+            mx = max(mx, max(max(x & 255u, (x >> 8) & 255u), max((x >> 16) & 255u, x >> 24)));
         }
-#pragma unroll
-        for (int x = 0; x < 4; ++x) {
-            const int b = 24 + (x ^ 1);
-            v2[x] = v3[x >> 1];
-            d2[x] = d3[x >> 1];
-            a_step(byte_of(gw[b >> 2], b & 3), 2, v2[x], d2[x]);
-        }
-#pragma unroll
-        for (int x = 0; x < 8; ++x) {
-            const int b = 16 + (x ^ 1);
-            v1[x] = v2[x >> 1];
-            d1[x] = d2[x >> 1];
-            a_step(byte_of(gw[b >> 2], b & 3), 1, v1[x], d1[x]);
-        }
-        uint32_t tw[4] = {0u, 0u, 0u, 0u}, dw[4] = {0u, 0u, 0u, 0u};
-#pragma unroll
-        for (int e = 0; e < 16; ++e) {
-            unsigned v0 = v1[e >> 1], d0 = d1[e >> 1];
-            a_step(byte_of(gw[(e ^ 1) >> 2], (e ^ 1) & 3), 0, v0, d0);
-            const unsigned leaf = byte_of(gw[e >> 2], e & 3);
-            const bool keep = leaf <= v0;
-            const unsigned tau = keep ? leaf : v0;
-            tw[e >> 2] |= tau << (8 * (e & 3));
-            dw[e >> 2] |= (keep ? 0u : d0) << (8 * (e & 3));
-            if (j == 0) mx = max(mx, tau);
-        }
-        const uint4 tv = make_uint4(tw[0], tw[1], tw[2], tw[3]);
         *reinterpret_cast<uint4*>(a.T + (((size_t)tile << kTL) | ((size_t)g << 4))) = tv;
         *reinterpret_cast<uint4*>(stau + (t << 4)) = tv;
-        *reinterpret_cast<uint4*>(sd + (t << 4)) = make_uint4(dw[0], dw[1], dw[2], dw[3]);
+        *reinterpret_cast<uint4*>(sd + (t << 4)) = dv;
     }
     __syncthreads();
     // the readings: leaf x = t + kTT i of the part (consecutive threads, consecutive leaves)
@@ -416,18 +426,22 @@ __device__ __forceinline__ uint32_t apply4_ldg(const Map4* M, uint32_t x) {
            __ldg(&M->t[3][x >> 24]);
 }
 
-// The forward reading: labels H = h0 + l * stride, l < kFwdL, of this thread.
-__global__ void __launch_bounds__(256) k_tiles_fwd(const uint32_t* __restrict__ K, const Map4* __restrict__ I0,
+// The forward reading: labels H = h0 + l * stride, l < L, of this thread.  A
+// label's chain of s dependent reads bounds it, so small nets give every label
+// a thread of its own (m = 15, s = 33: 114 us with 8 labels per thread, 21 us
+// with one); large ones keep 8 chains in flight per thread.
+template <int L, typename KT>
+__global__ void __launch_bounds__(256) k_tiles_fwd(const KT* __restrict__ K, const Map4* __restrict__ I0,
                                                    const Map4* __restrict__ Q, unsigned* flags, float* W,
                                                    uint8_t* cls, long long N, int s) {
     if (flags[0] >= kInfB || flags[2]) return;   // the backward sweep did not finish: nothing to read
     const long long stride = (long long)gridDim.x * blockDim.x;
     const long long h0 = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    uint32_t U[kFwdL];
-    unsigned long long pd[kFwdL];
-    uint32_t c[kFwdL];   // last coordinate with k_j != 0 | count << 8
+    uint32_t U[L];
+    unsigned long long pd[L];
+    uint32_t c[L];   // last coordinate with k_j != 0 | count << 8
 #pragma unroll
-    for (int l = 0; l < kFwdL; ++l) {
+    for (int l = 0; l < L; ++l) {
         const long long H = h0 + l * stride;
         U[l] = H < N ? apply4_ldg(I0, (uint32_t)H) : 0u;
         pd[l] = 1ull;
@@ -435,10 +449,10 @@ __global__ void __launch_bounds__(256) k_tiles_fwd(const uint32_t* __restrict__ 
     }
     bool over = false;
     for (int j = 0; j < s; ++j) {
-        const uint32_t* Kj = K + (size_t)j * N;
+        const KT* Kj = K + (size_t)j * N;
         const Map4* Qj = Q + j;
 #pragma unroll
-        for (int l = 0; l < kFwdL; ++l) {
+        for (int l = 0; l < L; ++l) {
             if (h0 + l * stride >= N) continue;
             const uint32_t k = __ldg(Kj + U[l]);
             if (k) {
@@ -451,7 +465,7 @@ __global__ void __launch_bounds__(256) k_tiles_fwd(const uint32_t* __restrict__ 
         }
     }
 #pragma unroll
-    for (int l = 0; l < kFwdL; ++l) {
+    for (int l = 0; l < L; ++l) {
         const long long H = h0 + l * stride;
         if (H >= N) continue;
         W[H] = __fdiv_rn(1.0f, __ull2float_rn(pd[l]));
@@ -459,6 +473,202 @@ __global__ void __launch_bounds__(256) k_tiles_fwd(const uint32_t* __restrict__ 
         cls[2 * H + 1] = (uint8_t)(c[l] >> 8);
     }
     if (over) atomicExch(flags + 1, 1u);
+}
+
+
+// ---------------------------------------------------------------------------
+// The cluster form, 12 <= m <= 16: the backward sweep of the tiled form by one
+// cluster of up to eight CTAs that keep T in shared memory.
+//
+// A coordinate of the tiled form costs two grid-wide waits of about 1.5 us
+// whatever the net's size, and its down pass also reads the representatives
+// k_j(U), which the sweep itself does not need.  Here a CTA owns the groups of
+// 2^ltpc tiles, one per thread, and a copy of the whole T_{j+1} for its gathers
+// T'[U] = T_{j+1}[Q_j(U)]; it writes its part of T_j into every CTA's copy
+// through distributed shared memory (whole rows: single bytes read there from
+// the CTA that owns them took 8 us per coordinate), and the waits are the
+// cluster's own barriers.  Leaves, minima, T_j and d go to global memory for
+// every coordinate, and one launch over all coordinates and labels (k_clu_read)
+// forms the representatives.  The tables are those of the tiled
+// form.  Scratch: 3.1 bytes per label and coordinate (the tiled form: 4), with
+// k_j(U) < 2^16 written over T_j and d, which bounds m.
+constexpr int kCluMax = 16;
+
+struct CluArgs {
+    const Map4* Q;      // Q_j, j = 0 .. s-2
+    uint8_t *leaf;      // [s][N]: T'[U]
+    uint8_t *gmin;      // [s][N/16]: group minima
+    uint8_t *bmin;      // [s][N/256]: block minima
+    uint16_t* td;       // [s][N]: T_j(U) | d << 8, then k_j(U)
+    unsigned* flags;
+    long long N;
+    int m, s, ltpc;
+};
+
+__device__ __forceinline__ uint32_t cluster_addr(uint32_t local, uint32_t rank) {
+    uint32_t r;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(local), "r"(rank));
+    return r;
+}
+__device__ __forceinline__ void st_cluster_v4(uint32_t addr, uint4 v) {
+    asm volatile("st.shared::cluster.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w)
+                 : "memory");
+}
+__device__ __forceinline__ void st_cluster_u8(uint32_t addr, uint32_t v) {
+    asm volatile("st.shared::cluster.u8 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
+}
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+
+// least byte of the n = 2^k bytes at p (aligned to n)
+__device__ __forceinline__ unsigned min_bytes(const uint8_t* p, int n) {
+    if (n == 1) return p[0];
+    if (n == 2) return min((unsigned)p[0], (unsigned)p[1]);
+    uint32_t v = *reinterpret_cast<const uint32_t*>(p);
+    for (int i = 4; i < n; i += 4) v = __vminu4(v, *reinterpret_cast<const uint32_t*>(p + i));
+    return min(min(v & 255u, (v >> 8) & 255u), min((v >> 16) & 255u, v >> 24));
+}
+
+// one cluster of gridDim.x CTAs, 2^ltpc tiles and 256 2^ltpc threads each
+__global__ void __launch_bounds__(512) k_clu_bwd(CluArgs a) {
+    extern __shared__ __align__(16) unsigned char sm[];
+    uint32_t (*qq)[4][256] = reinterpret_cast<uint32_t (*)[4][256]>(sm);   // two maps
+    uint8_t* Ts = sm + 8192;                                              // T
+    uint8_t* st4 = Ts + a.N;                                              // group minima
+    uint8_t* bm = st4 + (256 << a.ltpc);                                  // block minima
+    uint8_t* cl = bm + (16 << a.ltpc);                                    // every tile's minimum
+    const int t = threadIdx.x, nt = blockDim.x;
+    const uint32_t rank = blockIdx.x, ctas = gridDim.x;
+    const uint32_t slice = kTL + a.ltpc;
+    const uint32_t Tb = (uint32_t)__cvta_generic_to_shared(Ts), clb = (uint32_t)__cvta_generic_to_shared(cl);
+    const uint32_t U0 = (rank << slice) | ((uint32_t)t << 4);   // the group's first label
+    const uint32_t tile = (rank << a.ltpc) | (uint32_t)(t >> 8), gt = (uint32_t)(t & 255);
+    unsigned mx = 0;
+    // T_{s-1}(U) = (highest set bit of U) + 1
+    for (uint32_t U = 4u * (uint32_t)t; U < a.N; U += 4u * (uint32_t)nt) {
+        uint32_t x = 0;
+#pragma unroll
+        for (uint32_t b = 0; b < 4; ++b) x |= (U + b ? (uint32_t)(32 - __clz((int)(U + b))) : 0u) << (8 * b);
+        *reinterpret_cast<uint32_t*>(Ts + U) = x;
+    }
+    if (a.s == 1) mx = (unsigned)a.m;
+    for (int i = t; i < 1024 && a.s > 1; i += nt) (&qq[a.s & 1][0][0])[i] = (&a.Q[a.s - 2].t[0][0])[i];
+    cluster_arrive();
+    cluster_wait();
+    for (int j = a.s - 2; j >= 0; --j) {
+        uint32_t (*q)[256] = qq[j & 1];
+        // up: the group's leaves and the minima above them
+        const uint32_t base = apply4(q, U0);   // Q(U0 ^ e) = Q(U0) ^ Q(e), e < 16
+        uint32_t w[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            uint32_t x = 0;
+#pragma unroll
+            for (int b = 0; b < 4; ++b) {
+                x |= (uint32_t)Ts[base ^ q[0][4 * i + b]] << (8 * b);
+            }
+            w[i] = x;
+        }
+        const uint4 lo = make_uint4(w[0], w[1], w[2], w[3]), hi = rec_upper(lo);
+        const uint8_t least = (uint8_t)(hi.w >> 16);
+        st4[t] = least;
+        __syncwarp();
+        uint8_t bleast = 0;
+        if ((t & 15) == 0) bm[t >> 4] = bleast = (uint8_t)min_bytes(st4 + t, 16);
+        __syncthreads();
+        if (gt == 0) {
+            const unsigned v = min_bytes(bm + (t >> 4), 16);
+            for (uint32_t c = 0; c < ctas; ++c) st_cluster_u8(cluster_addr(clb, c) + tile, v);
+        }
+        // the global stores of a phase follow its arrival: a release waits for the
+        // stores before it (about 1 us), and these have until the next one
+        cluster_arrive();
+        uint4 mq = make_uint4(0, 0, 0, 0);   // the next coordinate's map
+        if (j > 0 && t < 256) mq = __ldg(reinterpret_cast<const uint4*>(&a.Q[j - 1].t[0][0]) + t);
+        *reinterpret_cast<uint4*>(a.leaf + (size_t)j * a.N + U0) = lo;
+        a.gmin[(size_t)j * (a.N >> 4) + (U0 >> 4)] = least;
+        if ((t & 15) == 0) a.bmin[(size_t)j * (a.N >> 8) + (U0 >> 8)] = bleast;
+        cluster_wait();   // every tile's minimum is in place; T_{j+1} has been read
+        // down: the candidates of the levels m-1 .. 0 (the sibling of the group's
+        // ancestor of each level, from the tile, block and group minima) and
+        // T_j = min(T', A_0)
+        unsigned av = kInfB, ad = 0;
+        for (int i = a.m - 1; i >= kTL; --i)
+            a_step(min_bytes(cl + (((tile >> (i - kTL)) ^ 1u) << (i - kTL)), 1 << (i - kTL)), i, av, ad);
+#pragma unroll
+        for (int i = 11; i >= 8; --i)
+            a_step(min_bytes(bm + ((t >> 8) << 4) + (((gt >> (i - 4)) ^ 1u) << (i - 8)), 1 << (i - 8)), i, av, ad);
+#pragma unroll
+        for (int i = 7; i >= 4; --i)
+            a_step(min_bytes(st4 + (t & ~255) + (((gt >> (i - 4)) ^ 1u) << (i - 4)), 1 << (i - 4)), i, av, ad);
+        const uint32_t gw[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
+        uint4 tv, dv;
+        group_down(gw, av, ad, tv, dv);
+        if (j == 0) {
+            const uint32_t x = __vmaxu4(__vmaxu4(tv.x, tv.y), __vmaxu4(tv.z, tv.w));
+            mx = max(max(x & 255u, (x >> 8) & 255u), max((x >> 16) & 255u, x >> 24));
+        }
+        if (j > 0)
+            for (uint32_t c = 0; c < ctas; ++c) st_cluster_v4(cluster_addr(Tb, (rank + c) & (ctas - 1)) + U0, tv);
+        if (j > 0 && t < 256) reinterpret_cast<uint4*>(&qq[(j - 1) & 1][0][0])[t] = mq;
+        if (j > 0) cluster_arrive();
+        uint4* o = reinterpret_cast<uint4*>(a.td + (size_t)j * a.N + U0);
+        o[0] = make_uint4(__byte_perm(tv.x, dv.x, 0x5140), __byte_perm(tv.x, dv.x, 0x7362),
+                          __byte_perm(tv.y, dv.y, 0x5140), __byte_perm(tv.y, dv.y, 0x7362));
+        o[1] = make_uint4(__byte_perm(tv.z, dv.z, 0x5140), __byte_perm(tv.z, dv.z, 0x7362),
+                          __byte_perm(tv.w, dv.w, 0x5140), __byte_perm(tv.w, dv.w, 0x7362));
+        if (j > 0) cluster_wait();   // T_j is complete before it is read
+    }
+    for (int o = 16; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    if ((t & 31) == 0) atomicMax(a.flags, mx);
+}
+
+// k_j(U) for every coordinate (blockIdx.y) and label, over T_j and d;
+// k_{s-1}(U) = U.  As representative(), from the leaves and minima.
+__global__ void __launch_bounds__(256) k_clu_read(CluArgs a) {
+    __shared__ __align__(16) uint8_t cl[2 << (kCluMax - kTL)];   // levels 12 .. m
+    const int j = blockIdx.y, t = threadIdx.x;
+    const uint32_t U = blockIdx.x * 256u + (uint32_t)t;
+    uint16_t* td = a.td + (size_t)j * a.N;
+    if (j == a.s - 1) {
+        td[U] = (uint16_t)U;
+        return;
+    }
+    const uint8_t* leaf = a.leaf + (size_t)j * a.N;
+    const uint8_t* gmin = a.gmin + (size_t)j * (a.N >> 4);
+    const uint8_t* bmin = a.bmin + (size_t)j * (a.N >> 8);
+    const int nLB = (int)(a.N >> kTL);
+    const uint32_t x = td[U];
+    if (t < nLB) cl[t] = (uint8_t)min_bytes(bmin + (t << 4), 16);
+    __syncthreads();
+    for (int i = 1; i <= a.m - kTL; ++i) {
+        const int n = nLB >> i;
+        if (t < n) cl[loff(nLB, i) + t] = min(cl[loff(nLB, i - 1) + 2 * t], cl[loff(nLB, i - 1) + 2 * t + 1]);
+        __syncthreads();
+    }
+    const int d = (int)(x >> 8);
+    if (d == 0) {
+        td[U] = 0;
+        return;
+    }
+    const uint32_t tgt = ((x & 255u) - (uint32_t)d) & 255u;
+    int l = d - 1;
+    uint32_t node = (U >> l) ^ 1u;
+    for (; l > kTL; --l) {
+        uint32_t c = (node << 1) | ((U >> (l - 1)) & 1u);
+        if ((uint32_t)cl[loff(nLB, l - 1 - kTL) + c] != tgt) c ^= 1u;
+        node = c;
+    }
+    if (l >= 8) {
+        node = record_step(bmin + ((size_t)(node >> (kTL - l)) << 4), 8, l, node, U, tgt);
+        l = 8;
+    }
+    if (l >= 4) {
+        node = record_step(gmin + ((size_t)(node >> (8 - l)) << 4), 4, l, node, U, tgt);
+        l = 4;
+    }
+    node = record_step(leaf + ((size_t)(node >> (4 - l)) << 4), 0, l, node, U, tgt);
+    td[U] = (uint16_t)(U ^ node);
 }
 
 // The whole construction for a net of N = 2^m <= 2^13 labels in one CTA: both
@@ -621,42 +831,52 @@ bool gf2_inverse(const uint32_t* c, int m, uint32_t* ci) {
     return true;
 }
 
-void make_map(const uint32_t* cols, int m, Map4& M) {
+// B x for the matrix with columns cols
+uint32_t gf2_apply(const uint32_t* cols, uint32_t x) {
+    uint32_t y = 0;
+    for (; x; x &= x - 1) y ^= cols[__builtin_ctz(x)];
+    return y;
+}
+
+// the maps with the given columns ([maps][m]): one block per map.  (Forming the
+// 1024-entry tables on the host and uploading them took about 90 us of a plan
+// build at s = 33.)
+__global__ void __launch_bounds__(256) k_maps(const uint32_t* __restrict__ cols, int m, Map4* M) {
+    const uint32_t* c = cols + (size_t)blockIdx.x * m;
+    const int x = threadIdx.x;
+#pragma unroll
     for (int b = 0; b < 4; ++b) {
-        M.t[b][0] = 0;
-        for (int x = 1; x < 256; ++x) {   // x = (x with its lowest set bit cleared) + that bit
-            const int l = __builtin_ctz((unsigned)x);
-            M.t[b][x] = M.t[b][x & (x - 1)] ^ (8 * b + l < m ? cols[8 * b + l] : 0u);
-        }
+        uint32_t v = 0;
+#pragma unroll
+        for (int l = 0; l < 8; ++l)
+            if (8 * b + l < m && ((x >> l) & 1)) v ^= __ldg(c + 8 * b + l);
+        M[blockIdx.x].t[b][x] = v;
     }
 }
 
-uint32_t host_apply(const Map4& M, uint32_t x) {
-    return M.t[0][x & 255] ^ M.t[1][(x >> 8) & 255] ^ M.t[2][(x >> 16) & 255] ^ M.t[3][x >> 24];
-}
-
 // the one-CTA form for N <= 2^13
-int tree_one(dwt_plan_s* Pl, const std::vector<Map4>& Imap, const std::vector<Map4>& Qmap, cudaStream_t st) {
+int tree_one(dwt_plan_s* Pl, const std::vector<uint32_t>& cols, cudaStream_t st) {
     const long long N = Pl->N;
     const int m = Pl->m, s = Pl->s;
     uint8_t *TU = nullptr, *DU = nullptr;
     Map4* dmaps = nullptr;
+    uint32_t* dcols = nullptr;
     unsigned* flags = nullptr;
     auto cleanup = [&]() {
-        dfree(TU, st); dfree(DU, st); dfree(dmaps, st); dfree(flags, st);
+        dfree(TU, st); dfree(DU, st); dfree(dmaps, st); dfree(dcols, st); dfree(flags, st);
     };
     if (dmalloc((void**)&TU, (size_t)s * N, st) || dmalloc((void**)&DU, (size_t)s * N, st) ||
-        dmalloc((void**)&dmaps, sizeof(Map4) * 2 * s, st) || dmalloc((void**)&flags, 8, st) ||
+        dmalloc((void**)&dmaps, sizeof(Map4) * 2 * s, st) || dmalloc((void**)&dcols, cols.size() * 4, st) ||
+        dmalloc((void**)&flags, 8, st) ||
         dmalloc((void**)&Pl->d_W, (size_t)N * 4, st) || dmalloc((void**)&Pl->d_cls, (size_t)N * 2, st)) {
         cleanup();
         return DWT_ENOMEM;
     }
-    std::vector<Map4> hm(2 * s);
-    for (int j = 0; j < s; ++j) {
-        hm[j] = Imap[j];
-        hm[s + j] = Qmap[j];
+    DWT_CK(cudaMemcpyAsync(dcols, cols.data(), cols.size() * 4, cudaMemcpyHostToDevice, st));
+    {
+        LaunchScope ls("tree_maps", st);
+        k_maps<<<(unsigned)(cols.size() / m), 256, 0, st>>>(dcols, m, dmaps);
     }
-    DWT_CK(cudaMemcpyAsync(dmaps, hm.data(), sizeof(Map4) * 2 * s, cudaMemcpyHostToDevice, st));
     DWT_CK(cudaMemsetAsync(flags, 0, 8, st));
     const size_t smem = 8192 + (size_t)4 * N + 2 * N + ((N + 15) & ~15ll) + 32 * 4;
     int rc = smem_limit_max(k_tree_one);
@@ -681,6 +901,45 @@ int tree_one(dwt_plan_s* Pl, const std::vector<Map4>& Imap, const std::vector<Ma
     return DWT_OK;
 }
 
+// the forward reading with as many labels per thread as keep the GPU full
+template <typename KT> void launch_fwd(const KT* K, const Map4* dmaps, unsigned* flags, dwt_plan_s* Pl, cudaStream_t st) {
+    const long long N = Pl->N;
+    LaunchScope ls("tree_read", st);
+    auto go = [&](auto kern, int L) {
+        kern<<<(unsigned)((N + 256ll * L - 1) / (256ll * L)), 256, 0, st>>>(K, dmaps, dmaps + 1, flags, Pl->d_W,
+                                                                            Pl->d_cls, N, Pl->s);
+    };
+    if (N <= (1 << 18)) go(k_tiles_fwd<1, KT>, 1);
+    else if (N <= (1 << 20)) go(k_tiles_fwd<2, KT>, 2);
+    else go(k_tiles_fwd<8, KT>, 8);
+}
+
+// the sweep of the cluster form and its readings
+cudaError_t launch_cluster(const CluArgs& A, cudaStream_t st) {
+    const int tpc = 1 << A.ltpc;
+    const unsigned ctas = (unsigned)(A.N >> (kTL + A.ltpc));   // a power of two
+    if (smem_limit_max(k_clu_bwd)) return cudaErrorInvalidValue;
+    const size_t smem = 8192 + (size_t)A.N + (size_t)tpc * (256 + 16) + 16;
+    {
+        LaunchScope ls("tree_sweep", st);
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(ctas);
+        cfg.blockDim = dim3(256u * (unsigned)tpc);
+        cfg.dynamicSmemBytes = smem;
+        cfg.stream = st;
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim = {ctas, 1, 1};
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+        const cudaError_t e = cudaLaunchKernelEx(&cfg, k_clu_bwd, A);
+        if (e != cudaSuccess) return e;
+    }
+    LaunchScope ls("tree_reps", st);
+    k_clu_read<<<dim3((unsigned)(A.N >> 8), (unsigned)A.s), 256, 0, st>>>(A);
+    return cudaGetLastError();
+}
+
 // Resident CTAs of the backward sweep on this GPU (0 if unknown).
 static long long tiles_resident(size_t smem) {
     int dev = 0, sms = 0, occ = 0;
@@ -695,16 +954,22 @@ static long long tiles_resident(size_t smem) {
 
 // The tiled form for 12 <= m <= 27 (one cooperative launch for the backward
 // sweep, one launch for the forward reading, one synchronisation).
-int tiles_build(dwt_plan_s* Pl, const Map4& I0, const std::vector<Map4>& Qmap, cudaStream_t st) {
+int tiles_build(dwt_plan_s* Pl, const std::vector<uint32_t>& cols, cudaStream_t st) {
     const long long N = Pl->N;
     const int m = Pl->m, s = Pl->s;
     const long long tiles = N >> kTL;
-    // one scratch block: flags (16 B, padded), the maps I_0, Q_0 .. Q_{s-2},
+    // one scratch block: flags (16 B, padded), the maps I_0, Q_0 .. Q_{s-2} (their columns first),
     // then T, the records, the block minima and K (256-byte aligned pieces)
+    // (the cluster form: leaves, minima and T_j, d of every coordinate)
+    const char* grid_env = getenv("DWT_TILE_GRID");
+    const bool cluster = m <= kCluMax && !grid_env;
     auto al = [](size_t x) { return (x + 255) & ~(size_t)255; };
-    const size_t o_maps = 256, o_T = al(o_maps + sizeof(Map4) * s), o_rec0 = al(o_T + (size_t)N),
-                 o_rec4 = al(o_rec0 + (size_t)N * 2), o_bmin = al(o_rec4 + (size_t)N / 8),
-                 o_K = al(o_bmin + (size_t)N / 256), total = al(o_K + (size_t)s * N * 4);
+    const size_t leaves = cluster ? (size_t)s * N : (size_t)N, per = cluster ? (size_t)s * N / 16 : (size_t)N * 2;
+    const size_t o_cols = 256, o_maps = al(o_cols + cols.size() * 4), o_T = al(o_maps + sizeof(Map4) * s),
+                 o_rec0 = al(o_T + leaves), o_rec4 = al(o_rec0 + per),
+                 o_bmin = al(o_rec4 + (cluster ? 0 : (size_t)N / 8)),
+                 o_K = al(o_bmin + (cluster ? (size_t)s * N / 256 : (size_t)N / 256)),
+                 total = al(o_K + (size_t)s * N * (cluster ? 2 : 4));
     unsigned char* ws = nullptr;
     auto cleanup = [&]() { dfree(ws, st); };
     int rc = DWT_OK;
@@ -726,69 +991,72 @@ int tiles_build(dwt_plan_s* Pl, const Map4& I0, const std::vector<Map4>& Qmap, c
     uint8_t* rec4 = ws + o_rec4;
     uint8_t* bmin = ws + o_bmin;
     uint32_t* K = reinterpret_cast<uint32_t*>(ws + o_K);
-    // flags zeroed and the maps in one upload, from page-locked staging when
-    // there is some (the stream is synchronised below, before it is reused)
-    const size_t nb = o_maps + sizeof(Map4) * s;
+    // flags zeroed and the maps' columns in one upload, from page-locked staging
+    // when there is some (the stream is synchronised below, before it is reused)
+    const size_t nb = o_cols + cols.size() * 4;
     std::vector<unsigned char> hv;
     unsigned char* hb = host_staging(nb);
     if (!hb) {
         hv.resize(nb);
         hb = hv.data();
     }
-    memset(hb, 0, o_maps);
-    memcpy(hb + o_maps, &I0, sizeof(Map4));
-    for (int j = 0; j + 1 < s; ++j) memcpy(hb + o_maps + sizeof(Map4) * (1 + j), &Qmap[j], sizeof(Map4));
+    memset(hb, 0, o_cols);
+    memcpy(hb + o_cols, cols.data(), cols.size() * 4);
     if ((rc = ck(cudaMemcpyAsync(ws, hb, nb, cudaMemcpyHostToDevice, st), "cudaMemcpyAsync"))) return rc;
-    const size_t smem = 4096 + kRecBytes + 8192 + 256 + 16 + (size_t)((2 * tiles + 15) & ~15ll);
-    rc = smem_limit_max(k_tiles_bwd);
-    if (rc) { cleanup(); return rc; }
-    // every resident CTA busy in the down pass: parts per tile (a power of two
-    // <= 16); the grid is capped by DWT_TILE_GRID if set (a tuning and testing
-    // knob: the tables do not depend on the grid or the parts)
-    const long long resident = tiles_resident(smem);
-    int parts = 1;
-    while (parts < 16 && tiles * parts * 2 <= resident) parts *= 2;
-    long long g = std::min(tiles * parts, resident);
     {
-        const char* e = getenv("DWT_TILE_GRID");
-        const long long cap = e ? atoll(e) : 0;
-        if (cap > 0) g = std::min(g, cap);
+        LaunchScope ls("tree_maps", st);
+        k_maps<<<(unsigned)s, 256, 0, st>>>(reinterpret_cast<const uint32_t*>(ws + o_cols), m, dmaps);
     }
-    if (g > 0) {
-        // as few CTAs as give the same number of rounds over the parts
-        const long long rounds = (tiles * parts + g - 1) / g;
-        g = (tiles * parts + rounds - 1) / rounds;
-    }
-    const int grid = (int)g;
-    if (grid < 1) {
-        cleanup();
-        set_error("no resident grid for the tiled coset-table sweep (%zu bytes of shared memory)", smem);
-        return DWT_ECUDA;
-    }
-    TileArgs A;
-    A.Q = dmaps + 1;
-    A.T = T;
-    A.K = K;
-    A.rec0 = rec0;
-    A.rec4 = rec4;
-    A.bmin = bmin;
-    A.flags = flags;
-    A.N = N;
-    A.m = m;
-    A.s = s;
-    {
-        LaunchScope ls("tree_sweep", st);
-        void* args[] = {&A, &parts};
-        if ((rc = ck(cudaLaunchCooperativeKernel((const void*)k_tiles_bwd, dim3((unsigned)grid), dim3(kTT), args, smem,
-                                                 st),
-                     "cooperative launch")))
-            return rc;
-    }
-    {
-        const long long per_cta = 256ll * kFwdL;
-        const unsigned fg = (unsigned)((N + per_cta - 1) / per_cta);
-        LaunchScope ls("tree_read", st);
-        k_tiles_fwd<<<fg, 256, 0, st>>>(K, dmaps, dmaps + 1, flags, Pl->d_W, Pl->d_cls, N, s);
+    if (cluster) {
+        const CluArgs A{dmaps + 1, T, rec0, bmin, reinterpret_cast<uint16_t*>(K), flags, N, m, s, std::max(0, m - kTL - 3)};
+        if ((rc = ck(launch_cluster(A, st), "cluster launch"))) return rc;
+        launch_fwd(reinterpret_cast<const uint16_t*>(K), dmaps, flags, Pl, st);
+    } else {
+        const size_t smem = 4096 + kRecBytes + 8192 + 256 + 16 + (size_t)((2 * tiles + 15) & ~15ll);
+        rc = smem_limit_max(k_tiles_bwd);
+        if (rc) { cleanup(); return rc; }
+        // every resident CTA busy in the down pass: parts per tile (a power of two
+        // <= 16); the grid is capped by DWT_TILE_GRID if set (a tuning and testing
+        // knob: the tables do not depend on the grid or the parts)
+        const long long resident = tiles_resident(smem);
+        int parts = 1;
+        while (parts < 16 && tiles * parts * 2 <= resident) parts *= 2;
+        long long g = std::min(tiles * parts, resident);
+        {
+            const long long cap = grid_env ? atoll(grid_env) : 0;
+            if (cap > 0) g = std::min(g, cap);
+        }
+        if (g > 0) {
+            // as few CTAs as give the same number of rounds over the parts
+            const long long rounds = (tiles * parts + g - 1) / g;
+            g = (tiles * parts + rounds - 1) / rounds;
+        }
+        const int grid = (int)g;
+        if (grid < 1) {
+            cleanup();
+            set_error("no resident grid for the tiled coset-table sweep (%zu bytes of shared memory)", smem);
+            return DWT_ECUDA;
+        }
+        TileArgs A;
+        A.Q = dmaps + 1;
+        A.T = T;
+        A.K = K;
+        A.rec0 = rec0;
+        A.rec4 = rec4;
+        A.bmin = bmin;
+        A.flags = flags;
+        A.N = N;
+        A.m = m;
+        A.s = s;
+        {
+            LaunchScope ls("tree_sweep", st);
+            void* args[] = {&A, &parts};
+            if ((rc = ck(cudaLaunchCooperativeKernel((const void*)k_tiles_bwd, dim3((unsigned)grid), dim3(kTT), args, smem,
+                                                     st),
+                         "cooperative launch")))
+                return rc;
+        }
+        launch_fwd(K, dmaps, flags, Pl, st);
     }
     if ((rc = ck(cudaGetLastError(), "tiled coset tables"))) return rc;
     unsigned hf[4] = {0, 0, 0, 0};
@@ -820,21 +1088,23 @@ int coset_tables_tree2(dwt_plan_s* Pl, cudaStream_t st, bool* used) {
     *used = false;
     if (Pl->p != 2 || m > 27 || m < 1) return DWT_OK;
     const std::vector<uint32_t>& R = Pl->R_host;
-    // maps: I_j (labels -> U_j) and Q_j (U_j -> U_{j+1})
-    std::vector<Map4> Imap(s), Qmap(s);
-    std::vector<uint32_t> inv(m);
-    for (int j = 0; j < s; ++j) {
-        if (!gf2_inverse(&R[(size_t)j * m], m, inv.data())) return DWT_OK;
-        make_map(inv.data(), m, Imap[j]);
-    }
-    for (int j = 0; j + 1 < s; ++j) {
-        std::vector<uint32_t> qc(m);
-        for (int i = 0; i < m; ++i) qc[i] = host_apply(Imap[j + 1], R[(size_t)j * m + i]);
-        make_map(qc.data(), m, Qmap[j]);
-    }
+    // columns of the maps I_j (labels -> U_j) and Q_j (U_j -> U_{j+1})
+    std::vector<uint32_t> I((size_t)s * m), Q((size_t)s * m);
+    for (int j = 0; j < s; ++j)
+        if (!gf2_inverse(&R[(size_t)j * m], m, &I[(size_t)j * m])) return DWT_OK;
+    for (int j = 0; j + 1 < s; ++j)
+        for (int i = 0; i < m; ++i)
+            Q[(size_t)j * m + i] = gf2_apply(&I[(size_t)(j + 1) * m], R[(size_t)j * m + i]);
     *used = true;
-    if (m < kTL) return tree_one(Pl, Imap, Qmap, st);
-    return tiles_build(Pl, Imap[0], Qmap, st);
+    std::vector<uint32_t> cols;
+    if (m < kTL) {
+        cols = I;
+        cols.insert(cols.end(), Q.begin(), Q.end());
+        return tree_one(Pl, cols, st);
+    }
+    cols.assign(I.begin(), I.begin() + m);   // I_0, then Q_0 .. Q_{s-2}
+    cols.insert(cols.end(), Q.begin(), Q.end() - m);
+    return tiles_build(Pl, cols, st);
 }
 
 }  // namespace dwt
