@@ -130,8 +130,11 @@ struct HiArgs {
     int nb;
 };
 
+// CTAs per SM: three of the plain pass (80 registers), but two where rows are 64
+// bytes (B = 10: m = 24, 32 functions 1462 us with two, 1538 us with three; B = 6:
+// m = 20 87 and 84 us; B = 9: m = 23 185 and 170 us).
 template <typename T, int LT, int B, bool FUSED, bool HAS_COEF>
-__global__ void __launch_bounds__(1 << (LT - 6), FUSED ? 4 : 1) k2_hi(HiArgs a) {
+__global__ void __launch_bounds__(1 << (LT - 6), FUSED ? 4 : B == 10 ? 2 : 3) k2_hi(HiArgs a) {
     static_assert(B >= 4 && B <= 10 && LT - B >= 2, "high-pass shape");
     using G = HiGeom<LT, B>;
     using V = typename P2<T>::t;
@@ -455,7 +458,12 @@ static int launch_hi_t(int B, const HiArgs& a, int nf, size_t bins_bytes, const 
     }
 }
 
-static const long long kL2GroupP2 = 48ll << 20;
+// Bytes of functions per group: the passes of a group run back to back so that
+// the intermediate stays in L2 between them.  p = 2, m = 20, 32 functions,
+// 48 / 64 / 80 / 96 MB: forward 97 / 90 / 97 / 100 us, int32 88 / 80 / 84 / 92,
+// interpolation 185 / 176 / 182 / 188; m = 24 (64 MB per function): the same up
+// to 112 MB, slower from two functions on.
+static const long long kL2GroupP2 = 64ll << 20;
 
 // forward (sgn < 0, scaled by 2^-m for FP32) or inverse transform, FP32 or int32
 template <typename T>
@@ -499,7 +507,6 @@ static int p2_transform_t(dwt_plan_s* Pl, const T* in, T* out, int batch, long l
 
 // only the FP32 high pass (digits L .. m-1) over data in place; forward scales by 2^-m
 int p2_hi_only(dwt_plan_s* Pl, float* data, int batch, long long ld, int L, int sgn, cudaStream_t st) {
-    if (L == 14 && p2i_transform_ok(Pl->m)) return p2i_hi_only(Pl, data, batch, ld, sgn, st);
     const int B = Pl->m - L;
     HiArgs a{};
     a.in = data;
@@ -524,8 +531,6 @@ int p2_hi_only(dwt_plan_s* Pl, float* data, int batch, long long ld, int L, int 
 
 int p2_transform(dwt_plan_s* Pl, const void* in, void* out, int batch, long long ld_in, long long ld_out,
                  dwt_dtype t, int sgn, cudaStream_t st) {
-    if (t == DWT_F32 && p2i_transform_ok(Pl->m))
-        return p2i_transform(Pl, (const float*)in, (float*)out, batch, ld_in, ld_out, sgn, st);
     if (t == DWT_F32)
         return p2_transform_t<float>(Pl, (const float*)in, (float*)out, batch, ld_in, ld_out, sgn, st);
     return p2_transform_t<int>(Pl, (const int*)in, (int*)out, batch, ld_in, ld_out, sgn, st);

@@ -191,8 +191,7 @@ __global__ void __launch_bounds__(Small<M>::NT) k2_small(SmallArgs a) {
                 for (int j = 0; j < 8; ++j) {
                     const int e = e0 + j * step;
                     const bool ok = e < N && e > 0;   // the label H = 0 is in no class
-                    const float x = ok ? sm[spos(e)] : 0.f;
-                    q[j] = x * x;
+                    q[j] = ok ? sm[spos(e)] : 0.f;
                     k[j] = ok ? scls[e] : 0u;
                 }
                 // two elements at a time: their bins are loaded together; if both
@@ -202,8 +201,10 @@ __global__ void __launch_bounds__(Small<M>::NT) k2_small(SmallArgs a) {
                     const int kt0 = (int)(k[j] & 255u), ks0 = (int)(k[j] >> 8);
                     const int kt1 = (int)(k[j + 1] & 255u), ks1 = (int)(k[j + 1] >> 8);
                     const float xt0 = bt[32 * kt0], xt1 = bt[32 * kt1], xs0 = bs[32 * ks0], xs1 = bs[32 * ks1];
-                    const float rt0 = xt0 + q[j], rs0 = xs0 + q[j];
-                    const float rt1 = (kt1 == kt0 ? rt0 : xt1) + q[j + 1], rs1 = (ks1 == ks0 ? rs0 : xs1) + q[j + 1];
+                    // (a bin grows by g^2 in one rounding, as in the generic pass)
+                    const float rt0 = __fmaf_rn(q[j], q[j], xt0), rs0 = __fmaf_rn(q[j], q[j], xs0);
+                    const float rt1 = __fmaf_rn(q[j + 1], q[j + 1], kt1 == kt0 ? rt0 : xt1);
+                    const float rs1 = __fmaf_rn(q[j + 1], q[j + 1], ks1 == ks0 ? rs0 : xs1);
                     bt[32 * kt0] = rt0;
                     bs[32 * ks0] = rs0;
                     bt[32 * kt1] = rt1;

@@ -416,6 +416,10 @@ struct MidArgs {
 template <typename T> __device__ __forceinline__ float mag2(T v);
 template <> __device__ __forceinline__ float mag2<float>(float v) { return v * v; }
 template <> __device__ __forceinline__ float mag2<float2>(float2 v) { return v.x * v.x + v.y * v.y; }
+// bin + |v|^2: one rounding for real v (a fused multiply-add)
+template <typename T> __device__ __forceinline__ float add_mag2(float bin, T v);
+template <> __device__ __forceinline__ float add_mag2<float>(float bin, float v) { return __fmaf_rn(v, v, bin); }
+template <> __device__ __forceinline__ float add_mag2<float2>(float bin, float2 v) { return bin + mag2<float2>(v); }
 template <typename T> __device__ __forceinline__ T mulw(T v, float w);
 template <> __device__ __forceinline__ float mulw<float>(float v, float w) { return v * w; }
 template <> __device__ __forceinline__ float2 mulw<float2>(float2 v, float w) { return make_float2(v.x * w, v.y * w); }
@@ -505,23 +509,23 @@ __global__ void __maxnreg__(96) k_mid(MidArgs m, int nwb, const __grid_constant_
             }
 #pragma unroll
             for (int j = 0; j < 8; j += 2) {
-                float q[2];
+                T q[2];
 #pragma unroll
                 for (int u = 0; u < 2; ++u) {
-                    q[u] = 0.f;   // the label H = 0 is in no class
+                    q[u] = zero_of<T>();   // the label H = 0 is in no class
                     if (ok[j + u]) {
                         T& x = sm[sx<P, T>(e0 + (j + u) * step)];
                         const T v = mulw<T>(scale_of<T>(a, x), wv[j + u]);
                         x = v;
                         if (coef) coef[H[j + u]] = v;
-                        if (H[j + u] != 0) q[u] = mag2<T>(v);
+                        if (H[j + u] != 0) q[u] = v;
                     }
                 }
                 const int kt0 = (int)(kc[j] & 255u), ks0 = (int)(kc[j] >> 8);
                 const int kt1 = (int)(kc[j + 1] & 255u), ks1 = (int)(kc[j + 1] >> 8);
                 const float xt0 = bt[32 * kt0], xt1 = bt[32 * kt1], xs0 = bs[32 * ks0], xs1 = bs[32 * ks1];
-                const float rt0 = xt0 + q[0], rs0 = xs0 + q[0];
-                const float rt1 = (kt1 == kt0 ? rt0 : xt1) + q[1], rs1 = (ks1 == ks0 ? rs0 : xs1) + q[1];
+                const float rt0 = add_mag2<T>(xt0, q[0]), rs0 = add_mag2<T>(xs0, q[0]);
+                const float rt1 = add_mag2<T>(kt1 == kt0 ? rt0 : xt1, q[1]), rs1 = add_mag2<T>(ks1 == ks0 ? rs0 : xs1, q[1]);
                 bt[32 * kt0] = rt0;
                 bs[32 * ks0] = rs0;
                 bt[32 * kt1] = rt1;
