@@ -165,7 +165,7 @@ __global__ void __launch_bounds__(Small<M>::NT) k2_small(SmallArgs a) {
     if (a.nwb) {
         for (int i = t; i < N / 8; i += NT)
             reinterpret_cast<uint4*>(scls)[i] = __ldg(reinterpret_cast<const uint4*>(a.cls) + i);
-        for (int i = t; i < a.nwb * nb2 * 32; i += NT) bins[i] = 0.f;
+        for (int i = t; i < a.nwb * nb2 * 8; i += NT) reinterpret_cast<float4*>(bins)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
     }
     forward<M, 0>(sm, v, t);
     // scale (a power of two), weight; the tile keeps g for the class sums
@@ -213,12 +213,24 @@ __global__ void __launch_bounds__(Small<M>::NT) k2_small(SmallArgs a) {
             }
         }
         __syncthreads();
-        for (int b = t >> 5; b < nb2; b += NT / 32) {
-            float x = 0.f;
-            for (int ww = 0; ww < a.nwb; ++ww) x += bins[(ww * nb2 + b) * 32 + (t & 31)];
+        // four classes at a time: their trees overlap
+        for (int b0 = 4 * (t >> 5); b0 < nb2; b0 += 4 * (NT / 32)) {
+            float x[4] = {0.f, 0.f, 0.f, 0.f};
+            for (int ww = 0; ww < a.nwb; ++ww) {
 #pragma unroll
-            for (int h = 16; h > 0; h >>= 1) x += __shfl_xor_sync(0xffffffffu, x, h);
-            if ((t & 31) == 0) tot[b] = (double)x;
+                for (int k = 0; k < 4; ++k)
+                    if (b0 + k < nb2) x[k] += bins[(ww * nb2 + b0 + k) * 32 + (t & 31)];
+            }
+#pragma unroll
+            for (int h = 16; h > 0; h >>= 1) {
+#pragma unroll
+                for (int k = 0; k < 4; ++k) x[k] += __shfl_xor_sync(0xffffffffu, x[k], h);
+            }
+            if ((t & 31) == 0) {
+#pragma unroll
+                for (int k = 0; k < 4; ++k)
+                    if (b0 + k < nb2) tot[b0 + k] = (double)x[k];
+            }
         }
     } else {
         stages<M, LAST>(v);

@@ -21,8 +21,8 @@
 // Tables are kept in the coordinates of their own coordinate's basis (T^U_j);
 // consecutive coordinates are linked by the F_2-linear map U_j -> U_{j+1}.
 // Linear maps are applied as four 256-entry XOR tables (one per byte).  Nets
-// of up to 2^11 labels run in one CTA; larger ones in tiles of 2^12 labels
-// (the tiled form below).  Nets whose row sets are dependent, and m > 27, use
+// of up to 2^11 labels run in one CTA, of 2^12 .. 2^16 in one cluster (the
+// cluster form below), larger ones in tiles of 2^12 labels (the tiled form).  Nets whose row sets are dependent, and m > 27, use
 // the per-digit programme.
 #include <stdlib.h>
 #include <string.h>
