@@ -37,7 +37,7 @@ template <typename T> struct LoJob {
     int nf;
     float scale;
     int do_scale;
-    int stream_out;   // store with evict-first (final results)
+    int last;         // final results: stored with evict-first; else kept in L2 for the next pass
 };
 
 // Tiles [0, tiles0) belong to job 0, the rest to job 1: two independent low
@@ -45,7 +45,7 @@ template <typename T> struct LoJob {
 // the next), which keeps the memory system busy while either one computes.
 // the low pass of one tile of 2^L elements, src -> dst
 template <typename T, int L>
-__device__ __forceinline__ void lo_body(const T* src, T* dst, float scale, int do_scale, bool stream_out) {
+__device__ __forceinline__ void lo_body(const T* src, T* dst, float scale, int do_scale, bool last) {
     using V = typename P2<T>::t;
     constexpr int NT = 1 << (L - 6);
     extern __shared__ __align__(16) unsigned char smraw[];
@@ -60,7 +60,7 @@ __device__ __forceinline__ void lo_body(const T* src, T* dst, float scale, int d
 #pragma unroll
         for (int k = 0; k < 32; ++k) v[k] = pmul(v[k], scale);
     }
-    lo_tile_store<T, L>(dst, v, t, stream_out);
+    lo_tile_store<T, L>(dst, v, t, last);
 }
 
 template <typename T, int L>
@@ -74,7 +74,7 @@ __global__ void __launch_bounds__(1 << (L - 6), (L == 14 ? 3 : 4))
     const T* src = (second ? j1.in : j0.in) + blockIdx.y * (second ? j1.ld_in : j0.ld_in) + (tile << L);
     T* dst = (second ? j1.out : j0.out) + blockIdx.y * (second ? j1.ld_out : j0.ld_out) + (tile << L);
     lo_body<T, L>(src, dst, second ? j1.scale : j0.scale, second ? j1.do_scale : j0.do_scale,
-                  (second ? j1.stream_out : j0.stream_out) != 0);
+                  (second ? j1.last : j0.last) != 0);
 }
 
 // Whole transforms of 2^L points (one tile per function) of several plans in
@@ -108,7 +108,7 @@ __global__ void __launch_bounds__(1 << (L - 6), (L == 14 ? 3 : 4))
     }
     const LoJob<T> j = jobs[lo].j;
     const long long fn = b - jobs[lo].first;
-    lo_body<T, L>(j.in + fn * j.ld_in, j.out + fn * j.ld_out, j.scale, j.do_scale, j.stream_out != 0);
+    lo_body<T, L>(j.in + fn * j.ld_in, j.out + fn * j.ld_out, j.scale, j.do_scale, j.last != 0);
 }
 
 // ---------------------------------------------------------------------------
@@ -149,8 +149,10 @@ __global__ void __launch_bounds__(1 << (LT - 6), FUSED ? 4 : B == 10 ? 2 : 3) k2
     T* dst = reinterpret_cast<T*>(a.out) + fn * a.ld_out + base;
     V v[32];
     // layout A loads
+    // the plain pass reads the intermediate and writes final results (evict first)
+    const uint64_t pol = FUSED ? policy_evict_last() : policy_evict_first();
 #pragma unroll
-    for (int q = 0; q < 16; ++q) ld16(src + G::goff(4 * (t + NT * q), a.S), v + 2 * q);
+    for (int q = 0; q < 16; ++q) ld16_hint(src + G::goff(4 * (t + NT * q), a.S), v + 2 * q, pol);
     if constexpr (FUSED) {
         // this tile's weights (4 B per element) and classes (2 B) are contiguous
         // in the tile-major tables: start moving them from HBM into L2 now, to be
@@ -183,10 +185,10 @@ __global__ void __launch_bounds__(1 << (LT - 6), FUSED ? 4 : B == 10 ? 2 : 3) k2
         }
         if constexpr (B > 4) {
 #pragma unroll
-            for (int j = 0; j < 64; ++j) dst[G::goff(ep | (j << P1), a.S)] = comp(v[j >> 1], j & 1);
+            for (int j = 0; j < 64; ++j) st_hint(dst + G::goff(ep | (j << P1), a.S), comp(v[j >> 1], j & 1), pol);
         } else {
 #pragma unroll
-            for (int q = 0; q < 16; ++q) st16(dst + G::goff(4 * (t + NT * q), a.S), v + 2 * q);
+            for (int q = 0; q < 16; ++q) st16_hint(dst + G::goff(4 * (t + NT * q), a.S), v + 2 * q, pol);
         }
     } else {
         // The class bins alias the exchange buffer: wait until every thread has
@@ -288,7 +290,7 @@ __global__ void __launch_bounds__(1 << (LT - 6), FUSED ? 4 : B == 10 ? 2 : 3) k2
         }
         bfly_range<2, 6>(v);
 #pragma unroll
-        for (int q = 0; q < 16; ++q) st16(dst + G::goff(4 * (t + NT * q), a.S), v + 2 * q);
+        for (int q = 0; q < 16; ++q) st16_hint(dst + G::goff(4 * (t + NT * q), a.S), v + 2 * q, pol);
     }
 }
 
@@ -370,7 +372,7 @@ static int lo_grouped_t(int L, const std::vector<GroupJob>& jobs, int sgn, cudaS
     for (const GroupJob& g : jobs) {
         const long long N = g.plan->N;
         LoGroup<T> x;
-        x.j = LoJob<T>{(const T*)g.in, (T*)g.out, g.ld_in, g.ld_out, g.batch, (float)(1.0 / (double)N), scale ? 1 : 0, 0};
+        x.j = LoJob<T>{(const T*)g.in, (T*)g.out, g.ld_in, g.ld_out, g.batch, (float)(1.0 / (double)N), scale ? 1 : 0, 1};
         x.first = blocks;
         blocks += g.batch;
         h.push_back(x);
@@ -421,7 +423,7 @@ int p2_lo_grouped(int L, const std::vector<GroupJob>& jobs, dwt_dtype t, int sgn
 template <typename T>
 static int launch_lo(int L, const T* in, T* out, long long ld_in, long long ld_out, int nf, long long N, float scale,
                      int do_scale, const char* fam, cudaStream_t st) {
-    LoJob<T> a{in, out, ld_in, ld_out, nf, scale, do_scale, 0};
+    LoJob<T> a{in, out, ld_in, ld_out, nf, scale, do_scale, L < 63 && N == (1ll << L) ? 1 : 0};
     return launch_lo2<T>(L, a, nullptr, N, fam, st);
 }
 

@@ -75,6 +75,39 @@ __device__ __forceinline__ void st16(T* p, const V* v2) {
     *reinterpret_cast<typename P2<T>::v4*>(p) = x;
 }
 
+// the same with an L2 eviction priority
+__device__ __forceinline__ uint64_t policy_evict_last() {
+    uint64_t p;
+    asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(p));
+    return p;
+}
+__device__ __forceinline__ uint64_t policy_evict_first() {
+    uint64_t p;
+    asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(p));
+    return p;
+}
+template <typename T, typename V>
+__device__ __forceinline__ void ld16_hint(const T* p, V* v2, uint64_t pol) {
+    int4 x;
+    asm volatile("ld.global.L2::cache_hint.v4.b32 {%0, %1, %2, %3}, [%4], %5;"
+                 : "=r"(x.x), "=r"(x.y), "=r"(x.z), "=r"(x.w)
+                 : "l"(p), "l"(pol));
+    memcpy(v2, &x, 16);
+}
+template <typename T, typename V>
+__device__ __forceinline__ void st16_hint(T* p, const V* v2, uint64_t pol) {
+    int4 x;
+    memcpy(&x, v2, 16);
+    asm volatile("st.global.L2::cache_hint.v4.b32 [%0], {%1, %2, %3, %4}, %5;" ::"l"(p), "r"(x.x), "r"(x.y), "r"(x.z),
+                 "r"(x.w), "l"(pol)
+                 : "memory");
+}
+template <typename T> __device__ __forceinline__ void st_hint(T* p, T v, uint64_t pol) {
+    int x;
+    memcpy(&x, &v, 4);
+    asm volatile("st.global.L2::cache_hint.b32 [%0], %1, %2;" ::"l"(p), "r"(x), "l"(pol) : "memory");
+}
+
 // bulk prefetch of [p, p + bytes) from global memory into L2 (bytes a multiple of 16)
 __device__ __forceinline__ void prefetch_l2(const void* p, unsigned bytes) {
     asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
@@ -121,20 +154,13 @@ __device__ __forceinline__ void lo_tile_compute(T* sm, typename P2<T>::t* v, int
     (void)sizeof(V);
 }
 
+// last: final results (evict first from L2), else read again by the next pass (kept)
 template <typename T, int L>
-__device__ __forceinline__ void lo_tile_store(T* dst, const typename P2<T>::t* v, int t, bool stream_out) {
+__device__ __forceinline__ void lo_tile_store(T* dst, const typename P2<T>::t* v, int t, bool last) {
     T* pd = dst + 4 * (t & 15) + 1024 * (t >> 4);
-    if (stream_out) {   // final output: evict first from L2
+    const uint64_t pol = last ? policy_evict_first() : policy_evict_last();
 #pragma unroll
-        for (int g = 0; g < 16; ++g) {
-            typename P2<T>::v4 x;
-            x.x = v[2 * g].x; x.y = v[2 * g].y; x.z = v[2 * g + 1].x; x.w = v[2 * g + 1].y;
-            __stcs(reinterpret_cast<typename P2<T>::v4*>(pd + 64 * g), x);
-        }
-    } else {
-#pragma unroll
-        for (int g = 0; g < 16; ++g) st16(pd + 64 * g, v + 2 * g);
-    }
+    for (int g = 0; g < 16; ++g) st16_hint(pd + 64 * g, v + 2 * g, pol);
 }
 
 template <int LT, int B> struct HiGeom {

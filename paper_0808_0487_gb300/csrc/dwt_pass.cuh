@@ -173,6 +173,56 @@ template <int P, int NK, int SGN, typename T> struct RegStages<P, NK, NK, SGN, T
     static __device__ __forceinline__ void run(T*, const Tw&) {}
 };
 
+// loads and stores with an L2 eviction priority: the first pass reads its input
+// for the last time and the last pass writes final results (evict first), so
+// that the intermediate of the passes between stays in L2
+__device__ __forceinline__ uint64_t l2_policy(int first) {
+    uint64_t p;
+    if (first) asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(p));
+    else asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(p));
+    return p;
+}
+__device__ __forceinline__ float ld_l2(const float* a, uint64_t p) {
+    float v;
+    asm volatile("ld.global.L2::cache_hint.f32 %0, [%1], %2;" : "=f"(v) : "l"(a), "l"(p));
+    return v;
+}
+__device__ __forceinline__ int ld_l2(const int* a, uint64_t p) {
+    int v;
+    asm volatile("ld.global.L2::cache_hint.s32 %0, [%1], %2;" : "=r"(v) : "l"(a), "l"(p));
+    return v;
+}
+__device__ __forceinline__ double ld_l2(const double* a, uint64_t p) {
+    double v;
+    asm volatile("ld.global.L2::cache_hint.f64 %0, [%1], %2;" : "=d"(v) : "l"(a), "l"(p));
+    return v;
+}
+__device__ __forceinline__ float2 ld_l2(const float2* a, uint64_t p) {
+    float2 v;
+    asm volatile("ld.global.L2::cache_hint.v2.f32 {%0, %1}, [%2], %3;" : "=f"(v.x), "=f"(v.y) : "l"(a), "l"(p));
+    return v;
+}
+__device__ __forceinline__ double2 ld_l2(const double2* a, uint64_t p) {
+    double2 v;
+    asm volatile("ld.global.L2::cache_hint.v2.f64 {%0, %1}, [%2], %3;" : "=d"(v.x), "=d"(v.y) : "l"(a), "l"(p));
+    return v;
+}
+__device__ __forceinline__ void st_l2(float* a, float v, uint64_t p) {
+    asm volatile("st.global.L2::cache_hint.f32 [%0], %1, %2;" ::"l"(a), "f"(v), "l"(p) : "memory");
+}
+__device__ __forceinline__ void st_l2(int* a, int v, uint64_t p) {
+    asm volatile("st.global.L2::cache_hint.s32 [%0], %1, %2;" ::"l"(a), "r"(v), "l"(p) : "memory");
+}
+__device__ __forceinline__ void st_l2(double* a, double v, uint64_t p) {
+    asm volatile("st.global.L2::cache_hint.f64 [%0], %1, %2;" ::"l"(a), "d"(v), "l"(p) : "memory");
+}
+__device__ __forceinline__ void st_l2(float2* a, float2 v, uint64_t p) {
+    asm volatile("st.global.L2::cache_hint.v2.f32 [%0], {%1, %2}, %3;" ::"l"(a), "f"(v.x), "f"(v.y), "l"(p) : "memory");
+}
+__device__ __forceinline__ void st_l2(double2* a, double2 v, uint64_t p) {
+    asm volatile("st.global.L2::cache_hint.v2.f64 [%0], {%1, %2}, %3;" ::"l"(a), "d"(v.x), "d"(v.y), "l"(p) : "memory");
+}
+
 // digits per register group: p^K elements per thread (27 complex FP32 at p = 3)
 template <int P, typename T> struct KMax {
     static constexpr int v = P == 2 ? (sizeof(T) == 8 ? 4 : 5)
@@ -200,6 +250,7 @@ struct PassArgs {
     float scalef;
     int do_scale;
     int direct_out;          // the last group writes global memory
+    int in_first, out_first; // input read, output written for the last time
     PassGroup g[kMaxGroups];
 };
 
@@ -248,9 +299,10 @@ __device__ __forceinline__ void rgroup(T* sm, const TI* gin, T* gout, const Pass
         T v[NK];
         if constexpr (SRC_G) {
             const TI* src = gin + (c + a.S * (long long)r0);
+            const uint64_t pol = l2_policy(a.in_first);
 #pragma unroll
             for (int i = 0; i < NK; ++i) {
-                v[i] = live ? promote<T, TI>(*src) : zero_of<T>();
+                v[i] = live ? promote<T, TI>(ld_l2(src, pol)) : zero_of<T>();
                 src += gstep;
             }
         } else {
@@ -269,9 +321,10 @@ __device__ __forceinline__ void rgroup(T* sm, const TI* gin, T* gout, const Pass
             }
             if (live) {
                 T* dst = gout + (c + a.S * (long long)r0);
+                const uint64_t pol = l2_policy(a.out_first);
 #pragma unroll
                 for (int i = 0; i < NK; ++i) {
-                    *dst = v[i];
+                    st_l2(dst, v[i], pol);
                     dst += gstep;
                 }
             }
@@ -589,6 +642,7 @@ static PassArgs pass_args(int p, int km, int elem, const PassGeom& g, const void
     a.scale = 1.0;
     a.scalef = 1.f;
     a.do_scale = 0;
+    a.in_first = a.out_first = 0;
     const int k0 = std::min(km, g.b);
     int g0 = g.b - k0, k = k0, g_last = 0;
     for (int i = 0; i < kMaxGroups; ++i) {
@@ -651,12 +705,13 @@ static int launch_pass(const PassGeom& g, const PassArgs& a, const Tw& tw, int n
 }
 
 // L2-sized groups of functions: the passes of one group run back to back so
-// that the intermediate stays in the 126 MB L2 between passes.  Groups of a
-// batch are equally large, so that none ends with launches of few blocks
-// (p = 3, m = 13: interpolation of 4 functions in groups of 3 + 1 100 us, of 4
-// 88 us; forward of 32: 48 MB 299 us, 64 MB 277 us, 96 MB 275 us; p = 5, m = 9,
-// 32 functions: 394, 394 and 406 us).
-static const long long kL2Group = 64ll << 20;
+// that the intermediate stays in the 126 MB L2 between passes (kept there by the
+// eviction priorities of the first and last pass).  Groups of a batch are
+// equally large, so that none ends with launches of few blocks.  48 / 64 / 96 /
+// 128 MB: p = 5, m = 9, 32 forward transforms 403 / 385 / 374 / 384 us; p = 3,
+// m = 13, 32 299 / 272 / 257 / 253; m = 14, 16 494 / 494 / 430 / 435; p = 7,
+// m = 7, 32 215 / 208 / 204 / 203.
+static const long long kL2Group = 96ll << 20;
 
 static int functions_per_group(long long bytes, long long fbytes, int batch) {
     const long long g = std::min(65535ll, std::max(1ll, bytes / fbytes));
@@ -693,11 +748,14 @@ static int transform_pp(dwt_plan_s* Pl, const PassPlan& pp, double scale_by_n, c
                 PassArgs a = pass_args(P, KMax<P, T>::v, (int)sizeof(T), g, (const TI*)in + (long long)f0 * ld_in, (T*)out + (long long)f0 * ld_out,
                                        ld_in, ld_out);
                 if (scale && pp.q == 1) pass_scale(a, scale_by_n);
+                a.in_first = 1;
+                a.out_first = pp.q == 1;
                 rc = launch_pass<P, T, TI, SGN>(g, a, tw, nf, pass_family(t, pp.q), st);
             } else {
                 PassArgs a = pass_args(P, KMax<P, T>::v, (int)sizeof(T), g, (const T*)out + (long long)f0 * ld_out, (T*)out + (long long)f0 * ld_out,
                                        ld_out, ld_out);
                 if (scale && t == pp.q - 1) pass_scale(a, scale_by_n);
+                a.in_first = a.out_first = t == pp.q - 1;
                 rc = launch_pass<P, T, T, SGN>(g, a, tw, nf, pass_family(t, pp.q), st);
             }
             if (rc) return rc;
@@ -909,6 +967,7 @@ static int interpolate_t(dwt_plan_s* Pl, const void* f, void* c, void* coef, int
             const PassGeom& g = pp.g[t];
             if (t == 0) {
                 PassArgs a = pass_args(P, KMax<P, T>::v, (int)sizeof(T), g, (const TI*)f + off, (T*)c + off, ld, ld);
+                a.in_first = 1;
                 rc = launch_pass<P, T, TI, -1>(g, a, tw, nf, "interp_fwd", st);
             } else {
                 PassArgs a = pass_args(P, KMax<P, T>::v, (int)sizeof(T), g, (const T*)c + off, (T*)c + off, ld, ld);
@@ -939,6 +998,7 @@ static int interpolate_t(dwt_plan_s* Pl, const void* f, void* c, void* coef, int
         for (int t = pp.q - 2; t >= 0; --t) {
             const PassGeom& g = pp.g[t];
             PassArgs a = pass_args(P, KMax<P, T>::v, (int)sizeof(T), g, (const T*)c + off, (T*)c + off, ld, ld);
+            a.in_first = a.out_first = t == 0;
             rc = launch_pass<P, T, T, +1>(g, a, tw, nf, "interp_inv", st);
             if (rc) return rc;
         }

@@ -264,7 +264,7 @@ int tune_passes(dwt_plan_s* P, long long min_tiles, cudaStream_t st) {
             long long best_g = 0;
             float gbest = -1.f;
             int last_G = -1;
-            for (long long mb : {64ll, 16ll, 128ll, 1024ll}) {
+            for (long long mb : {96ll, 16ll, 64ll, 1024ll}) {
                 const long long bytes = mb << 20;
                 const int G = (int)std::max(1ll, bytes / fbytes);
                 if (G == last_G || (G >= nbatch && last_G >= nbatch)) continue;
@@ -279,7 +279,7 @@ int tune_passes(dwt_plan_s* P, long long min_tiles, cudaStream_t st) {
                 }
             }
             P->tuned_group_bytes = 0;
-            if (!rc && best_g != (64ll << 20)) ts.group = best_g;
+            if (!rc && best_g != (96ll << 20)) ts.group = best_g;
         }
     }
     if (!rc && p == 2 && m >= 16 && m <= 19) {
