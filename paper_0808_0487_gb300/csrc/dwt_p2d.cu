@@ -73,23 +73,18 @@ __device__ __forceinline__ W96 negate_if(W96 v, uint32_t mask) {
 
 __device__ __forceinline__ int exponent_of(uint32_t hi) { return (int)((hi >> 20) & 0x7ffu); }
 
-// significand of a double at 2^g below the largest exponent E (>= 1) of its group
-__device__ __forceinline__ W96 to_fixed(uint32_t hi, uint32_t lo, int E, int g) {
+constexpr int kG = 30;   // bits below the largest element's last place: 2^12 sums of 53 + 30 bits fit 95
+
+// fixed point of a double against the largest exponent E (>= 1) of its group
+__device__ __forceinline__ W96 to_fixed_any(uint32_t hi, uint32_t lo, int E) {
     const int ex = exponent_of(hi);
     uint32_t mh = hi & 0xfffffu;
     if (ex) mh |= 0x100000u;
     const int d = min(E - max(ex, 1), 95);
-    // significand << g, g = 30 .. 38: up to 91 bits; right by d in two steps
-    W96 v;
-    if (g >= 32) {
-        v.a = 0;
-        v.b = lo << (g - 32);
-        v.c = __funnelshift_l(lo, mh, g - 32);
-    } else {
-        v.a = lo << g;
-        v.b = __funnelshift_l(lo, mh, g);
-        v.c = mh >> (32 - g);
-    }
+    W96 v;   // significand << 30, then right by d
+    v.a = lo << kG;
+    v.b = __funnelshift_l(lo, mh, kG);
+    v.c = mh >> (32 - kG);
     if (d >= 64) {
         v.a = v.c;
         v.b = v.c = 0;
@@ -105,11 +100,36 @@ __device__ __forceinline__ W96 to_fixed(uint32_t hi, uint32_t lo, int E, int g) 
     return negate_if(v, (uint32_t)((int)hi >> 31));
 }
 
-// fixed point -> nearest double (ties to even), times 2^shift
-__device__ __forceinline__ double from_fixed(W96 v, int E, int g, int shift) {
-    const uint32_t sign = (uint32_t)((int)v.c >> 31);
-    v = negate_if(v, sign);
-    int e = 95 + E - 52 - g + shift;   // exponent field of bit 95
+// the same for a normal double within 2^30 of E: one shift of the signed significand
+__device__ __forceinline__ W96 to_fixed_near(uint32_t hi, uint32_t lo, int sh) {   // sh = 30 - E
+    const uint32_t sign = (uint32_t)((int)hi >> 31);
+    const int s = exponent_of(hi) + sh;
+    uint32_t ml, mh;
+    asm("sub.cc.u32 %0, %2, %4;\n subc.u32 %1, %3, %4;"
+        : "=r"(ml), "=r"(mh)
+        : "r"(lo ^ sign), "r"(((hi & 0xfffffu) | 0x100000u) ^ sign), "r"(sign));
+    W96 v;
+    v.a = ml << s;
+    v.b = __funnelshift_l(ml, mh, s);
+    v.c = __funnelshift_l(mh, sign, s);
+    return v;
+}
+
+// the bits of a nonnegative v, normalised to bit 31 of h (lz places up), rounded
+// to 53 (ties to even), with exponent field e of its top bit
+__device__ __forceinline__ double round53(uint32_t h, uint32_t l, uint32_t rest, int e, uint32_t sign) {
+    const uint32_t uh = h >> 11, ul = __funnelshift_r(l, h, 11);
+    const uint32_t rem = (l & 0x7ffu) | (rest ? 1u : 0u);
+    const uint32_t up = rem + (ul & 1u) > 0x400u ? 1u : 0u;
+    uint32_t rl, rh;   // the implicit bit adds one to the exponent field
+    asm("add.cc.u32 %0, %2, %3;\n addc.u32 %1, %4, %5;"
+        : "=r"(rl), "=r"(rh)
+        : "r"(ul), "r"(up), "r"(uh), "r"((uint32_t)(e - 1) << 20));
+    return __hiloint2double((int)(rh | (sign & 0x80000000u)), (int)rl);
+}
+
+// fixed point of any size -> nearest double; top = exponent field of bit 95
+__device__ __noinline__ double from_fixed_any(W96 v, uint32_t sign, int e) {   // v = |value|
     if (v.c == 0) {
         v.c = v.b;
         v.b = v.a;
@@ -124,26 +144,22 @@ __device__ __forceinline__ double from_fixed(W96 v, int E, int g, int shift) {
     const int lz = __clz((int)v.c);   // 32 when the value is zero
     if (lz == 32) return 0.0;
     e -= lz;
-    v.c = __funnelshift_l(v.b, v.c, lz);
-    v.b = __funnelshift_l(v.a, v.b, lz);
-    v.a <<= lz;
-    // 53 bits of c:b, the rest rounds
-    uint32_t uh = v.c >> 11, ul = __funnelshift_r(v.b, v.c, 11);
-    const uint32_t rem = (v.b & 0x7ffu) | (v.a ? 1u : 0u);
-    const uint32_t up = rem + (ul & 1u) > 0x400u ? 1u : 0u;
-    const bool tiny = e < 1, huge = e >= 0x7ff;
-    const int ef = tiny ? e + 128 : e;   // the implicit bit adds one to the field
-    uint32_t rl, rh;
-    asm("add.cc.u32 %0, %2, %3;\n addc.u32 %1, %4, %5;"
-        : "=r"(rl), "=r"(rh)
-        : "r"(ul), "r"(up), "r"(uh), "r"((uint32_t)(ef - 1) << 20));
-    if (huge) {
-        rh = 0x7ff00000u;
-        rl = 0;
-    }
-    double x = __hiloint2double((int)(rh | (sign & 0x80000000u)), (int)rl);
-    if (tiny) x = ef < 1 ? 0.0 : x * 0x1p-128;
-    return x;
+    const uint32_t h = __funnelshift_l(v.b, v.c, lz), l = __funnelshift_l(v.a, v.b, lz), rest = v.a << lz;
+    if (e >= 0x7ff) return __hiloint2double((int)(0x7ff00000u | (sign & 0x80000000u)), 0);
+    if (e >= 1) return round53(h, l, rest, e, sign);
+    return e + 128 < 1 ? 0.0 : round53(h, l, rest, e + 128, sign) * 0x1p-128;   // below the normal range
+}
+
+// fixed point -> nearest double (ties to even); top = the exponent field of bit
+// 95.  All lanes of the warp call it: results in the top word's range and of
+// normal size take the short way, a warp with any other takes the long one.
+__device__ __forceinline__ double from_fixed(W96 v, int top) {
+    const uint32_t sign = (uint32_t)((int)v.c >> 31);
+    v = negate_if(v, sign);
+    const int lz = __clz((int)v.c), e = top - lz;
+    const bool odd = v.c == 0 || (unsigned)(e - 1) >= 0x7feu;
+    if (__any_sync(0xffffffffu, odd)) return from_fixed_any(v, sign, top);
+    return round53(__funnelshift_l(v.b, v.c, lz), __funnelshift_l(v.a, v.b, lz), v.a << lz, e, sign);
 }
 
 // stages of register bits LO .. 3
@@ -184,7 +200,6 @@ template <int (*EL)(int, int)> __device__ __forceinline__ void get(const uint32_
 template <int B>
 __global__ void __launch_bounds__(kNT, 3) k2d_pass(DArgs a) {
     constexpr int LC = kLT - B;          // column bits
-    constexpr int G = 42 - B;            // bits below the largest element's last place
     extern __shared__ __align__(16) unsigned char smraw[];
     uint32_t* plane = reinterpret_cast<uint32_t*>(smraw);
     int* emax = reinterpret_cast<int*>(plane + 3 * kPlane);   // per column
@@ -214,9 +229,13 @@ __global__ void __launch_bounds__(kNT, 3) k2d_pass(DArgs a) {
 #pragma unroll
         for (int r = 0; r < 16; ++r) dst[off(e_a(t, r))] = a.exp_shift ? x[r] * sc : x[r];
     } else {
-        int mx = 1;
+        int mx = 1, mn = 0x7ff;
 #pragma unroll
-        for (int r = 0; r < 16; ++r) mx = max(mx, exponent_of((uint32_t)__double2hiint(x[r])));
+        for (int r = 0; r < 16; ++r) {
+            const int ex = exponent_of((uint32_t)__double2hiint(x[r]));
+            mx = max(mx, ex);
+            mn = min(mn, ex);
+        }
         if (t < (1 << LC)) emax[t] = 1;
         if (__syncthreads_or(mx == 0x7ff)) {
             // an infinity or a NaN: FP64 stages through shared memory
@@ -245,17 +264,21 @@ __global__ void __launch_bounds__(kNT, 3) k2d_pass(DArgs a) {
         }
         __syncthreads();
         W96 v[16];
-        {
-            const int E = emax[t & ((1 << LC) - 1)];
+        const int E = emax[t & ((1 << LC) - 1)];
+        if (__all_sync(0xffffffffu, mn >= max(1, E - kG))) {
 #pragma unroll
             for (int r = 0; r < 16; ++r)
-                v[r] = to_fixed((uint32_t)__double2hiint(x[r]), (uint32_t)__double2loint(x[r]), E, G);
+                v[r] = to_fixed_near((uint32_t)__double2hiint(x[r]), (uint32_t)__double2loint(x[r]), kG - E);
+        } else {
+#pragma unroll
+            for (int r = 0; r < 16; ++r)
+                v[r] = to_fixed_any((uint32_t)__double2hiint(x[r]), (uint32_t)__double2loint(x[r]), E);
         }
+        const int top = 95 - 52 - kG + a.exp_shift;   // + E: exponent field of bit 95
         stages<0>(v);
         if constexpr (B == 4) {
-            const int E = emax[t];
 #pragma unroll
-            for (int r = 0; r < 16; ++r) dst[off(e_a(t, r))] = from_fixed(v[r], E, G, a.exp_shift);
+            for (int r = 0; r < 16; ++r) dst[off(e_a(t, r))] = from_fixed(v[r], E + top);
         } else {
             put<e_a>(plane, v, t);
             __syncthreads();
@@ -270,7 +293,7 @@ __global__ void __launch_bounds__(kNT, 3) k2d_pass(DArgs a) {
 #pragma unroll
             for (int r = 0; r < 16; ++r) {
                 const int e = e_b(t, r);
-                dst[off(e)] = from_fixed(v[r], emax[e & ((1 << LC) - 1)], G, a.exp_shift);
+                dst[off(e)] = from_fixed(v[r], emax[e & ((1 << LC) - 1)] + top);
             }
         }
     }
