@@ -9,9 +9,9 @@
 //
 // Precision.  The elements that a pass combines (a contiguous tile, or the rows
 // of one column) share the exponent E of their largest.  Their 53-bit
-// significands are placed so that the b stages cannot overflow 95 bits and a
-// sign, which leaves 42 - b >= 30 bits below the largest one's last place:
-// elements down to 2^-30 of it enter exactly, smaller ones within 2^-83 of it.
+// significands are placed 30 bits above the lowest, so that a pass's stages (12
+// at most) cannot overflow 95 bits and a sign: elements down to 2^-30 of the
+// largest enter exactly, smaller ones within 2^-83 of it.
 // Every result is the exact sum of those, rounded once, where FP64 stages round
 // b times at 2^-53 of the partial sums.  A tile with an infinity or a NaN runs
 // the FP64 stages; results below the normal range go through one FP64 scaling.
