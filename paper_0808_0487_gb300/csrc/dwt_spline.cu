@@ -879,27 +879,28 @@ int run_spline(dwt_plan_s* P, const double* f, void* c, int batch, long long ld,
     const int s = P->s;
     const bool cplx = P->p != 2;
     const size_t eb = cplx ? 16 : 8;
-    // f~ and c~ lie in c when there is one (the transforms run in place)
+    // f~ and c~ lie in c when there is one (the transforms run in place), unless
+    // it shares memory with f in another way than p = 2's in place
+    const size_t rows = (size_t)(batch - 1) * ld + N;
+    const char *f0 = reinterpret_cast<const char*>(f), *c0 = reinterpret_cast<const char*>(c);
+    const bool apart = f0 + rows * 8 <= c0 || c0 + rows * eb <= f0;
+    const bool own = !c || !(apart || (!cplx && f0 == c0));
     double* ft = reinterpret_cast<double*>(c);
-    const long long ldt = c ? ld : N;
+    const long long ldt = own ? N : ld;
     double* part = nullptr;
     const bool want_var = var_trc || var_sup || dim;
-    const int groups = (batch + kDotRows - 1) / kDotRows;
-    if (groups > 65535) {
-        set_error("dwt_spline: batch too large");
-        return DWT_EINVAL;
-    }
+    const long long groups = ((long long)batch + kDotRows - 1) / kDotRows;
     // tiles of 1024 labels, shorter ones where those leave SMs without a tile
     int labels = 1024;
     while (labels > kDotK && (N + labels - 1) / labels * groups < 2 * 152) labels /= 2;
     const int ntile = (int)((N + labels - 1) / labels);
-    if ((!c && dmalloc((void**)&ft, (size_t)batch * N * eb, st)) ||
+    if ((own && dmalloc((void**)&ft, (size_t)batch * N * eb, st)) ||
         (want_var && dmalloc((void**)&part, (size_t)batch * 2 * s * ntile * 8, st))) {
-        if (!c) dfree(ft, st);
+        if (own) dfree(ft, st);
         return DWT_ENOMEM;
     }
     auto cleanup = [&]() {
-        if (!c) dfree(ft, st);
+        if (own) dfree(ft, st);
         dfree(part, st);
     };
     int rc = run_transform(P, f, ft, batch, ld, ldt, DWT_F64, cplx ? DWT_C128 : DWT_F64, -1, st);
@@ -907,9 +908,14 @@ int run_spline(dwt_plan_s* P, const double* f, void* c, int batch, long long ld,
     if (want_var) {
         auto kern = cplx ? k_spline_dots<true> : k_spline_dots<false>;
         if ((rc = smem_limit_max(kern))) { cleanup(); return rc; }
-        LaunchScope ls("spline_dots", st);
-        kern<<<dim3((unsigned)ntile, (unsigned)groups), kDotThreads, cplx ? kDotSmem : kDotSmemReal, st>>>(
-            ft, N, ldt, batch, 2 * s, P->d_splT, P->d_splW, part, ntile, labels);
+        constexpr int kRows = 65535 * kDotRows;   // functions of one grid
+        for (long long b0 = 0; b0 < batch; b0 += kRows) {
+            const int nb = (int)std::min<long long>(kRows, batch - b0);
+            LaunchScope ls("spline_dots", st);
+            kern<<<dim3((unsigned)ntile, (unsigned)((nb + kDotRows - 1) / kDotRows)), kDotThreads,
+                   cplx ? kDotSmem : kDotSmemReal, st>>>(ft + b0 * ldt * (cplx ? 2 : 1), N, ldt, nb, 2 * s, P->d_splT,
+                                                         P->d_splW, part + b0 * 2 * s * ntile, ntile, labels);
+        }
     } else {
         LaunchScope ls("spline_scale", st);
         k_spline_scale<<<grid_sp((long long)batch * N), 256, 0, st>>>(ft, cplx ? 1 : 0, N, ldt, (long long)batch * N,

@@ -71,3 +71,26 @@ def test_rows_of_different_size_and_special_values(dwt, dev, orc):
         else:
             assert np.array_equal(vt[b], np.ldexp(vt[ref], 2 * e[b])) and np.array_equal(vs[b], np.ldexp(vs[ref], 2 * e[b]))
             assert np.array_equal(dim[b], dim[ref])
+
+
+# the coefficients' buffer holds the intermediate values unless it shares memory
+# with the samples: in place (p = 2), or samples inside the complex coefficients
+@pytest.mark.parametrize("p,m,off", [(2, 13, 0), (2, 13, 40), (3, 6, 0), (3, 6, 729)])
+def test_samples_inside_the_coefficients(dwt, dev, orc, p, m, off):
+    N, s, B = p ** m, 3, 3
+    C = S.small_net(p, m, s, index=430 + m)
+    f0 = orc.eval_product(p, m, orc.net_points(p, m, C), 1.0 / np.arange(1, s + 1))
+    fs = f0[None, :] * np.array([[1.0], [-2.5], [0.3]])
+    plan = dwt.dwt_plan(p, m, s, C, dwt.DWT_PLAN_TRANSFORM_ONLY)
+    dwt.dwt_spline_prepare(plan, 2.0, 0.9 / np.arange(1, s + 1))
+    vt, vs, dim, c = _spline(dwt, dev, plan, fs, s)
+    buf = torch.zeros(2 * B * N + 64, dtype=torch.float64, device=dev)
+    f = buf[off:off + B * N].view(B, N)
+    f.copy_(torch.from_numpy(fs))
+    cb = buf[:B * N].view(B, N) if p == 2 else torch.view_as_complex(buf[:2 * B * N].view(B, N, 2))
+    v = torch.empty((2, B, s + 1), dtype=torch.float64, device=dev)
+    d = torch.empty((B, 2), dtype=torch.int32, device=dev)
+    dwt.dwt_spline(plan, f, cb, B, N, v[0], v[1], d)
+    assert np.array_equal(cb.cpu().numpy(), c)
+    assert np.array_equal(v[0].cpu().numpy(), vt) and np.array_equal(v[1].cpu().numpy(), vs)
+    assert np.array_equal(d.cpu().numpy(), dim)
