@@ -328,22 +328,22 @@ int launch(int B, const DArgs& a, long long N, int nf, const char* fam, cudaStre
     }
 }
 
-const long long kL2GroupD = 48ll << 20;   // bytes of functions kept in L2 between the passes
-
 }  // namespace
 
 bool p2d_ok(int m) { return m >= kLT; }
 
 // dwt_forward / dwt_inverse for p = 2, FP64, m >= 12: the 12 low digits, then
 // the others in passes of at most 9 (rows of 64 bytes at least), as even as
-// possible.
+// possible.  Each pass takes all functions: its conversions and additions bound
+// it, not the traffic that groups of functions within L2 would save, and a
+// group's last wave is short (32 functions of 2^20: 305 us in groups of 48 MB,
+// 287 of 96 MB, 270 so; 8 of 2^22: 443, 416, 391; 2 of 2^24: 407, 407, 398).
 int p2d_transform(dwt_plan_s* Pl, const double* in, double* out, int batch, long long ld_in, long long ld_out,
                   int sgn, cudaStream_t st) {
     const int m = Pl->m, high = m - kLT, nh = (high + 8) / 9;
     const long long N = Pl->N;
-    const int G = (int)std::min(65535ll, std::max(1ll, kL2GroupD / (N * 8)));
-    for (int f0 = 0; f0 < batch; f0 += G) {
-        const int nf = std::min(G, batch - f0);
+    for (int f0 = 0; f0 < batch; f0 += 65535) {
+        const int nf = std::min(65535, batch - f0);
         DArgs a{in + (long long)f0 * ld_in, out + (long long)f0 * ld_out, ld_in, ld_out, 1, 0};
         if (nh == 0 && sgn < 0) a.exp_shift = -m;
         int rc = launch(kLT, a, N, nf, "pass_lo", st);
