@@ -150,16 +150,40 @@ __device__ __noinline__ double from_fixed_any(W96 v, uint32_t sign, int e) {   /
     return e + 128 < 1 ? 0.0 : round53(h, l, rest, e + 128, sign) * 0x1p-128;   // below the normal range
 }
 
-// fixed point -> nearest double (ties to even); top = the exponent field of bit
-// 95.  All lanes of the warp call it: results in the top word's range and of
-// normal size take the short way, a warp with any other takes the long one.
-__device__ __forceinline__ double from_fixed(W96 v, int top) {
-    const uint32_t sign = (uint32_t)((int)v.c >> 31);
-    v = negate_if(v, sign);
-    const int lz = __clz((int)v.c), e = top - lz;
-    const bool odd = v.c == 0 || (unsigned)(e - 1) >= 0x7feu;
-    if (__any_sync(0xffffffffu, odd)) return from_fixed_any(v, sign, top);
-    return round53(__funnelshift_l(v.b, v.c, lz), __funnelshift_l(v.a, v.b, lz), v.a << lz, e, sign);
+// fixed point -> nearest double (ties to even) of four numbers; top[i] = the
+// exponent field of bit 95.  All lanes of the warp call it: results of normal
+// size in the top word's range take the shortest way, and those in the second
+// word's (below 2^-19 of the group's largest element, as high coefficients of
+// smooth functions) the next one.
+__device__ __forceinline__ void from_fixed4(const W96* v, const int* top, double* y) {
+    uint32_t sign[4];
+    W96 n[4];
+    bool odd = false;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        sign[i] = (uint32_t)((int)v[i].c >> 31);
+        n[i] = negate_if(v[i], sign[i]);
+        odd = odd || n[i].c == 0 || (unsigned)(top[i] - 32) >= 0x7ffu - 32u;   // exponent 1 .. 0x7fe with up to 31 zeros
+    }
+    if (!__any_sync(0xffffffffu, odd)) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int lz = __clz((int)n[i].c);
+            y[i] = round53(__funnelshift_l(n[i].b, n[i].c, lz), __funnelshift_l(n[i].a, n[i].b, lz), n[i].a << lz,
+                           top[i] - lz, sign[i]);
+        }
+        return;
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const bool z = n[i].c == 0;
+        const uint32_t h = z ? n[i].b : n[i].c, l = z ? n[i].a : n[i].b, r = z ? 0u : n[i].a;
+        const int lz = __clz((int)h), e = top[i] - lz - (z ? 32 : 0);
+        if (__any_sync(0xffffffffu, h == 0 || (unsigned)(e - 1) >= 0x7feu))
+            y[i] = from_fixed_any(n[i], sign[i], top[i]);
+        else
+            y[i] = round53(__funnelshift_l(l, h, lz), __funnelshift_l(r, l, lz), r << lz, e, sign[i]);
+    }
 }
 
 // stages of register bits LO .. 3
@@ -278,7 +302,13 @@ __global__ void __launch_bounds__(kNT, 3) k2d_pass(DArgs a) {
         stages<0>(v);
         if constexpr (B == 4) {
 #pragma unroll
-            for (int r = 0; r < 16; ++r) dst[off(e_a(t, r))] = from_fixed(v[r], E + top);
+            for (int r = 0; r < 16; r += 4) {
+                const int tops[4] = {E + top, E + top, E + top, E + top};
+                double y[4];
+                from_fixed4(v + r, tops, y);
+#pragma unroll
+                for (int i = 0; i < 4; ++i) dst[off(e_a(t, r + i))] = y[i];
+            }
         } else {
             put<e_a>(plane, v, t);
             __syncthreads();
@@ -291,9 +321,14 @@ __global__ void __launch_bounds__(kNT, 3) k2d_pass(DArgs a) {
             get<e_b>(plane, v, t);
             stages<(LC > 4 ? LC - 4 : 0)>(v);
 #pragma unroll
-            for (int r = 0; r < 16; ++r) {
-                const int e = e_b(t, r);
-                dst[off(e)] = from_fixed(v[r], emax[e & ((1 << LC) - 1)] + top);
+            for (int r = 0; r < 16; r += 4) {
+                int tops[4];
+                double y[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) tops[i] = emax[e_b(t, r + i) & ((1 << LC) - 1)] + top;
+                from_fixed4(v + r, tops, y);
+#pragma unroll
+                for (int i = 0; i < 4; ++i) dst[off(e_b(t, r + i))] = y[i];
             }
         }
     }
