@@ -111,15 +111,17 @@ __global__ void k_spline_scale(double* ft, int cplx, long long N, long long ld, 
 // A batch of 32 functions against 32 tables is a matrix product with the labels
 // as inner dimension, in FP64.  This GPU multiplies 1.7 FP64 numbers per clock
 // and SM, so the product runs on the tensor cores in exact pieces instead: in
-// blocks of 64 labels every operand becomes a 64-bit fixed-point number, scaled
-// by its row's largest exponent so far in the tile, split into eight signed
+// blocks of 64 labels every operand (for real data the square straight from c~'s
+// significand) becomes a 64-bit fixed-point number, scaled by its row's largest
+// exponent so far in the tile, split into eight signed
 // digits of base 256 that FP16 holds exactly; a digit product is below 2^14 and
 // the 8 x 64 products that share a weight sum to less than 2^24, exact in FP32.
 // The 36 digit pairs of weight >= 256^7 are multiplied (the others lie 2^-62
 // below the largest product); the sums join 128-bit integers per pair of
 // function and table, shifted when a row's exponent grows, and become FP64 once
 // per tile.  FP64 rounds every product and every sum at 2^-53.  Rows with an
-// infinity or a NaN in the tile take FP64 sums at the end.
+// infinity, a NaN or a square near the largest number in the tile take FP64 sums
+// at the end.
 //
 // The next block's numbers come into a thread's own part of shared memory while
 // this block's digits are multiplied (real data; complex data are loaded when
@@ -127,7 +129,8 @@ __global__ void k_spline_scale(double* ft, int cplx, long long N, long long ld, 
 //
 // p = 2, m = 20, s = 16, 32 functions: 2920 us on the FP64 pipe (one CTA per
 // function and 4096 labels) plus 95 us for the scaling; so 459 us, with the
-// asynchronous loads 420 us.
+// asynchronous loads 420 us, with fewer instructions per number (integer squares,
+// one bounds check per block, sums of the upper weights read off the bits) 376 us.
 constexpr int kDotThreads = 256;
 constexpr int kDotRows = 32;                  // functions, and tables, per round
 constexpr int kDotK = 64;                     // labels per block
@@ -143,23 +146,36 @@ __device__ __forceinline__ void cp_async8(uint32_t dst, const void* src) {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(dst), "l"(src) : "memory");
 }
 
-__device__ __forceinline__ int expo(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
+__device__ __forceinline__ uint32_t abs_hi(double x) { return (uint32_t)__double2hiint(x) & 0x7fffffffu; }
 
-// 64-bit fixed point of x against exponent E (>= x's): significand 2^9 at E
-__device__ __forceinline__ unsigned long long to_fix64(double x, int E) {
-    const int ex = expo(x);
-    unsigned long long mnt = (unsigned long long)__double_as_longlong(x) & 0xfffffffffffffull;
-    if (ex) mnt |= 0x10000000000000ull;
-    const int d = E - max(ex, 1);
-    mnt = d > 63 ? 0ull : (mnt << 9) >> d;
-    return __double2hiint(x) < 0 ? 0ull - mnt : mnt;
+// 64-bit fixed point of x against exponent E (>= x's), significand 2^9 at E, plus
+// 128 in every byte with carries: byte - 128 is the signed digit
+template <bool SIGNED> __device__ __forceinline__ unsigned long long to_fix64(double x, int E) {
+    const uint32_t h = (uint32_t)__double2hiint(x);
+    const int ex = (int)((h >> 20) & 0x7ffu);
+    const uint32_t mh = (h & 0xfffffu) | (ex ? 0x100000u : 0u);
+    const int d = min(E - max(ex, 1), 63);   // 62 bits
+    unsigned long long v = ((((unsigned long long)mh << 32) | (uint32_t)__double2loint(x)) << 9) >> d;
+    if constexpr (SIGNED) {   // -v = ~v + 1
+        const uint32_t s = (uint32_t)((int)h >> 31);
+        v ^= ((unsigned long long)s << 32) | s;
+        return v + ((0x80808080ull << 32) | (0x80808080u - s));
+    }
+    return v + 0x8080808080808080ull;
+}
+
+// u^2 the same way, u's exponents against E: the top 62 of its 106 bits at E
+__device__ __forceinline__ unsigned long long square_fix64(double u, int E) {
+    const uint32_t h = (uint32_t)__double2hiint(u), lo = (uint32_t)__double2loint(u);
+    const int ex = (int)((h >> 20) & 0x7ffu);
+    const uint32_t mh = (h & 0xfffffu) | (ex ? 0x100000u : 0u);
+    const unsigned long long hh = (unsigned long long)mh * mh, mid = (unsigned long long)(2 * mh) * lo + __umulhi(lo, lo);
+    const int d = min(2 * (E - max(ex, 1)), 63);
+    return (((hh << 20) + (mid >> 12)) >> d) + 0x8080808080808080ull;
 }
 
 // the digits of two numbers (label l and l + 32 of a block) into their planes
 __device__ __forceinline__ void put_digits(__half* row, unsigned long long f0, unsigned long long f1, int lane) {
-    // + 128 in every byte with carries: byte - 128 is the signed digit
-    f0 += 0x8080808080808080ull;
-    f1 += 0x8080808080808080ull;
     const uint32_t lo0 = (uint32_t)f0, hi0 = (uint32_t)(f0 >> 32), lo1 = (uint32_t)f1, hi1 = (uint32_t)(f1 >> 32);
     const __half2 off = __halves2half2(__ushort_as_half(0xE480), __ushort_as_half(0xE480));   // -(1024 + 128)
 #pragma unroll
@@ -203,7 +219,7 @@ __global__ void __launch_bounds__(kDotThreads, 2) k_spline_dots(double* ct, long
     __half* B = A + kDotOperand;
     int* grow = reinterpret_cast<int*>(B + kDotOperand);   // [2][32]: growth of the rows' exponents in this block
     int* bad = grow + 2 * kDotRows;                        // [2][32]: rows with an infinity or a NaN
-    const double* mine = reinterpret_cast<const double*>(bad + 2 * kDotRows) + threadIdx.x;   // real data: [18][threads]
+    double* mine = reinterpret_cast<double*>(bad + 2 * kDotRows) + threadIdx.x;   // real data: [18][threads]
     const uint32_t stage = (uint32_t)__cvta_generic_to_shared(mine);
     const int t = threadIdx.x, lane = t & 31, w = t >> 5;
     const int tile = blockIdx.x, f0 = blockIdx.y * kDotRows;
@@ -214,29 +230,46 @@ __global__ void __launch_bounds__(kDotThreads, 2) k_spline_dots(double* ct, long
     const uint32_t aoff = sA + 2u * (uint32_t)((fo + (lane & 15)) * kDotStride + 8 * (lane >> 4));
     const uint32_t boff = sB + 2u * (uint32_t)((to + (lane & 7)) * kDotStride + 8 * ((lane >> 3) & 1));
     for (int t0 = 0; t0 < nt; t0 += kDotRows) {
+        // top word of the first function-side number whose row takes FP64 sums: real
+        // rows hold c~, whose square must not overflow
+        constexpr int kDotPower = CPLX ? 1 : 2;   // powers of two of the sum per exponent of a function-side number
+        constexpr uint32_t kDotHuge = CPLX ? 0x7ff00000u : (1023u + 511u) << 20;
         __syncthreads();
         if (t < 2 * kDotRows) bad[t] = 0;
         int Ea[4] = {1, 1, 1, 1}, Et[4] = {1, 1, 1, 1};   // exponents of this warp's rows
-        int ea[2] = {1, 1}, et[2] = {1, 1};               // of the rows of this thread's sums
+        int ea[2] = {CPLX ? 1 : 2, CPLX ? 1 : 2}, et[2] = {1, 1};   // of the rows of this thread's sums
         long long hi[4] = {0, 0, 0, 0}, lo[4] = {0, 0, 0, 0};   // sum = hi 2^32 + lo
         // real data: this thread's numbers of a block, requested one block ahead
+        // (zeros past the last function, table or label)
+        const bool all = f0 + kDotRows <= batch && t0 + kDotRows <= nt;
+        const double* pa = ct + (f0 + 4 * w) * ld + lane;
+        const double* pt = tab + (t0 + 4 * w) * N + lane;
         auto request = [&](long long hb) {
-            const long long l0 = hb + lane, l1 = l0 + 32;
+            if (all && hb + kDotK <= h1) {
+                const double *ra = pa + hb, *rt = pt + hb;
 #pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const int f = f0 + 4 * w + k, tb = t0 + 4 * w + k;
-                if (f < batch) {
-                    if (l0 < h1) cp_async8(stage + (2 * k) * kDotThreads * 8, ct + f * ld + l0);
-                    if (l1 < h1) cp_async8(stage + (2 * k + 1) * kDotThreads * 8, ct + f * ld + l1);
+                for (int k = 0; k < 4; ++k) {
+                    cp_async8(stage + (2 * k) * kDotThreads * 8, ra);
+                    cp_async8(stage + (2 * k + 1) * kDotThreads * 8, ra + 32);
+                    cp_async8(stage + (8 + 2 * k) * kDotThreads * 8, rt);
+                    cp_async8(stage + (9 + 2 * k) * kDotThreads * 8, rt + 32);
+                    ra += ld;
+                    rt += N;
                 }
-                if (tb < nt) {
-                    if (l0 < h1) cp_async8(stage + (8 + 2 * k) * kDotThreads * 8, tab + (long long)tb * N + l0);
-                    if (l1 < h1) cp_async8(stage + (9 + 2 * k) * kDotThreads * 8, tab + (long long)tb * N + l1);
+                if (t0 == 0) {
+                    cp_async8(stage + 16 * kDotThreads * 8, W + hb + lane);
+                    cp_async8(stage + 17 * kDotThreads * 8, W + hb + lane + 32);
                 }
+                return;
             }
-            if (t0 == 0) {
-                if (l0 < h1) cp_async8(stage + 16 * kDotThreads * 8, W + l0);
-                if (l1 < h1) cp_async8(stage + 17 * kDotThreads * 8, W + l1);
+#pragma unroll 1
+            for (int i = 0; i < kDotStage; ++i) {
+                const int k = (i >> 1) & 3;
+                const long long off = hb + 32 * (i & 1);
+                const double* src = i < 8 ? pa + k * ld + off : i < 16 ? pt + k * N + off : W + lane + off;
+                const bool there = off + lane < h1 && (i < 8 ? f0 + 4 * w + k < batch : i < 16 ? t0 + 4 * w + k < nt : t0 == 0);
+                if (there) cp_async8(stage + i * kDotThreads * 8, src);
+                else mine[i * kDotThreads] = 0.0;
             }
         };
         if constexpr (!CPLX) request(h0);
@@ -244,21 +277,15 @@ __global__ void __launch_bounds__(kDotThreads, 2) k_spline_dots(double* ct, long
             const long long l0 = hb + lane, l1 = l0 + 32;
             const bool in0 = l0 < h1, in1 = l1 < h1;
             double a[4][2], x[4][2];
-            double w0 = 1.0, w1 = 1.0;
             if constexpr (CPLX) {
+                double w0 = 1.0, w1 = 1.0;
                 if (t0 == 0 && in0) w0 = W[l0];
                 if (t0 == 0 && in1) w1 = W[l1];
-            } else {
-                asm volatile("cp.async.wait_all;" ::: "memory");
-                if (t0 == 0 && in0) w0 = mine[16 * kDotThreads];
-                if (t0 == 0 && in1) w1 = mine[17 * kDotThreads];
-            }
 #pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const int f = f0 + 4 * w + k, tb = t0 + 4 * w + k;
-                a[k][0] = a[k][1] = x[k][0] = x[k][1] = 0.0;
-                if (f < batch) {
-                    if constexpr (CPLX) {
+                for (int k = 0; k < 4; ++k) {
+                    const int f = f0 + 4 * w + k, tb = t0 + 4 * w + k;
+                    a[k][0] = a[k][1] = x[k][0] = x[k][1] = 0.0;
+                    if (f < batch) {
                         double2* row = reinterpret_cast<double2*>(ct) + f * ld;
                         double2 u = in0 ? row[l0] : make_double2(0.0, 0.0), v = in1 ? row[l1] : make_double2(0.0, 0.0);
                         if (t0 == 0) {
@@ -269,53 +296,87 @@ __global__ void __launch_bounds__(kDotThreads, 2) k_spline_dots(double* ct, long
                         }
                         a[k][0] = u.x * u.x + u.y * u.y;
                         a[k][1] = v.x * v.x + v.y * v.y;
-                    } else {
-                        double* row = ct + f * ld;
-                        double u = in0 ? mine[(2 * k) * kDotThreads] : 0.0, v = in1 ? mine[(2 * k + 1) * kDotThreads] : 0.0;
-                        if (t0 == 0) {
-                            u *= w0;
-                            v *= w1;
-                            if (in0) row[l0] = u;
-                            if (in1) row[l1] = v;
-                        }
-                        a[k][0] = u * u;
-                        a[k][1] = v * v;
                     }
-                }
-                if (tb < nt) {
-                    if constexpr (CPLX) {
+                    if (tb < nt) {
                         const double* row = tab + (long long)tb * N;
                         if (in0) x[k][0] = row[l0];
                         if (in1) x[k][1] = row[l1];
-                    } else {
-                        if (in0) x[k][0] = mine[(8 + 2 * k) * kDotThreads];
-                        if (in1) x[k][1] = mine[(9 + 2 * k) * kDotThreads];
+                    }
+                }
+            } else {
+                asm volatile("cp.async.wait_all;" ::: "memory");
+#pragma unroll
+                for (int k = 0; k < 4; ++k)
+#pragma unroll
+                    for (int u = 0; u < 2; ++u) {
+                        a[k][u] = mine[(2 * k + u) * kDotThreads];
+                        x[k][u] = mine[(8 + 2 * k + u) * kDotThreads];
+                    }
+                if (t0 == 0) {
+                    const double w0 = mine[16 * kDotThreads], w1 = mine[17 * kDotThreads];
+                    double* row = ct + (f0 + 4 * w) * ld + l0;
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        a[k][0] *= w0;
+                        a[k][1] *= w1;
+                        if (all || f0 + 4 * w + k < batch) {
+                            if (in0) row[0] = a[k][0];
+                            if (in1) row[32] = a[k][1];
+                        }
+                        row += ld;
                     }
                 }
             }
             __syncthreads();   // the previous block's digits and growths have been read
+            // the rows' largest exponents: eight reductions in flight
+            uint32_t ma[4], mx[4], most = 0;
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
-                auto put = [&](double (&v)[2], int& E, int side, __half* plane) {
-                    const int r = 4 * w + k;
-                    int m0 = expo(v[0]), m1 = expo(v[1]);
-                    if (m0 == 0x7ff || m1 == 0x7ff) {
-                        bad[side * kDotRows + r] = 1;
-                        v[0] = v[1] = 0.0;
-                        m0 = m1 = 0;
-                    }
-                    const int top = max((int)__reduce_max_sync(0xffffffffu, max(m0, m1)), E);
-                    if (lane == 0) grow[side * kDotRows + r] = top - E;
-                    E = top;
-                    put_digits(plane + r * kDotStride, to_fix64(v[0], E), to_fix64(v[1], E), lane);
-                };
-                put(a[k], Ea[k], 0, A);
-                put(x[k], Et[k], 1, B);
+                ma[k] = __reduce_max_sync(0xffffffffu, max(abs_hi(a[k][0]), abs_hi(a[k][1])));
+                mx[k] = __reduce_max_sync(0xffffffffu, max(abs_hi(x[k][0]), abs_hi(x[k][1])));
+                most = max(most, max(ma[k], mx[k]));
+            }
+            if (most >= kDotHuge) {
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    double(&v)[2] = i < 4 ? a[i] : x[i - 4];
+                    uint32_t& m = i < 4 ? ma[i] : mx[i - 4];
+                    if (m < (i < 4 ? kDotHuge : 0x7ff00000u)) continue;
+                    bad[(i >> 2) * kDotRows + 4 * w + (i & 3)] = 1;
+                    v[0] = v[1] = 0.0;
+                    m = 0;
+                }
+            }
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const int r = 4 * w + k;
+                const int na = max((int)(ma[k] >> 20), Ea[k]), nx = max((int)(mx[k] >> 20), Et[k]);
+                if (lane == 0) {
+                    grow[r] = kDotPower * (na - Ea[k]);
+                    grow[kDotRows + r] = nx - Et[k];
+                }
+                Ea[k] = na;
+                Et[k] = nx;
+            }
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const int r = 4 * w + k;
+                if constexpr (CPLX)
+                    put_digits(A + r * kDotStride, to_fix64<false>(a[k][0], Ea[k]), to_fix64<false>(a[k][1], Ea[k]), lane);
+                else
+                    put_digits(A + r * kDotStride, square_fix64(a[k][0], Ea[k]), square_fix64(a[k][1], Ea[k]), lane);
+                put_digits(B + r * kDotStride, to_fix64<true>(x[k][0], Et[k]), to_fix64<true>(x[k][1], Et[k]), lane);
             }
             if constexpr (!CPLX)
                 if (hb + kDotK < h1) request(hb + kDotK);   // this block's numbers have been used
             __syncthreads();
-            float acc[kDotDigits][4] = {};
+            // weights 256^11 and up: at most 4 x 64 products of 2^14 onto 3 2^22, whose
+            // last place is one: the sum is read off the bits
+            float acc[kDotDigits][4];
+#pragma unroll
+            for (int c = 0; c < kDotDigits; ++c)
+#pragma unroll
+                for (int q = 0; q < 4; ++q) acc[c][q] = c < 4 ? 0.f : 12582912.f;
 #pragma unroll 1
             for (int k = 0; k < kDotK / 16; ++k) {
                 uint32_t fb[kDotDigits][2];
@@ -347,14 +408,12 @@ __global__ void __launch_bounds__(kDotThreads, 2) k_spline_dots(double* ct, long
                     hi[q] = (long long)(v >> 32);
                     lo[q] = (long long)((unsigned long long)v & 0xffffffffull);
                 }
-                long long s0 = 0, s1 = 0;
-#pragma unroll
-                for (int c = 3; c >= 0; --c) {
-                    s0 = s0 * 256 + (long long)__float2int_rn(acc[c][q]);
-                    s1 = s1 * 256 + (long long)__float2int_rn(acc[c + 4][q]);
-                }
-                lo[q] += s0;
-                hi[q] += s1;
+                // pairs of weights fit 32 bits: 5 x 64 x 2^22 and 7 x 64 x 2^22 at most
+                auto whole = [&](int c) { return c < 4 ? __float2int_rn(acc[c][q]) : __float_as_int(acc[c][q]) - 0x4b400000; };
+                lo[q] += whole(1) * 256 + whole(0);
+                lo[q] += (long long)(whole(3) * 256 + whole(2)) * 65536;
+                hi[q] += whole(5) * 256 + whole(4);
+                hi[q] += (long long)(whole(7) * 256 + whole(6)) * 65536;
             }
         }
         __syncthreads();   // bad is complete, c~ of the tile is written
@@ -372,8 +431,10 @@ __global__ void __launch_bounds__(kDotThreads, 2) k_spline_dots(double* ct, long
                     v += m2 * tab[(long long)tb * N + H];
                 }
             } else {
-                // digits of weight 256^7 and up; 2^(E - 1084) is the unit of a row
-                v = scalbn((double)hi[q] * 4294967296.0 + (double)lo[q], 56 + ea[q >> 1] + et[q & 1] - 2168);
+                // digits of weight 256^7 and up; the unit of a row is 2^(E - 1084), of a
+                // row of squares 2^(2 E - 2106)
+                v = scalbn((double)hi[q] * 4294967296.0 + (double)lo[q],
+                           56 + ea[q >> 1] + et[q & 1] - 1084 - (CPLX ? 1084 : 2106));
             }
             part[((long long)f * nt + tb) * ntile + tile] = v;
         }
