@@ -94,3 +94,24 @@ def test_samples_inside_the_coefficients(dwt, dev, orc, p, m, off):
     assert np.array_equal(cb.cpu().numpy(), c)
     assert np.array_equal(v[0].cpu().numpy(), vt) and np.array_equal(v[1].cpu().numpy(), vs)
     assert np.array_equal(d.cpu().numpy(), dim)
+
+
+def test_squares_near_the_largest_number(dwt, dev, orc):
+    # rows whose squares come near the largest double, or pass it, take FP64 sums:
+    # finite ones within 2^12 roundings of the scaled row, the others infinite
+    p, m, s = 2, 12, 6
+    C = S.small_net(p, m, s, index=440)
+    f0 = orc.eval_product(p, m, orc.net_points(p, m, C), 1.0 / np.arange(1, s + 1))
+    e = np.array([0, 470, 490, 500, 530, 600])
+    fs = np.ldexp(f0[None, :], e[:, None])
+    plan = dwt.dwt_plan(p, m, s, C, dwt.DWT_PLAN_TRANSFORM_ONLY)
+    dwt.dwt_spline_prepare(plan, 2.0, 0.9 / np.arange(1, s + 1))
+    vt, vs, _, _ = _spline(dwt, dev, plan, fs, s)
+    with np.errstate(over="ignore"):
+        for b in range(len(e)):
+            for v in (vt, vs):
+                want = np.ldexp(v[0], 2 * e[b])
+                if e[b] >= 530:
+                    assert not np.isfinite(v[b, 1:]).any()
+                else:
+                    assert np.allclose(v[b], want, rtol=0, atol=2.0 ** -41 * want[-1])
