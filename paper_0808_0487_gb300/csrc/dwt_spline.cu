@@ -130,7 +130,9 @@ __global__ void k_spline_scale(double* ft, int cplx, long long N, long long ld, 
 // p = 2, m = 20, s = 16, 32 functions: 2920 us on the FP64 pipe (one CTA per
 // function and 4096 labels) plus 95 us for the scaling; so 459 us, with the
 // asynchronous loads 420 us, with fewer instructions per number (integer squares,
-// one bounds check per block, sums of the upper weights read off the bits) 376 us.
+// one bounds check per block, sums of the upper weights read off the bits) 376 us,
+// with whole waves of tiles 361 us.  (Eight warps that convert beside eight that
+// multiply, double buffered, one CTA per SM: 388 us.)
 constexpr int kDotThreads = 256;
 constexpr int kDotRows = 32;                  // functions, and tables, per round
 constexpr int kDotK = 64;                     // labels per block
@@ -951,9 +953,13 @@ int run_spline(dwt_plan_s* P, const double* f, void* c, int batch, long long ld,
     double* part = nullptr;
     const bool want_var = var_trc || var_sup || dim;
     const long long groups = ((long long)batch + kDotRows - 1) / kDotRows;
-    // tiles of 1024 labels, shorter ones where those leave SMs without a tile
-    int labels = 1024;
-    while (labels > kDotK && (N + labels - 1) / labels * groups < 2 * 152) labels /= 2;
+    // tiles of at most 2048 labels (an odd row's FP64 sums walk one), as many as
+    // fill whole waves of two CTAs per SM: p = 2, m = 20, 32 functions take 608
+    // tiles of 27 blocks, 361 us, where 1024 of 16 in 3.4 waves took 376
+    const long long blocks = (N + kDotK - 1) / kDotK, slots = 2 * 152;
+    const long long waves = std::max(1ll, ((blocks + 31) / 32 * groups + slots - 1) / slots);
+    const long long want = std::max(1ll, std::min(blocks, waves * slots / groups));
+    const int labels = (int)((blocks + want - 1) / want) * kDotK;
     const int ntile = (int)((N + labels - 1) / labels);
     if ((own && dmalloc((void**)&ft, (size_t)batch * N * eb, st)) ||
         (want_var && dmalloc((void**)&part, (size_t)batch * 2 * s * ntile * 8, st))) {
