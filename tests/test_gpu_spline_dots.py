@@ -115,3 +115,25 @@ def test_squares_near_the_largest_number(dwt, dev, orc):
                     assert not np.isfinite(v[b, 1:]).any()
                 else:
                     assert np.allclose(v[b], want, rtol=0, atol=2.0 ** -41 * want[-1])
+
+
+def test_tiles_of_several_waves(dwt, dev, orc):
+    # 10 groups of functions times 1024 blocks of labels: two waves of tiles of 18
+    # blocks and a shorter last one, against one function's tiles of one wave and
+    # the oracle
+    p, m, s, B = 2, 16, 2, 320
+    C = S.small_net(p, m, s, index=450)
+    Y = orc.net_points(p, m, C)
+    gamma = 0.9 / np.arange(1, s + 1)
+    f0 = orc.eval_product(p, m, Y, 1.0 / np.arange(1, s + 1))
+    fs = f0[None, :] * (1.0 + np.arange(B)[:, None] / 64.0)
+    plan = dwt.dwt_plan(p, m, s, C, dwt.DWT_PLAN_TRANSFORM_ONLY)
+    dwt.dwt_spline_prepare(plan, 2.0, gamma)
+    vt, vs, dim, _ = _spline(dwt, dev, plan, fs, s)
+    r = orc.spline(p, m, Y, fs[319], 2.0, gamma)
+    assert np.all(np.abs(vt[319] - r["var_trc"]) <= 1e-9 * r["var_trc"][-1])
+    for b in (0, 31, 32, 200, 319):
+        v1, w1, d1, _ = _spline(dwt, dev, plan, fs[b:b + 1], s)
+        # sums of 2^10 tiles at most, rounded at 2^-53 each
+        assert np.all(np.abs(vt[b] - v1[0]) <= 2.0 ** -43 * v1[0, -1]) and np.all(np.abs(vs[b] - w1[0]) <= 2.0 ** -43 * v1[0, -1])
+        assert np.array_equal(dim[b], d1[0])
