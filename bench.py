@@ -296,9 +296,9 @@ def accuracy_vs_oracle(acc_in, f):
 # that source makes the figures stale: they are then reported as null.
 MEASURED_TRAFFIC = {
     "source": "paper_0808_0487_gb300/csrc/dwt_p2i.cu",
-    "sha256": "9f4acc73da8a8b9bcace41645fce869a7c34ae351e67f03c4ba7061996fe0bc8",
-    # top pass: mean of two launches (81.5 and 100.9 MB); paired low pass: one launch
-    "bytes_per_launch": {"interp_top": 91.2e6, "interp_inv_fwd": 138.5e6},
+    "sha256": "3e5866ec963e04d8f230cce9aecd1f10c721db449d9dd01ae16dc0046d3d9481",
+    # top pass: mean of two launches (80.2 and 104.8 MB); paired low pass: one launch
+    "bytes_per_launch": {"interp_top": 92.5e6, "interp_inv_fwd": 140.2e6},
 }
 
 
@@ -462,14 +462,16 @@ def run_other_configs(dwt, dev, stream, timed, steps):
         dwt.dwt_spline(plan2, fs, cs, 32, N2, vts, vss, dims, stream=stream)
 
     ms_s, _ = timed(spl, steps)
-    # the variance contraction reads |c~|^2 and the 2s tables once per function
+    # the variance contraction reads f~ and W_K, writes c~, and reads the 2s tables
+    # once for its 32 functions
+    dots_bpp = 16 + (2 * 16 + 1) * 8 / 32
     dwt.dwt_profile_reset()
     dwt.dwt_profile_enable(True)
     timed(spl, 1)
     dwt.dwt_profile_enable(False)
     nd, td = dwt.dwt_profile_query("spline_dots")
     dwt.dwt_profile_reset()
-    dots_gbs = (2 * 16 + 1) * N2 * 8 * 32 / (td / max(nd, 1) / 1e3) / 1e9 if nd else None
+    dots_gbs = dots_bpp * N2 * 32 / (td / max(nd, 1) / 1e3) / 1e9 if nd else None
     # values at the net shifted by one point of the finer net (the hold-out half
     # of a 2N-point net) and the squared error against the function there
     delta = [int(S.integers(S.stream_seed(2, S.P_SAMPLE, j), 1, 0, (1 << 21) - 1)[0]) | 1 for j in range(16)]
@@ -501,7 +503,7 @@ def run_other_configs(dwt, dev, stream, timed, steps):
                                                        "ms": ms_e / ne,
                                                        "function_values_per_s": 32 * Qe * ne / (ms_e / 1e3),
                                                        "fp64_mul_per_s": fp64_ops},
-                                    "dots_kernel": {"achieved_gbs": dots_gbs, "bytes_per_point": (2 * 16 + 1) * 8,
+                                    "dots_kernel": {"achieved_gbs": dots_gbs, "bytes_per_point": dots_bpp,
                                                     "frac": dots_gbs / _peaks()[0] if dots_gbs else None}}
     del fs, cs, vals, ve
     w = S.workload_p3_m13()
