@@ -296,7 +296,7 @@ def accuracy_vs_oracle(acc_in, f):
 # that source makes the figures stale: they are then reported as null.
 MEASURED_TRAFFIC = {
     "source": "paper_0808_0487_gb300/csrc/dwt_p2i.cu",
-    "sha256": "3e5866ec963e04d8f230cce9aecd1f10c721db449d9dd01ae16dc0046d3d9481",
+    "sha256": "ce189fa2289c2e643514c309a17258d9b1e6232015091b8b5cf3fbe5312cd07d",
     # top pass: mean of two launches (80.2 and 104.8 MB); paired low pass: one launch
     "bytes_per_launch": {"interp_top": 92.5e6, "interp_inv_fwd": 140.2e6},
 }

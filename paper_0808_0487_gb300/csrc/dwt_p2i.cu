@@ -7,9 +7,9 @@
 // Between the passes the function's 64 MB stay in L2.  This file holds
 //
 //  k2i_top<B>: the fused top pass.  A tile is 2^B rows (2^14 apart) of
-//    Wc = 2^(14-B) consecutive columns, 64 KB, moved between L2 and shared
+//    Wc = 2^(13-B) consecutive columns, 32 KB, moved between L2 and shared
 //    memory by the tensor-memory-access unit (cp.async.bulk.tensor), so that
-//    the narrow row segments cost no load/store-unit work; 256 threads hold 64
+//    the narrow row segments cost no load/store-unit work; 128 threads hold 64
 //    elements each.  Register layouts as in the p = 2 high pass: layout A
 //    (float4 at 4(t + 256 q), the top four row digits in thread) and layout P
 //    (six row digits in thread).  Between the forward and inverse stages the
