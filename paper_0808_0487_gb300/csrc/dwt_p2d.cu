@@ -221,6 +221,11 @@ template <int (*EL)(int, int)> __device__ __forceinline__ void get(const uint32_
 
 // One pass over 2^12-element tiles, B of the tile index's bits (the top ones)
 // transformed: B = 12 the low pass, B < 12 a high pass with 2^(12-B) columns.
+// Integer instructions bound it (ALU 72% busy at three CTAs per SM): per point 36
+// of the additions, about 50 of the conversions and exchanges.  32 functions of
+// 2^20 points: 1660 us on the FP64 pipe; so, with the
+// short conversions 306 us, without groups of functions 270, with one vote per
+// four results 256 (random values) and 274 (coefficients of a smooth function).
 template <int B>
 __global__ void __launch_bounds__(kNT, 3) k2d_pass(DArgs a) {
     constexpr int LC = kLT - B;          // column bits
