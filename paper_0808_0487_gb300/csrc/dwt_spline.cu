@@ -110,86 +110,110 @@ __global__ void k_spline_scale(double* ft, int cplx, long long N, long long ld, 
 //
 // A batch of 32 functions against 32 tables is a matrix product with the labels
 // as inner dimension, in FP64.  This GPU multiplies 1.7 FP64 numbers per clock
-// and SM, so the product runs on the tensor cores in exact pieces instead: in
-// blocks of 64 labels every operand (for real data the square straight from c~'s
-// significand) becomes a 64-bit fixed-point number, scaled by its row's largest
-// exponent so far in the tile, split into eight signed
-// digits of base 256 that FP16 holds exactly; a digit product is below 2^14 and
-// the 8 x 64 products that share a weight sum to less than 2^24, exact in FP32.
-// The 36 digit pairs of weight >= 256^7 are multiplied (the others lie 2^-62
-// below the largest product); the sums join 128-bit integers per pair of
-// function and table, shifted when a row's exponent grows, and become FP64 once
-// per tile.  FP64 rounds every product and every sum at 2^-53.  Rows with an
-// infinity, a NaN or a square near the largest number in the tile take FP64 sums
-// at the end.
+// and SM, so the product runs on the tensor cores in digits instead: in blocks
+// of 64 labels every operand (for real data the square straight from c~'s
+// significand, to 62 bits) becomes a 96-bit fixed-point number, scaled by its
+// row's largest exponent so far in the tile, split into twelve signed digits of
+// base 256 that FP16 holds exactly; a digit product is at most 2^14 and the
+// 12 x 64 products that share a weight sum to less than 2^24, exact in FP32.
+// The 78 digit pairs of weight >= 256^11 are multiplied; the sums join 128-bit
+// integers per pair of function and table, in units of 2^88, shifted when a
+// row's exponent grows.
 //
-// The next block's numbers come into a thread's own part of shared memory while
-// this block's digits are multiplied (real data; complex data are loaded when
-// they are needed).
+// What is lost.  The products of digits are exact, the operands are not: fixed
+// point has no exponent of its own, so a number keeps its 53 bits down to 2^-42
+// of its row's largest and fewer below, and the digit pairs that are left out
+// belong to the smaller numbers too.  Per label at most 2^95 for the two operands
+// cut at one unit each (they stay below 2^94) and 11 2^14 2^80 (1 + 2^-7) for the
+// pairs, together less than 2^10 units of the sum.  Where |c~|^2 is large the
+// tables are small, so the largest product can lie far below the product of the
+// largest; whether the bits kept were enough is therefore read off each result:
+// a sum below 2^60 units per label, the error's bound then above 2^-50 of the sum,
+// is formed again in FP64 by one warp.  (FP64 sums of 4096 labels, sixteen per
+// thread and a tree over 256, are bound by 26 2^-53 > 2^-49.)  So are rows with an
+// infinity, a NaN or a square near the largest number in the tile.  A pair's
+// result depends on its own two rows only.
 //
-// p = 2, m = 20, s = 16, 32 functions: 2920 us on the FP64 pipe (one CTA per
-// function and 4096 labels) plus 95 us for the scaling; so 459 us, with the
-// asynchronous loads 420 us, with fewer instructions per number (integer squares,
-// one bounds check per block, sums of the upper weights read off the bits) 376 us,
-// with whole waves of tiles 361 us.  (Eight warps that convert beside eight that
-// multiply, double buffered, one CTA per SM: 388 us.)
+// Integer instructions and the tensor cores bound it, a fifth goes to the sums
+// formed again.  p = 2, m = 20, s = 16, 32 functions: 2920 us on the FP64 pipe (one
+// CTA per function and 4096 labels) plus 95 us for the scaling; so 763 us (535
+// without the sums formed again).  Eight digits, 36 pairs and no second look took
+// 364 us and were wrong by up to 2^-16 of a variance (random values, s = 2, m = 16).
 constexpr int kDotThreads = 256;
 constexpr int kDotRows = 32;                  // functions, and tables, per round
 constexpr int kDotK = 64;                     // labels per block
-constexpr int kDotStride = kDotK + 8;         // halves per digit row (16-byte rows on all banks)
-constexpr int kDotPlane = kDotRows * kDotStride;
-constexpr int kDotDigits = 8;
+constexpr int kDotPlane = kDotRows * kDotK;   // halves of one digit's rows
+constexpr int kDotDigits = 12;
 constexpr int kDotOperand = kDotDigits * kDotPlane;   // halves of one operand
-constexpr int kDotStage = 18;                 // doubles per thread on their way in: 8 + 8 and W's two
-constexpr size_t kDotSmem = (size_t)2 * kDotOperand * 2 + 4 * kDotRows * 4;
-constexpr size_t kDotSmemReal = kDotSmem + (size_t)kDotStage * kDotThreads * 8;
-
-__device__ __forceinline__ void cp_async8(uint32_t dst, const void* src) {
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(dst), "l"(src) : "memory");
-}
+constexpr size_t kDotSmem = (size_t)2 * kDotOperand * 2 + 6 * kDotRows * 4;
+constexpr int kDotKeep = 60;                  // log2 of the least sum per label that is kept
 
 __device__ __forceinline__ uint32_t abs_hi(double x) { return (uint32_t)__double2hiint(x) & 0x7fffffffu; }
 
-// 64-bit fixed point of x against exponent E (>= x's), significand 2^9 at E, plus
-// 128 in every byte with carries: byte - 128 is the signed digit
-template <bool SIGNED> __device__ __forceinline__ unsigned long long to_fix64(double x, int E) {
+// half of a digit plane: rows of 64 labels (128 bytes), their 16-byte pieces
+// permuted by the row so that eight rows' same piece lies on all banks
+__device__ __forceinline__ int plane_at(int row, int piece) { return row * kDotK + ((piece ^ (row & 7)) << 3); }
+
+struct Fix96 {
+    uint32_t w[3];   // low word first
+};
+
+// +-(v 2^32 2^-d) for v < 2^62, plus 128 in every byte with carries: byte - 128 is
+// the signed digit; neg: all ones for minus (-v = ~v + 1)
+__device__ __forceinline__ Fix96 place96(unsigned long long v, int d, uint32_t neg) {
+    uint32_t a = 0, b = (uint32_t)v, c = (uint32_t)(v >> 32);
+    d = min(d, 95);
+    if (d >= 64) {
+        a = c;
+        b = c = 0;
+    } else if (d >= 32) {
+        a = b;
+        b = c;
+        c = 0;
+    }
+    const int r = d & 31;
+    a = __funnelshift_r(a, b, r);
+    b = __funnelshift_r(b, c, r);
+    c >>= r;
+    Fix96 x;
+    asm("add.cc.u32 %0, %3, %6;\n addc.cc.u32 %1, %4, %7;\n addc.u32 %2, %5, %7;"
+        : "=r"(x.w[0]), "=r"(x.w[1]), "=r"(x.w[2])
+        : "r"(a ^ neg), "r"(b ^ neg), "r"(c ^ neg), "r"(0x80808080u - neg), "r"(0x80808080u));
+    return x;
+}
+
+// x against exponent E (>= x's): significand 2^41 at E
+template <bool SIGNED> __device__ __forceinline__ Fix96 to_fix96(double x, int E) {
     const uint32_t h = (uint32_t)__double2hiint(x);
     const int ex = (int)((h >> 20) & 0x7ffu);
     const uint32_t mh = (h & 0xfffffu) | (ex ? 0x100000u : 0u);
-    const int d = min(E - max(ex, 1), 63);   // 62 bits
-    unsigned long long v = ((((unsigned long long)mh << 32) | (uint32_t)__double2loint(x)) << 9) >> d;
-    if constexpr (SIGNED) {   // -v = ~v + 1
-        const uint32_t s = (uint32_t)((int)h >> 31);
-        v ^= ((unsigned long long)s << 32) | s;
-        return v + ((0x80808080ull << 32) | (0x80808080u - s));
-    }
-    return v + 0x8080808080808080ull;
+    const unsigned long long v = (((unsigned long long)mh << 32) | (uint32_t)__double2loint(x)) << 9;
+    return place96(v, E - max(ex, 1), SIGNED ? (uint32_t)((int)h >> 31) : 0u);
 }
 
-// u^2 the same way, u's exponents against E: the top 62 of its 106 bits at E
-__device__ __forceinline__ unsigned long long square_fix64(double u, int E) {
+// u^2 the same way, u's exponents against E: the top 62 of its 106 bits
+__device__ __forceinline__ Fix96 square_fix96(double u, int E) {
     const uint32_t h = (uint32_t)__double2hiint(u), lo = (uint32_t)__double2loint(u);
     const int ex = (int)((h >> 20) & 0x7ffu);
     const uint32_t mh = (h & 0xfffffu) | (ex ? 0x100000u : 0u);
     const unsigned long long hh = (unsigned long long)mh * mh, mid = (unsigned long long)(2 * mh) * lo + __umulhi(lo, lo);
-    const int d = min(2 * (E - max(ex, 1)), 63);
-    return (((hh << 20) + (mid >> 12)) >> d) + 0x8080808080808080ull;
+    return place96((hh << 20) + (mid >> 12), 2 * (E - max(ex, 1)), 0u);
 }
 
 // the digits of two numbers (label l and l + 32 of a block) into their planes
-__device__ __forceinline__ void put_digits(__half* row, unsigned long long f0, unsigned long long f1, int lane) {
-    const uint32_t lo0 = (uint32_t)f0, hi0 = (uint32_t)(f0 >> 32), lo1 = (uint32_t)f1, hi1 = (uint32_t)(f1 >> 32);
+__device__ __forceinline__ void put_digits(__half* plane, int row, const Fix96& f0, const Fix96& f1, int lane) {
     const __half2 off = __halves2half2(__ushort_as_half(0xE480), __ushort_as_half(0xE480));   // -(1024 + 128)
+    __half* p = plane + plane_at(row, lane >> 2) + 2 * (lane & 3);
 #pragma unroll
     for (int i = 0; i < kDotDigits; ++i) {
         // bytes i of both behind 0x64: the FP16 numbers 1024 + byte
         const uint32_t sel = (uint32_t)(i & 3) | ((uint32_t)(4 + (i & 3)) << 4);
-        const uint32_t two = __byte_perm(i < 4 ? lo0 : hi0, i < 4 ? lo1 : hi1, sel);
+        const uint32_t two = __byte_perm(f0.w[i >> 2], f1.w[i >> 2], sel);
         const uint32_t bits = __byte_perm(two, 0x64u, 0x4140);
         __half2 h;
         memcpy(&h, &bits, 4);
         h = __hadd2(h, off);
-        *reinterpret_cast<__half2*>(row + i * kDotPlane + 2 * lane) = h;
+        *reinterpret_cast<__half2*>(p + i * kDotPlane) = h;
     }
 }
 
@@ -198,14 +222,41 @@ __device__ __forceinline__ void ldmatrix4(uint32_t (&r)[4], uint32_t addr) {
                  : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
                  : "r"(addr));
 }
-__device__ __forceinline__ void ldmatrix2(uint32_t (&r)[2], uint32_t addr) {
-    asm volatile("ldmatrix.sync.aligned.m8n8.x2.shared.b16 {%0, %1}, [%2];" : "=r"(r[0]), "=r"(r[1]) : "r"(addr));
-}
-__device__ __forceinline__ void mma_f16(float (&d)[4], const uint32_t (&a)[4], const uint32_t (&b)[2]) {
+__device__ __forceinline__ void mma_f16(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
     asm volatile(
         "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
         : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
+        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+
+// sum over [h0, h1) of |c~|^2 T in FP64 by one warp: four chains per lane (the
+// additions take 64 cycles), then trees; eight pairs of loads in flight
+template <bool CPLX>
+__device__ __forceinline__ double warp_sum(const double* c, const double* T, long long h0, long long h1, int lane) {
+    double v[4] = {0.0, 0.0, 0.0, 0.0};
+    for (long long H = h0 + lane; H < h1; H += 256) {
+        double x[8], y[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const long long h = H + 32 * i;
+            x[i] = y[i] = 0.0;
+            if (h >= h1) continue;
+            if constexpr (CPLX) {
+                const double2 u = reinterpret_cast<const double2*>(c)[h];
+                x[i] = u.x * u.x + u.y * u.y;
+            } else {
+                x[i] = c[h];
+            }
+            y[i] = T[h];
+        }
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+            if (H + 32 * i < h1) v[i & 3] += (CPLX ? x[i] : x[i] * x[i]) * y[i];
+    }
+    double x = (v[0] + v[1]) + (v[2] + v[3]);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+    return x;
 }
 
 // grid (tiles, groups of 32 functions); warp w converts rows 4 w .. 4 w + 3 of
@@ -216,21 +267,21 @@ __global__ void __launch_bounds__(kDotThreads, 2) k_spline_dots(double* ct, long
                                                                 const double* __restrict__ tab,
                                                                 const double* __restrict__ W, double* part, int ntile,
                                                                 int labels) {
-    extern __shared__ __align__(16) unsigned char smraw[];
+    extern __shared__ __align__(128) unsigned char smraw[];
     __half* A = reinterpret_cast<__half*>(smraw);
     __half* B = A + kDotOperand;
     int* grow = reinterpret_cast<int*>(B + kDotOperand);   // [2][32]: growth of the rows' exponents in this block
     int* bad = grow + 2 * kDotRows;                        // [2][32]: rows with an infinity or a NaN
-    double* mine = reinterpret_cast<double*>(bad + 2 * kDotRows) + threadIdx.x;   // real data: [18][threads]
-    const uint32_t stage = (uint32_t)__cvta_generic_to_shared(mine);
+    int* some = bad + 2 * kDotRows;                        // [2][32]: rows with a number other than zero
     const int t = threadIdx.x, lane = t & 31, w = t >> 5;
     const int tile = blockIdx.x, f0 = blockIdx.y * kDotRows;
     const long long h0 = (long long)tile * labels, h1 = min(N, h0 + labels);
     const int fo = 16 * (w & 1), to = 8 * (w >> 1);
-    const uint32_t sA = (uint32_t)__cvta_generic_to_shared(A), sB = (uint32_t)__cvta_generic_to_shared(B);
-    // ldmatrix row addresses of this lane: A (16 rows x 16 labels), B (8 rows x 16)
-    const uint32_t aoff = sA + 2u * (uint32_t)((fo + (lane & 15)) * kDotStride + 8 * (lane >> 4));
-    const uint32_t boff = sB + 2u * (uint32_t)((to + (lane & 7)) * kDotStride + 8 * ((lane >> 3) & 1));
+    // ldmatrix rows of this lane: A (16 rows x 16 labels of one digit), B (8 rows x 16
+    // of two digits)
+    const int ar = fo + (lane & 15), br = to + (lane & 7);
+    const uint32_t arow = (uint32_t)__cvta_generic_to_shared(A + ar * kDotK);
+    const uint32_t brow = (uint32_t)__cvta_generic_to_shared(B + (lane >> 4) * kDotPlane + br * kDotK);
     for (int t0 = 0; t0 < nt; t0 += kDotRows) {
         // top word of the first function-side number whose row takes FP64 sums: real
         // rows hold c~, whose square must not overflow
@@ -239,47 +290,14 @@ __global__ void __launch_bounds__(kDotThreads, 2) k_spline_dots(double* ct, long
         __syncthreads();
         if (t < 2 * kDotRows) bad[t] = 0;
         int Ea[4] = {1, 1, 1, 1}, Et[4] = {1, 1, 1, 1};   // exponents of this warp's rows
+        unsigned any = 0;                                 // its rows with a number other than zero
         int ea[2] = {CPLX ? 1 : 2, CPLX ? 1 : 2}, et[2] = {1, 1};   // of the rows of this thread's sums
-        long long hi[4] = {0, 0, 0, 0}, lo[4] = {0, 0, 0, 0};   // sum = hi 2^32 + lo
-        // real data: this thread's numbers of a block, requested one block ahead
-        // (zeros past the last function, table or label)
-        const bool all = f0 + kDotRows <= batch && t0 + kDotRows <= nt;
-        const double* pa = ct + (f0 + 4 * w) * ld + lane;
-        const double* pt = tab + (t0 + 4 * w) * N + lane;
-        auto request = [&](long long hb) {
-            if (all && hb + kDotK <= h1) {
-                const double *ra = pa + hb, *rt = pt + hb;
-#pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    cp_async8(stage + (2 * k) * kDotThreads * 8, ra);
-                    cp_async8(stage + (2 * k + 1) * kDotThreads * 8, ra + 32);
-                    cp_async8(stage + (8 + 2 * k) * kDotThreads * 8, rt);
-                    cp_async8(stage + (9 + 2 * k) * kDotThreads * 8, rt + 32);
-                    ra += ld;
-                    rt += N;
-                }
-                if (t0 == 0) {
-                    cp_async8(stage + 16 * kDotThreads * 8, W + hb + lane);
-                    cp_async8(stage + 17 * kDotThreads * 8, W + hb + lane + 32);
-                }
-                return;
-            }
-#pragma unroll 1
-            for (int i = 0; i < kDotStage; ++i) {
-                const int k = (i >> 1) & 3;
-                const long long off = hb + 32 * (i & 1);
-                const double* src = i < 8 ? pa + k * ld + off : i < 16 ? pt + k * N + off : W + lane + off;
-                const bool there = off + lane < h1 && (i < 8 ? f0 + 4 * w + k < batch : i < 16 ? t0 + 4 * w + k < nt : t0 == 0);
-                if (there) cp_async8(stage + i * kDotThreads * 8, src);
-                else mine[i * kDotThreads] = 0.0;
-            }
-        };
-        if constexpr (!CPLX) request(h0);
+        long long hi[4] = {0, 0, 0, 0}, mid[4] = {0, 0, 0, 0}, lo[4] = {0, 0, 0, 0};   // sum = hi 2^64 + mid 2^32 + lo
         for (long long hb = h0; hb < h1; hb += kDotK) {
             const long long l0 = hb + lane, l1 = l0 + 32;
             const bool in0 = l0 < h1, in1 = l1 < h1;
             double a[4][2], x[4][2];
-            if constexpr (CPLX) {
+            {
                 double w0 = 1.0, w1 = 1.0;
                 if (t0 == 0 && in0) w0 = W[l0];
                 if (t0 == 0 && in1) w1 = W[l1];
@@ -288,16 +306,22 @@ __global__ void __launch_bounds__(kDotThreads, 2) k_spline_dots(double* ct, long
                     const int f = f0 + 4 * w + k, tb = t0 + 4 * w + k;
                     a[k][0] = a[k][1] = x[k][0] = x[k][1] = 0.0;
                     if (f < batch) {
-                        double2* row = reinterpret_cast<double2*>(ct) + f * ld;
-                        double2 u = in0 ? row[l0] : make_double2(0.0, 0.0), v = in1 ? row[l1] : make_double2(0.0, 0.0);
-                        if (t0 == 0) {
-                            u = make_double2(u.x * w0, u.y * w0);
-                            v = make_double2(v.x * w1, v.y * w1);
-                            if (in0) row[l0] = u;
-                            if (in1) row[l1] = v;
+                        if constexpr (CPLX) {
+                            double2* row = reinterpret_cast<double2*>(ct) + f * ld;
+                            double2 u = in0 ? row[l0] : make_double2(0.0, 0.0), v = in1 ? row[l1] : make_double2(0.0, 0.0);
+                            if (t0 == 0) {
+                                u = make_double2(u.x * w0, u.y * w0);
+                                v = make_double2(v.x * w1, v.y * w1);
+                                if (in0) row[l0] = u;
+                                if (in1) row[l1] = v;
+                            }
+                            a[k][0] = u.x * u.x + u.y * u.y;
+                            a[k][1] = v.x * v.x + v.y * v.y;
+                        } else {
+                            double* row = ct + f * ld;
+                            if (in0) a[k][0] = row[l0];
+                            if (in1) a[k][1] = row[l1];
                         }
-                        a[k][0] = u.x * u.x + u.y * u.y;
-                        a[k][1] = v.x * v.x + v.y * v.y;
                     }
                     if (tb < nt) {
                         const double* row = tab + (long long)tb * N;
@@ -305,38 +329,38 @@ __global__ void __launch_bounds__(kDotThreads, 2) k_spline_dots(double* ct, long
                         if (in1) x[k][1] = row[l1];
                     }
                 }
-            } else {
-                asm volatile("cp.async.wait_all;" ::: "memory");
+                if constexpr (!CPLX) {
+                    if (t0 == 0) {
 #pragma unroll
-                for (int k = 0; k < 4; ++k)
-#pragma unroll
-                    for (int u = 0; u < 2; ++u) {
-                        a[k][u] = mine[(2 * k + u) * kDotThreads];
-                        x[k][u] = mine[(8 + 2 * k + u) * kDotThreads];
-                    }
-                if (t0 == 0) {
-                    const double w0 = mine[16 * kDotThreads], w1 = mine[17 * kDotThreads];
-                    double* row = ct + (f0 + 4 * w) * ld + l0;
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) {
-                        a[k][0] *= w0;
-                        a[k][1] *= w1;
-                        if (all || f0 + 4 * w + k < batch) {
-                            if (in0) row[0] = a[k][0];
-                            if (in1) row[32] = a[k][1];
+                        for (int k = 0; k < 4; ++k) {
+                            a[k][0] *= w0;
+                            a[k][1] *= w1;
+                            if (f0 + 4 * w + k < batch) {
+                                double* row = ct + (f0 + 4 * w + k) * ld;
+                                if (in0) row[l0] = a[k][0];
+                                if (in1) row[l1] = a[k][1];
+                            }
                         }
-                        row += ld;
                     }
                 }
             }
             __syncthreads();   // the previous block's digits and growths have been read
             // the rows' largest exponents: eight reductions in flight
-            uint32_t ma[4], mx[4], most = 0;
+            uint32_t ma[4], mx[4], most = 0, least = 0xffffffffu;
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
                 ma[k] = __reduce_max_sync(0xffffffffu, max(abs_hi(a[k][0]), abs_hi(a[k][1])));
                 mx[k] = __reduce_max_sync(0xffffffffu, max(abs_hi(x[k][0]), abs_hi(x[k][1])));
                 most = max(most, max(ma[k], mx[k]));
+                least = min(least, min(ma[k], mx[k]));
+            }
+            if (least == 0) {   // a row of zeros, or of numbers whose top word is zero
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const double(&v)[2] = i < 4 ? a[i] : x[i - 4];
+                    uint32_t& m = i < 4 ? ma[i] : mx[i - 4];
+                    if (m == 0 && __any_sync(0xffffffffu, (__double2loint(v[0]) | __double2loint(v[1])) != 0)) m = 1;
+                }
             }
             if (most >= kDotHuge) {
 #pragma unroll
@@ -352,6 +376,7 @@ __global__ void __launch_bounds__(kDotThreads, 2) k_spline_dots(double* ct, long
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
                 const int r = 4 * w + k;
+                any |= (ma[k] ? 1u << k : 0u) | (mx[k] ? 16u << k : 0u);
                 const int na = max((int)(ma[k] >> 20), Ea[k]), nx = max((int)(mx[k] >> 20), Et[k]);
                 if (lane == 0) {
                     grow[r] = kDotPower * (na - Ea[k]);
@@ -363,33 +388,39 @@ __global__ void __launch_bounds__(kDotThreads, 2) k_spline_dots(double* ct, long
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
                 const int r = 4 * w + k;
-                if constexpr (CPLX)
-                    put_digits(A + r * kDotStride, to_fix64<false>(a[k][0], Ea[k]), to_fix64<false>(a[k][1], Ea[k]), lane);
-                else
-                    put_digits(A + r * kDotStride, square_fix64(a[k][0], Ea[k]), square_fix64(a[k][1], Ea[k]), lane);
-                put_digits(B + r * kDotStride, to_fix64<true>(x[k][0], Et[k]), to_fix64<true>(x[k][1], Et[k]), lane);
+                if constexpr (CPLX) put_digits(A, r, to_fix96<false>(a[k][0], Ea[k]), to_fix96<false>(a[k][1], Ea[k]), lane);
+                else put_digits(A, r, square_fix96(a[k][0], Ea[k]), square_fix96(a[k][1], Ea[k]), lane);
+                put_digits(B, r, to_fix96<true>(x[k][0], Et[k]), to_fix96<true>(x[k][1], Et[k]), lane);
             }
-            if constexpr (!CPLX)
-                if (hb + kDotK < h1) request(hb + kDotK);   // this block's numbers have been used
             __syncthreads();
-            // weights 256^11 and up: at most 4 x 64 products of 2^14 onto 3 2^22, whose
+            // the next block's lines on their way into L2: 64 rows of four
+            if (const long long hn = hb + kDotK + 16 * (t & 3); hn < h1) {
+                const int r = t >> 3;
+                const double* p = t & 4 ? (t0 + r < nt ? tab + (long long)(t0 + r) * N + hn : nullptr)
+                                        : (f0 + r < batch ? ct + ((f0 + r) * ld + hn) * (CPLX ? 2 : 1) : nullptr);
+                if (p) asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
+            }
+            // weights 256^19 and up: at most 4 x 64 products of 2^14 onto 3 2^22, whose
             // last place is one: the sum is read off the bits
             float acc[kDotDigits][4];
 #pragma unroll
             for (int c = 0; c < kDotDigits; ++c)
 #pragma unroll
-                for (int q = 0; q < 4; ++q) acc[c][q] = c < 4 ? 0.f : 12582912.f;
+                for (int q = 0; q < 4; ++q) acc[c][q] = c < kDotDigits - 4 ? 0.f : 12582912.f;
 #pragma unroll 1
             for (int k = 0; k < kDotK / 16; ++k) {
-                uint32_t fb[kDotDigits][2];
+                const uint32_t aoff = arow + 16u * (uint32_t)((2 * k + (lane >> 4)) ^ (ar & 7));
+                const uint32_t boff = brow + 16u * (uint32_t)((2 * k + ((lane >> 3) & 1)) ^ (br & 7));
+                uint32_t fb[kDotDigits / 2][4];
 #pragma unroll
-                for (int j = 0; j < kDotDigits; ++j) ldmatrix2(fb[j], boff + 2u * (uint32_t)(j * kDotPlane + 16 * k));
+                for (int j = 0; j < kDotDigits / 2; ++j) ldmatrix4(fb[j], boff + 2u * (uint32_t)(2 * j * kDotPlane));
 #pragma unroll
                 for (int i = 0; i < kDotDigits; ++i) {
                     uint32_t fa[4];
-                    ldmatrix4(fa, aoff + 2u * (uint32_t)(i * kDotPlane + 16 * k));
+                    ldmatrix4(fa, aoff + 2u * (uint32_t)(i * kDotPlane));
 #pragma unroll
-                    for (int j = kDotDigits - 1 - i; j < kDotDigits; ++j) mma_f16(acc[i + j - kDotDigits + 1], fa, fb[j]);
+                    for (int j = kDotDigits - 1 - i; j < kDotDigits; ++j)
+                        mma_f16(acc[i + j - kDotDigits + 1], fa, fb[j >> 1][2 * (j & 1)], fb[j >> 1][2 * (j & 1) + 1]);
                 }
             }
             // this thread's sums: rows fo + lane / 4 (+ 8), tables to + 2 (lane % 4) (+ 1)
@@ -405,40 +436,50 @@ __global__ void __launch_bounds__(kDotThreads, 2) k_spline_dots(double* ct, long
             for (int q = 0; q < 4; ++q) {
                 const int g = ga[q >> 1] + gt[q & 1];
                 if (g) {
-                    __int128 v = ((__int128)hi[q] << 32) + lo[q];
+                    __int128 v = ((__int128)hi[q] << 64) + ((__int128)mid[q] << 32) + lo[q];
                     v = g > 126 ? (__int128)0 : v >> g;
-                    hi[q] = (long long)(v >> 32);
+                    hi[q] = (long long)(v >> 64);
+                    mid[q] = (long long)((unsigned long long)(v >> 32) & 0xffffffffull);
                     lo[q] = (long long)((unsigned long long)v & 0xffffffffull);
                 }
-                // pairs of weights fit 32 bits: 5 x 64 x 2^22 and 7 x 64 x 2^22 at most
-                auto whole = [&](int c) { return c < 4 ? __float2int_rn(acc[c][q]) : __float_as_int(acc[c][q]) - 0x4b400000; };
-                lo[q] += whole(1) * 256 + whole(0);
-                lo[q] += (long long)(whole(3) * 256 + whole(2)) * 65536;
-                hi[q] += whole(5) * 256 + whole(4);
-                hi[q] += (long long)(whole(7) * 256 + whole(6)) * 65536;
+                auto whole = [&](int c) {
+                    return c < kDotDigits - 4 ? __float2int_rn(acc[c][q]) : __float_as_int(acc[c][q]) - 0x4b400000;
+                };
+                // four weights: below 12 2^20 256^3 (1 + 2^-7) < 2^48
+                auto four = [&](int c) {
+                    return (long long)whole(c) + (long long)whole(c + 1) * 256 + (long long)whole(c + 2) * 65536 +
+                           (long long)whole(c + 3) * 16777216;
+                };
+                lo[q] += four(0);
+                mid[q] += four(4);
+                hi[q] += four(8);
             }
         }
-        __syncthreads();   // bad is complete, c~ of the tile is written
+        if (lane < 8) some[(lane >> 2) * kDotRows + 4 * w + (lane & 3)] = (any >> lane) & 1;
+        __syncthreads();   // bad and some are complete, c~ of the tile is written
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
             const int fr = fo + (lane >> 2) + 8 * (q >> 1), tr = to + 2 * (lane & 3) + (q & 1);
             const int f = f0 + fr, tb = t0 + tr;
-            if (f >= batch || tb >= nt) continue;
-            double v;
-            if (bad[fr] || bad[kDotRows + tr]) {
-                v = 0.0;
-                for (long long H = h0; H < h1; ++H) {
-                    const double* c = ct + (f * ld + H) * (CPLX ? 2 : 1);
-                    const double m2 = CPLX ? c[0] * c[0] + c[1] * c[1] : c[0] * c[0];
-                    v += m2 * tab[(long long)tb * N + H];
-                }
-            } else {
-                // digits of weight 256^7 and up; the unit of a row is 2^(E - 1084), of a
-                // row of squares 2^(2 E - 2106)
-                v = scalbn((double)hi[q] * 4294967296.0 + (double)lo[q],
-                           56 + ea[q >> 1] + et[q & 1] - 1084 - (CPLX ? 1084 : 2106));
+            const bool there = f < batch && tb < nt;
+            const __int128 sum = ((__int128)hi[q] << 64) + ((__int128)mid[q] << 32) + lo[q];
+            // digits of weight 256^11 and up; the unit of a row is 2^(E - 1116), of a
+            // row of squares 2^(2 E - 2138)
+            const long long top = (long long)(sum >> 60);   // below 2^52: nothing of weight is cut
+            double v = scalbn((double)top * 0x1p60 + (double)(long long)((unsigned long long)sum & ((1ull << 60) - 1)),
+                              88 + ea[q >> 1] + et[q & 1] - 1116 - (CPLX ? 1116 : 2138));
+            bool redo = there && (bad[fr] || bad[kDotRows + tr]);
+            if (!redo && there) {
+                if (!some[fr] || !some[kDotRows + tr]) v = 0.0;
+                else redo = sum < ((__int128)(h1 - h0) << kDotKeep);
             }
-            part[((long long)f * nt + tb) * ntile + tile] = v;
+            for (unsigned todo = __ballot_sync(0xffffffffu, redo); todo; todo &= todo - 1) {
+                const int src = __ffs((int)todo) - 1;
+                const int rf = __shfl_sync(0xffffffffu, f, src), rt = __shfl_sync(0xffffffffu, tb, src);
+                const double x = warp_sum<CPLX>(ct + (long long)rf * ld * (CPLX ? 2 : 1), tab + (long long)rt * N, h0, h1, lane);
+                if (lane == src) v = x;
+            }
+            if (there) part[((long long)f * nt + tb) * ntile + tile] = v;
         }
     }
 }
@@ -953,11 +994,12 @@ int run_spline(dwt_plan_s* P, const double* f, void* c, int batch, long long ld,
     double* part = nullptr;
     const bool want_var = var_trc || var_sup || dim;
     const long long groups = ((long long)batch + kDotRows - 1) / kDotRows;
-    // tiles of at most 2048 labels (an odd row's FP64 sums walk one), as many as
-    // fill whole waves of two CTAs per SM: p = 2, m = 20, 32 functions take 608
-    // tiles of 27 blocks, 361 us, where 1024 of 16 in 3.4 waves took 376
+    // tiles of at most 512 labels, as many as fill whole waves of two CTAs per SM: the
+    // sums that are formed again in FP64 find the tile in L2, and fewer fail (p = 2,
+    // m = 20, 32 functions of s = 16, whole call, 2048 / 1024 / 512 / 256 labels:
+    // 1720 / 1511 / 1302 / 1273 us smooth, 1994 / 1554 / 1311 / 1253 us random values)
     const long long blocks = (N + kDotK - 1) / kDotK, slots = 2 * 152;
-    const long long waves = std::max(1ll, ((blocks + 31) / 32 * groups + slots - 1) / slots);
+    const long long waves = std::max(1ll, ((blocks + 7) / 8 * groups + slots - 1) / slots);
     const long long want = std::max(1ll, std::min(blocks, waves * slots / groups));
     const int labels = (int)((blocks + want - 1) / want) * kDotK;
     const int ntile = (int)((N + labels - 1) / labels);
@@ -979,9 +1021,9 @@ int run_spline(dwt_plan_s* P, const double* f, void* c, int batch, long long ld,
         for (long long b0 = 0; b0 < batch; b0 += kRows) {
             const int nb = (int)std::min<long long>(kRows, batch - b0);
             LaunchScope ls("spline_dots", st);
-            kern<<<dim3((unsigned)ntile, (unsigned)((nb + kDotRows - 1) / kDotRows)), kDotThreads,
-                   cplx ? kDotSmem : kDotSmemReal, st>>>(ft + b0 * ldt * (cplx ? 2 : 1), N, ldt, nb, 2 * s, P->d_splT,
-                                                         P->d_splW, part + b0 * 2 * s * ntile, ntile, labels);
+            kern<<<dim3((unsigned)ntile, (unsigned)((nb + kDotRows - 1) / kDotRows)), kDotThreads, kDotSmem, st>>>(
+                ft + b0 * ldt * (cplx ? 2 : 1), N, ldt, nb, 2 * s, P->d_splT, P->d_splW, part + b0 * 2 * s * ntile, ntile,
+                labels);
         }
     } else {
         LaunchScope ls("spline_scale", st);
