@@ -311,6 +311,10 @@ int dwt_interpolate_host(dwt_plan_t plan, const void *f, void *c, int batch, lon
  * c~ = f~ W_K divides by K~, which is small at high H: the coefficients are as
  * well conditioned as that quotient (relative error about
  * 1e-16 max|K(x_n, 0)| / min|K~|).  DWT_EINVAL without dwt_spline_prepare.
+ * The variances' sums run in FP64 for few functions or dimensions and in exact
+ * digit products (checked, and formed again in FP64 where those do not carry
+ * them) for many: a function's variances may differ in their last bits between
+ * calls of different batch.
  * No counterpart in the paper for the superposition route: the degree-j
  * tables come from the elementary symmetric polynomials of the per-coordinate
  * terms instead of the interpolation in beta^2 of Sec. 4 (same quantities).

@@ -121,7 +121,7 @@ __global__ void k_spline_scale(double* ft, int cplx, long long N, long long ld, 
 // row's exponent grows.
 //
 // What is lost.  The products of digits are exact, the operands are not: fixed
-// point has no exponent of its own, so a number keeps its 53 bits down to 2^-42
+// point has no exponent of its own, so a number keeps its 53 bits down to 2^-41
 // of its row's largest and fewer below, and the digit pairs that are left out
 // belong to the smaller numbers too.  Per label at most 2^95 for the two operands
 // cut at one unit each (they stay below 2^94) and 11 2^14 2^80 (1 + 2^-7) for the
@@ -136,8 +136,8 @@ __global__ void k_spline_scale(double* ft, int cplx, long long N, long long ld, 
 //
 // Integer instructions and the tensor cores bound it, a fifth goes to the sums
 // formed again.  p = 2, m = 20, s = 16, 32 functions: 2920 us on the FP64 pipe (one
-// CTA per function and 4096 labels) plus 95 us for the scaling; so 763 us (535
-// without the sums formed again).  Eight digits, 36 pairs and no second look took
+// CTA per function and 4096 labels) plus 95 us for the scaling; so 654 us
+// (535 without the sums formed again; 763 with every warp forming its own again).  Eight digits, 36 pairs and no second look took
 // 364 us and were wrong by up to 2^-16 of a variance (random values, s = 2, m = 16).
 constexpr int kDotThreads = 256;
 constexpr int kDotRows = 32;                  // functions, and tables, per round
@@ -145,7 +145,7 @@ constexpr int kDotK = 64;                     // labels per block
 constexpr int kDotPlane = kDotRows * kDotK;   // halves of one digit's rows
 constexpr int kDotDigits = 12;
 constexpr int kDotOperand = kDotDigits * kDotPlane;   // halves of one operand
-constexpr size_t kDotSmem = (size_t)2 * kDotOperand * 2 + 6 * kDotRows * 4;
+constexpr size_t kDotSmem = (size_t)2 * kDotOperand * 2 + 6 * kDotRows * 4 + 16;
 constexpr int kDotKeep = 60;                  // log2 of the least sum per label that is kept
 
 __device__ __forceinline__ uint32_t abs_hi(double x) { return (uint32_t)__double2hiint(x) & 0x7fffffffu; }
@@ -273,6 +273,7 @@ __global__ void __launch_bounds__(kDotThreads, 2) k_spline_dots(double* ct, long
     int* grow = reinterpret_cast<int*>(B + kDotOperand);   // [2][32]: growth of the rows' exponents in this block
     int* bad = grow + 2 * kDotRows;                        // [2][32]: rows with an infinity or a NaN
     int* some = bad + 2 * kDotRows;                        // [2][32]: rows with a number other than zero
+    int* again = some + 2 * kDotRows;                      // sums to form again
     const int t = threadIdx.x, lane = t & 31, w = t >> 5;
     const int tile = blockIdx.x, f0 = blockIdx.y * kDotRows;
     const long long h0 = (long long)tile * labels, h1 = min(N, h0 + labels);
@@ -456,31 +457,82 @@ __global__ void __launch_bounds__(kDotThreads, 2) k_spline_dots(double* ct, long
             }
         }
         if (lane < 8) some[(lane >> 2) * kDotRows + 4 * w + (lane & 3)] = (any >> lane) & 1;
+        if (t == 0) *again = 0;
         __syncthreads();   // bad and some are complete, c~ of the tile is written
+        uint16_t* list = reinterpret_cast<uint16_t*>(smraw);   // pairs to form again, in the digits' place
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
             const int fr = fo + (lane >> 2) + 8 * (q >> 1), tr = to + 2 * (lane & 3) + (q & 1);
             const int f = f0 + fr, tb = t0 + tr;
-            const bool there = f < batch && tb < nt;
+            if (f >= batch || tb >= nt) continue;
             const __int128 sum = ((__int128)hi[q] << 64) + ((__int128)mid[q] << 32) + lo[q];
             // digits of weight 256^11 and up; the unit of a row is 2^(E - 1116), of a
             // row of squares 2^(2 E - 2138)
             const long long top = (long long)(sum >> 60);   // below 2^52: nothing of weight is cut
             double v = scalbn((double)top * 0x1p60 + (double)(long long)((unsigned long long)sum & ((1ull << 60) - 1)),
                               88 + ea[q >> 1] + et[q & 1] - 1116 - (CPLX ? 1116 : 2138));
-            bool redo = there && (bad[fr] || bad[kDotRows + tr]);
-            if (!redo && there) {
+            bool redo = bad[fr] || bad[kDotRows + tr];
+            if (!redo) {
                 if (!some[fr] || !some[kDotRows + tr]) v = 0.0;
                 else redo = sum < ((__int128)(h1 - h0) << kDotKeep);
             }
-            for (unsigned todo = __ballot_sync(0xffffffffu, redo); todo; todo &= todo - 1) {
-                const int src = __ffs((int)todo) - 1;
-                const int rf = __shfl_sync(0xffffffffu, f, src), rt = __shfl_sync(0xffffffffu, tb, src);
-                const double x = warp_sum<CPLX>(ct + (long long)rf * ld * (CPLX ? 2 : 1), tab + (long long)rt * N, h0, h1, lane);
-                if (lane == src) v = x;
-            }
-            if (there) part[((long long)f * nt + tb) * ntile + tile] = v;
+            if (redo) list[atomicAdd(again, 1)] = (uint16_t)(fr * kDotRows + tr);
+            else part[((long long)f * nt + tb) * ntile + tile] = v;
         }
+        __syncthreads();
+        for (int i = w; i < *again; i += kDotThreads / 32) {
+            const int f = f0 + list[i] / kDotRows, tb = t0 + list[i] % kDotRows;
+            const double v = warp_sum<CPLX>(ct + (long long)f * ld * (CPLX ? 2 : 1), tab + (long long)tb * N, h0, h1, lane);
+            if (lane == 0) part[((long long)f * nt + tb) * ntile + tile] = v;
+        }
+    }
+}
+
+// The same sums in FP64, for few functions or tables: a CTA scales one function's
+// part of c~, keeps the squares in shared memory, and its warps take the tables in
+// turn.  The FP64 pipe bounds it (an addition of a warp every 19 cycles per SM):
+// p = 2, m = 20, one function, 4 / 32 / 128 tables: 20 / 91 / 329 us.
+constexpr int kFewThreads = 256;
+constexpr int kFewTile = 2048;   // labels per CTA at most
+
+template <bool CPLX>
+__global__ void __launch_bounds__(kFewThreads) k_spline_dots_fp64(double* ct, long long N, long long ld, int nt,
+                                                                  const double* __restrict__ tab,
+                                                                  const double* __restrict__ W, double* part, int ntile,
+                                                                  int labels, long long b0) {
+    __shared__ double a[kFewTile];
+    const long long b = b0 + blockIdx.y, h0 = (long long)blockIdx.x * labels;
+    const int n = (int)min((long long)labels, N - h0), t = threadIdx.x, lane = t & 31;
+    double* c = ct + b * ld * (CPLX ? 2 : 1);
+    for (int i = t; i < n; i += kFewThreads) {
+        const double w = W[h0 + i];
+        if constexpr (CPLX) {
+            double2* p = reinterpret_cast<double2*>(c) + h0 + i;
+            const double2 u = make_double2(p->x * w, p->y * w);
+            *p = u;
+            a[i] = u.x * u.x + u.y * u.y;
+        } else {
+            const double u = c[h0 + i] * w;
+            c[h0 + i] = u;
+            a[i] = u * u;
+        }
+    }
+    __syncthreads();
+    for (int tb = t >> 5; tb < nt; tb += kFewThreads / 32) {
+        const double* T = tab + (long long)tb * N + h0;
+        double v[4] = {0.0, 0.0, 0.0, 0.0};
+        for (int i0 = lane; i0 < n; i0 += 256) {   // eight loads in flight
+            double x[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) x[k] = i0 + 32 * k < n ? T[i0 + 32 * k] : 0.0;
+#pragma unroll
+            for (int k = 0; k < 8; ++k)
+                if (i0 + 32 * k < n) v[k & 3] += a[i0 + 32 * k] * x[k];
+        }
+        double x = (v[0] + v[1]) + (v[2] + v[3]);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+        if (lane == 0) part[(b * nt + tb) * ntile + blockIdx.x] = x;
     }
 }
 
@@ -993,15 +1045,27 @@ int run_spline(dwt_plan_s* P, const double* f, void* c, int batch, long long ld,
     const long long ldt = own ? N : ld;
     double* part = nullptr;
     const bool want_var = var_trc || var_sup || dim;
-    const long long groups = ((long long)batch + kDotRows - 1) / kDotRows;
-    // tiles of at most 512 labels, as many as fill whole waves of two CTAs per SM: the
-    // sums that are formed again in FP64 find the tile in L2, and fewer fail (p = 2,
-    // m = 20, 32 functions of s = 16, whole call, 2048 / 1024 / 512 / 256 labels:
-    // 1720 / 1511 / 1302 / 1273 us smooth, 1994 / 1554 / 1311 / 1253 us random values)
-    const long long blocks = (N + kDotK - 1) / kDotK, slots = 2 * 152;
-    const long long waves = std::max(1ll, ((blocks + 7) / 8 * groups + slots - 1) / slots);
-    const long long want = std::max(1ll, std::min(blocks, waves * slots / groups));
-    const int labels = (int)((blocks + want - 1) / want) * kDotK;
+    const long long groups = ((long long)batch + kDotRows - 1) / kDotRows, rounds = (2 * s + kDotRows - 1) / kDotRows;
+    // a round of up to 32 functions and 32 tables costs as much in digits as 300 pairs
+    // in FP64 (2^20 points, contraction: 9 x 32 pairs 621 us in FP64, 10 x 32 591 us in
+    // digits; 30 x 10 722, 32 x 10 676; 2^16 points 79 and 54 us; 3^12 344 and 406);
+    // with fewer the FP64 form is faster (1 x 4 pairs 20 us, 361 us before in digits)
+    const bool few = (long long)batch * 2 * s <= 300 * groups * rounds;
+    int labels;
+    if (few) {
+        // tiles for two CTAs per SM of one function, of 256 labels at least
+        const long long want = (N + P->min_tiles - 1) / P->min_tiles;
+        labels = (int)std::min<long long>(kFewTile, std::max(256ll, (want + 255) / 256 * 256));
+    } else {
+        // tiles of at most 512 labels, as many as fill whole waves of two CTAs per SM: the
+        // sums that are formed again in FP64 find the tile in L2, and fewer fail (p = 2,
+        // m = 20, 32 functions of s = 16, whole call, 2048 / 1024 / 512 / 256 labels:
+        // 1720 / 1511 / 1302 / 1273 us smooth, 1994 / 1554 / 1311 / 1253 us random values)
+        const long long blocks = (N + kDotK - 1) / kDotK, slots = 2 * 152;
+        const long long waves = std::max(1ll, ((blocks + 7) / 8 * groups + slots - 1) / slots);
+        const long long want = std::max(1ll, std::min(blocks, waves * slots / groups));
+        labels = (int)((blocks + want - 1) / want) * kDotK;
+    }
     const int ntile = (int)((N + labels - 1) / labels);
     if ((own && dmalloc((void**)&ft, (size_t)batch * N * eb, st)) ||
         (want_var && dmalloc((void**)&part, (size_t)batch * 2 * s * ntile * 8, st))) {
@@ -1014,7 +1078,14 @@ int run_spline(dwt_plan_s* P, const double* f, void* c, int batch, long long ld,
     };
     int rc = run_transform(P, f, ft, batch, ld, ldt, DWT_F64, cplx ? DWT_C128 : DWT_F64, -1, st);
     if (rc) { cleanup(); return rc; }
-    if (want_var) {
+    if (want_var && few) {
+        auto kern = cplx ? k_spline_dots_fp64<true> : k_spline_dots_fp64<false>;
+        for (int b0 = 0; b0 < batch; b0 += 65535) {
+            LaunchScope ls("spline_dots_fp64", st);
+            kern<<<dim3((unsigned)ntile, (unsigned)std::min(65535, batch - b0)), kFewThreads, 0, st>>>(
+                ft, N, ldt, 2 * s, P->d_splT, P->d_splW, part, ntile, labels, b0);
+        }
+    } else if (want_var) {
         auto kern = cplx ? k_spline_dots<true> : k_spline_dots<false>;
         if ((rc = smem_limit_max(kern))) { cleanup(); return rc; }
         constexpr int kRows = 65535 * kDotRows;   // functions of one grid
