@@ -314,7 +314,8 @@ int dwt_interpolate_host(dwt_plan_t plan, const void *f, void *c, int batch, lon
  * The variances' sums run in FP64 for few functions or dimensions and in exact
  * digit products (checked, and formed again in FP64 where those do not carry
  * them) for many: a function's variances may differ in their last bits between
- * calls of different batch.
+ * a call with few functions and one with many, but do not depend on the others
+ * of its call otherwise.
  * No counterpart in the paper for the superposition route: the degree-j
  * tables come from the elementary symmetric polynomials of the per-coordinate
  * terms instead of the interpolation in beta^2 of Sec. 4 (same quantities).

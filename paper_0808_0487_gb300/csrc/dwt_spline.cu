@@ -136,8 +136,9 @@ __global__ void k_spline_scale(double* ft, int cplx, long long N, long long ld, 
 //
 // Integer instructions and the tensor cores bound it, a fifth goes to the sums
 // formed again.  p = 2, m = 20, s = 16, 32 functions: 2920 us on the FP64 pipe (one
-// CTA per function and 4096 labels) plus 95 us for the scaling; so 654 us
-// (535 without the sums formed again; 763 with every warp forming its own again).  Eight digits, 36 pairs and no second look took
+// CTA per function and 4096 labels) plus 95 us for the scaling; so 623 us
+// (535 without the sums formed again; with every warp forming its own again, in
+// tiles of 512 labels, 763).  Eight digits, 36 pairs and no second look took
 // 364 us and were wrong by up to 2^-16 of a variance (random values, s = 2, m = 16).
 constexpr int kDotThreads = 256;
 constexpr int kDotRows = 32;                  // functions, and tables, per round
@@ -499,9 +500,9 @@ template <bool CPLX>
 __global__ void __launch_bounds__(kFewThreads) k_spline_dots_fp64(double* ct, long long N, long long ld, int nt,
                                                                   const double* __restrict__ tab,
                                                                   const double* __restrict__ W, double* part, int ntile,
-                                                                  int labels, long long b0) {
+                                                                  int labels) {
     __shared__ double a[kFewTile];
-    const long long b = b0 + blockIdx.y, h0 = (long long)blockIdx.x * labels;
+    const long long b = blockIdx.y, h0 = (long long)blockIdx.x * labels;
     const int n = (int)min((long long)labels, N - h0), t = threadIdx.x, lane = t & 31;
     double* c = ct + b * ld * (CPLX ? 2 : 1);
     for (int i = t; i < n; i += kFewThreads) {
@@ -1051,24 +1052,23 @@ int run_spline(dwt_plan_s* P, const double* f, void* c, int batch, long long ld,
     // digits; 30 x 10 722, 32 x 10 676; 2^16 points 79 and 54 us; 3^12 344 and 406);
     // with fewer the FP64 form is faster (1 x 4 pairs 20 us, 361 us before in digits)
     const bool few = (long long)batch * 2 * s <= 300 * groups * rounds;
-    int labels;
-    if (few) {
-        // tiles for two CTAs per SM of one function, of 256 labels at least
-        const long long want = (N + P->min_tiles - 1) / P->min_tiles;
-        labels = (int)std::min<long long>(kFewTile, std::max(256ll, (want + 255) / 256 * 256));
-    } else {
-        // tiles of at most 512 labels, as many as fill whole waves of two CTAs per SM: the
-        // sums that are formed again in FP64 find the tile in L2, and fewer fail (p = 2,
-        // m = 20, 32 functions of s = 16, whole call, 2048 / 1024 / 512 / 256 labels:
-        // 1720 / 1511 / 1302 / 1273 us smooth, 1994 / 1554 / 1311 / 1253 us random values)
-        const long long blocks = (N + kDotK - 1) / kDotK, slots = 2 * 152;
-        const long long waves = std::max(1ll, ((blocks + 7) / 8 * groups + slots - 1) / slots);
-        const long long want = std::max(1ll, std::min(blocks, waves * slots / groups));
-        labels = (int)((blocks + want - 1) / want) * kDotK;
-    }
+    // labels per tile, from the net alone: a function's sums do not depend on the
+    // others of its call.  Tiles for two CTAs per SM of one group; in digits at most
+    // 256 labels (the sums that are formed again in FP64 find the tile in L2, fewer
+    // fail and no SM is left with a long list: p = 2, 32 functions of s = 16,
+    // contraction of smooth functions, 2048 / 1024 / 512 / 256 labels: m = 20
+    // 880 / 744 / 651 / 623 us, m = 18 - / 286 / 221 / 174, random values 1418 / 878 /
+    // 707 / 638 and - / 509 / 368 / 267) or 16 s, so that the tiles' sums take a byte
+    // per point at most; in FP64 between 256 and 2048
+    long long labels = (N + P->min_tiles - 1) / P->min_tiles;
+    if (few) labels = std::min<long long>(kFewTile, std::max(256ll, (labels + 255) / 256 * 256));
+    else labels = std::min<long long>(std::max(256, s / 4 * kDotK), (labels + kDotK - 1) / kDotK * kDotK);
     const int ntile = (int)((N + labels - 1) / labels);
+    // functions per launch: the tiles' sums within 512 MB, one group of 32 at least
+    const long long most = std::max(1ll, (64ll << 20) / ((long long)2 * s * ntile * kDotRows)) * kDotRows;
+    const int chunk = (int)std::min<long long>(batch, std::min(most, few ? 65504ll : 65535ll * kDotRows));
     if ((own && dmalloc((void**)&ft, (size_t)batch * N * eb, st)) ||
-        (want_var && dmalloc((void**)&part, (size_t)batch * 2 * s * ntile * 8, st))) {
+        (want_var && dmalloc((void**)&part, (size_t)chunk * 2 * s * ntile * 8, st))) {
         if (own) dfree(ft, st);
         return DWT_ENOMEM;
     }
@@ -1078,40 +1078,41 @@ int run_spline(dwt_plan_s* P, const double* f, void* c, int batch, long long ld,
     };
     int rc = run_transform(P, f, ft, batch, ld, ldt, DWT_F64, cplx ? DWT_C128 : DWT_F64, -1, st);
     if (rc) { cleanup(); return rc; }
-    if (want_var && few) {
-        auto kern = cplx ? k_spline_dots_fp64<true> : k_spline_dots_fp64<false>;
-        for (int b0 = 0; b0 < batch; b0 += 65535) {
-            LaunchScope ls("spline_dots_fp64", st);
-            kern<<<dim3((unsigned)ntile, (unsigned)std::min(65535, batch - b0)), kFewThreads, 0, st>>>(
-                ft, N, ldt, 2 * s, P->d_splT, P->d_splW, part, ntile, labels, b0);
-        }
-    } else if (want_var) {
+    if (want_var) {
         auto kern = cplx ? k_spline_dots<true> : k_spline_dots<false>;
+        auto kern64 = cplx ? k_spline_dots_fp64<true> : k_spline_dots_fp64<false>;
         if ((rc = smem_limit_max(kern))) { cleanup(); return rc; }
-        constexpr int kRows = 65535 * kDotRows;   // functions of one grid
-        for (long long b0 = 0; b0 < batch; b0 += kRows) {
-            const int nb = (int)std::min<long long>(kRows, batch - b0);
-            LaunchScope ls("spline_dots", st);
-            kern<<<dim3((unsigned)ntile, (unsigned)((nb + kDotRows - 1) / kDotRows)), kDotThreads, kDotSmem, st>>>(
-                ft + b0 * ldt * (cplx ? 2 : 1), N, ldt, nb, 2 * s, P->d_splT, P->d_splW, part + b0 * 2 * s * ntile, ntile,
-                labels);
+        const int lg = sum_rows_lanes(2 * s, ntile, kFinThreads);
+        for (long long b0 = 0; b0 < batch; b0 += chunk) {
+            const int nb = (int)std::min<long long>(chunk, batch - b0);
+            double* rows0 = ft + b0 * ldt * (cplx ? 2 : 1);
+            if (few) {
+                LaunchScope ls("spline_dots_fp64", st);
+                kern64<<<dim3((unsigned)ntile, (unsigned)nb), kFewThreads, 0, st>>>(rows0, N, ldt, 2 * s, P->d_splT,
+                                                                                    P->d_splW, part, ntile, (int)labels);
+            } else {
+                LaunchScope ls("spline_dots", st);
+                kern<<<dim3((unsigned)ntile, (unsigned)((nb + kDotRows - 1) / kDotRows)), kDotThreads, kDotSmem, st>>>(
+                    rows0, N, ldt, nb, 2 * s, P->d_splT, P->d_splW, part, ntile, (int)labels);
+            }
+            DWT_CK_LAUNCH("k_spline_dots");
+            LaunchScope ls("spline_finalize", st);
+            k_spline_finalize<<<nb, kFinThreads, 0, st>>>(part, ntile, s, lg, (double)N * (double)N, thr,
+                                                          var_trc ? var_trc + b0 * (s + 1) : nullptr,
+                                                          var_sup ? var_sup + b0 * (s + 1) : nullptr,
+                                                          dim ? dim + 2 * b0 : nullptr);
         }
+        DWT_CK_LAUNCH("k_spline_finalize");
     } else {
         LaunchScope ls("spline_scale", st);
         k_spline_scale<<<grid_sp((long long)batch * N), 256, 0, st>>>(ft, cplx ? 1 : 0, N, ldt, (long long)batch * N,
                                                                      P->d_splW);
     }
-    DWT_CK_LAUNCH("k_spline_dots");
+    DWT_CK_LAUNCH("k_spline_scale");
     if (c) {
         rc = run_transform(P, ft, c, batch, ldt, ld, cplx ? DWT_C128 : DWT_F64, cplx ? DWT_C128 : DWT_F64, +1, st);
         if (rc) { cleanup(); return rc; }
     }
-    if (want_var) {
-        LaunchScope ls("spline_finalize", st);
-        k_spline_finalize<<<batch, kFinThreads, 0, st>>>(part, ntile, s, sum_rows_lanes(2 * s, ntile, kFinThreads),
-                                                         (double)N * (double)N, thr, var_trc, var_sup, dim);
-    }
-    DWT_CK_LAUNCH("k_spline_finalize");
     cleanup();
     return DWT_OK;
 }
