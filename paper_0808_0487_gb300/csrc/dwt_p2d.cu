@@ -11,10 +11,14 @@
 // of one column) share the exponent E of their largest.  Their 53-bit
 // significands are placed 30 bits above the lowest, so that a pass's stages (12
 // at most) cannot overflow 95 bits and a sign: elements down to 2^-30 of the
-// largest enter exactly, smaller ones within 2^-83 of it.
+// largest enter exactly, smaller ones lose what lies below 2^-83 of it.
 // Every result is the exact sum of those, rounded once, where FP64 stages round
-// b times at 2^-53 of the partial sums.  A tile with an infinity or a NaN runs
-// the FP64 stages; results below the normal range go through one FP64 scaling.
+// b times at 2^-53 of the partial sums.  The bits that were cut are fewer than
+// 2^b units of the sum, so they matter only to a result below 2^(52+b) units (the
+// large elements cancelled): a tile that has both is done again in levels, the
+// cut remainders transformed in their own turn until nothing is left, and no
+// result is off by more than 2^-52 of itself.  A tile with an infinity or a NaN
+// runs the FP64 stages; results below the normal range go through one FP64 scaling.
 //
 // Tiles are 2^12 elements for 256 threads, 16 elements (48 words) each:
 //   layout A  e = t + 256 r               bits 8..11 of the tile index in thread
@@ -75,12 +79,14 @@ __device__ __forceinline__ int exponent_of(uint32_t hi) { return (int)((hi >> 20
 
 constexpr int kG = 30;   // bits below the largest element's last place: 2^12 sums of 53 + 30 bits fit 95
 
-// fixed point of a double against the largest exponent E (>= 1) of its group
-__device__ __forceinline__ W96 to_fixed_any(uint32_t hi, uint32_t lo, int E) {
+// fixed point of a double against the largest exponent E (>= 1) of its group; cut:
+// set if bits below the lowest are lost
+__device__ __forceinline__ W96 to_fixed_any(uint32_t hi, uint32_t lo, int E, bool& cut) {
     const int ex = exponent_of(hi);
     uint32_t mh = hi & 0xfffffu;
     if (ex) mh |= 0x100000u;
     const int d = min(E - max(ex, 1), 95);
+    if (d > kG) cut = cut || ((((unsigned long long)mh << 32) | lo) << (64 - min(d - kG, 64))) != 0;
     W96 v;   // significand << 30, then right by d
     v.a = lo << kG;
     v.b = __funnelshift_l(lo, mh, kG);
@@ -219,6 +225,91 @@ template <int (*EL)(int, int)> __device__ __forceinline__ void get(const uint32_
     }
 }
 
+// |v| below 2^(52+B)
+template <int B> __device__ __forceinline__ bool small96(const W96& v) {
+    const W96 n = negate_if(v, (uint32_t)((int)v.c >> 31));
+    if constexpr (B >= 12) return n.c == 0;
+    else return n.c == 0 && n.b < (1u << (20 + B));
+}
+
+// element e of a tile in global memory
+template <int B> __device__ __forceinline__ long long tile_off(int e, long long S) {
+    constexpr int LC = kLT - B;
+    return B == kLT ? (long long)e : (long long)(e & ((1 << LC) - 1)) + S * (long long)(e >> LC);
+}
+
+// A whole tile in levels: the part of every element that fits the fixed point of
+// its group's largest is transformed exactly and taken off, then the next largest
+// remainders, until none is left (each level's largest lies 2^-30 below the last
+// one's at least).  Results add up in FP64 from the largest level down.
+template <int B>
+__device__ __noinline__ void tile_levels(const double* src, double* dst, long long S, int exp_shift, uint32_t* plane,
+                                         int* emax) {
+    constexpr int LC = kLT - B;
+    const int t = threadIdx.x;
+    const int top = 95 - 52 - kG + exp_shift;
+    double x[16], y[16];
+#pragma unroll
+    for (int r = 0; r < 16; ++r) {
+        x[r] = src[tile_off<B>(e_a(t, r), S)];
+        y[r] = 0.0;
+    }
+    for (;;) {
+        __syncthreads();   // the last level's exponents and planes have been read
+        if (t < (1 << LC)) emax[t] = 1;
+        __syncthreads();
+        int mx = 1;
+#pragma unroll
+        for (int r = 0; r < 16; ++r) mx = max(mx, exponent_of((uint32_t)__double2hiint(x[r])));
+        atomicMax(emax + (t & ((1 << LC) - 1)), mx);
+        __syncthreads();
+        const int E = emax[t & ((1 << LC) - 1)];
+        W96 v[16];
+        bool left = false;
+#pragma unroll
+        for (int r = 0; r < 16; ++r) {
+            const uint32_t hi = (uint32_t)__double2hiint(x[r]), lo = (uint32_t)__double2loint(x[r]);
+            bool cut = false;
+            v[r] = to_fixed_any(hi, lo, E, cut);
+            if (cut) {   // the significand's low bits, exactly
+                const int n = E - max(exponent_of(hi), 1) - kG;
+                const unsigned long long keep = n >= 53 ? 0ull : ((((unsigned long long)hi << 32) | lo) >> n) << n;
+                x[r] -= __longlong_as_double((long long)keep);
+                left = true;
+            } else {
+                x[r] = 0.0;
+            }
+        }
+        stages<0>(v);
+        if constexpr (B > 4) {
+            put<e_a>(plane, v, t);
+            __syncthreads();
+            if constexpr (B > 8) {
+                get<e_c>(plane, v, t);
+                stages<LC>(v);
+                put<e_c>(plane, v, t);
+                __syncthreads();
+            }
+            get<e_b>(plane, v, t);
+            stages<(LC > 4 ? LC - 4 : 0)>(v);
+        }
+#pragma unroll
+        for (int r = 0; r < 16; r += 4) {
+            int tops[4];
+            double z[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                tops[i] = emax[(B > 4 ? e_b(t, r + i) : e_a(t, r + i)) & ((1 << LC) - 1)] + top;
+            from_fixed4(v + r, tops, z);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) y[r + i] += z[i];
+        }
+        if (!__syncthreads_or(left)) break;
+    }
+#pragma unroll
+    for (int r = 0; r < 16; ++r) dst[tile_off<B>(B > 4 ? e_b(t, r) : e_a(t, r), S)] = y[r];
+}
+
 // One pass over 2^12-element tiles, B of the tile index's bits (the top ones)
 // transformed: B = 12 the low pass, B < 12 a high pass with 2^(12-B) columns.
 // Integer instructions bound it (ALU 72% busy at three CTAs per SM): per point 36
@@ -239,7 +330,7 @@ __global__ void __launch_bounds__(kNT, 3) k2d_pass(DArgs a) {
     const long long base = B == kLT ? tile << kLT : ((tile % nlo) << LC) + (tile / nlo) * (a.S << B);
     const double* src = a.in + blockIdx.y * a.ld_in + base;
     double* dst = a.out + blockIdx.y * a.ld_out + base;
-    auto off = [&](int e) { return B == kLT ? (long long)e : (long long)(e & ((1 << LC) - 1)) + a.S * (long long)(e >> LC); };
+    auto off = [&](int e) { return tile_off<B>(e, a.S); };
     double x[16];
 #pragma unroll
     for (int r = 0; r < 16; ++r) x[r] = src[off(e_a(t, r))];
@@ -293,6 +384,7 @@ __global__ void __launch_bounds__(kNT, 3) k2d_pass(DArgs a) {
         }
         __syncthreads();
         W96 v[16];
+        bool cut = false;
         const int E = emax[t & ((1 << LC) - 1)];
         if (__all_sync(0xffffffffu, mn >= max(1, E - kG))) {
 #pragma unroll
@@ -301,11 +393,19 @@ __global__ void __launch_bounds__(kNT, 3) k2d_pass(DArgs a) {
         } else {
 #pragma unroll
             for (int r = 0; r < 16; ++r)
-                v[r] = to_fixed_any((uint32_t)__double2hiint(x[r]), (uint32_t)__double2loint(x[r]), E);
+                v[r] = to_fixed_any((uint32_t)__double2hiint(x[r]), (uint32_t)__double2loint(x[r]), E, cut);
         }
         const int top = 95 - 52 - kG + a.exp_shift;   // + E: exponent field of bit 95
         stages<0>(v);
+        // nothing is written before this: bits cut and a result that would miss them
+        auto missed = [&]() {
+            bool lost = false;
+#pragma unroll
+            for (int r = 0; r < 16; ++r) lost = lost || small96<B>(v[r]);
+            return __syncthreads_or(lost) != 0;
+        };
         if constexpr (B == 4) {
+            if (__syncthreads_or(cut) && missed()) return tile_levels<B>(src, dst, a.S, a.exp_shift, plane, emax);
 #pragma unroll
             for (int r = 0; r < 16; r += 4) {
                 const int tops[4] = {E + top, E + top, E + top, E + top};
@@ -316,7 +416,7 @@ __global__ void __launch_bounds__(kNT, 3) k2d_pass(DArgs a) {
             }
         } else {
             put<e_a>(plane, v, t);
-            __syncthreads();
+            const bool any_cut = __syncthreads_or(cut) != 0;
             if constexpr (B > 8) {
                 get<e_c>(plane, v, t);
                 stages<LC>(v);
@@ -325,6 +425,7 @@ __global__ void __launch_bounds__(kNT, 3) k2d_pass(DArgs a) {
             }
             get<e_b>(plane, v, t);
             stages<(LC > 4 ? LC - 4 : 0)>(v);
+            if (any_cut && missed()) return tile_levels<B>(src, dst, a.S, a.exp_shift, plane, emax);
 #pragma unroll
             for (int r = 0; r < 16; r += 4) {
                 int tops[4];
