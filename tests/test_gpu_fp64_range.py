@@ -53,3 +53,25 @@ def test_small_elements_where_large_ones_cancel(dwt, dev, m, a, b):
     ref = np.array([r / one for r in ref])   # rounded correctly
     # one rounding per pass (of a column's sums) and one more where levels are added
     assert np.all(np.abs(got - ref) <= 2.0 ** -51 * np.abs(ref))
+
+
+# The columns of the high pass (one per value of the low digits) lie up to 2^-50
+# apart: one exponent for a whole tile would round them all at the largest.
+@pytest.mark.parametrize("m", [16, 20, 21])
+def test_each_column_keeps_its_own_exponent(dwt, dev, m):
+    N, low = 1 << m, 1 << 12
+    u = (S.uniform(S.stream_seed(82, S.P_VALUES, m), N) - 0.5).reshape(-1, low) * 2.0 ** -(8.0 * (np.arange(low) % 12))
+    # samples whose low pass delivers u, in whole multiples of 2^-58
+    X = np.round(_fwht(u) * 2.0 ** 46).astype(np.int64)
+    assert np.abs(X).max() < 1 << 53
+    got = _inverse(dwt, dev, m, (X * 2.0 ** -58).reshape(1, N)).reshape(-1, low)
+    # exact in two 64-bit halves, added in 80 bits
+    hi, lo = X >> 27, X & ((1 << 27) - 1)
+    ref = (_fwht(hi.reshape(1, N)).astype(np.longdouble) * 2.0 ** 27 + _fwht(lo.reshape(1, N))).reshape(-1, low) * 2.0 ** -58
+    col = np.abs(ref).max(0)
+    assert col.min() < 2.0 ** -45 * col.max()
+    # the low pass rounds each of a column's 2^b numbers at 2^-53, the high pass each
+    # result: at most 2^-53 (2^b max / largest result + 1), the largest result at least
+    # 2^(b/2) rms, so 2^-53 (2^4.5 4 + 1) < 1e-14 of the column's largest
+    err = np.abs(got - ref).max(0)
+    assert np.all(err <= 1e-14 * col), float((err / col).max())
