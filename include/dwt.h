@@ -196,7 +196,8 @@ int dwt_inverse(dwt_plan_t plan, const void *in, void *out, int batch, long long
  * p; in_t / out_t apply to every job.  The jobs' passes run as one launch per
  * pass index (the generic passes of every prime), and p = 2 F32 / I32 jobs of
  * 2^12 .. 2^14 points as one launch per size; p = 2 F32 / I32 jobs of
- * 2^16 .. 2^24 points, which fill the GPU alone, run their own launches.
+ * 2^16 .. 2^24 points, which fill the GPU alone, run their own launches; p = 2
+ * F64 jobs of 2^12 points and more as one launch per pass index of their own.
  * Jobs with batch 0 are skipped.  The host array is read before return.
  * Errors: DWT_EINVAL (NULL or empty list, a bad job, mixed p, more than
  * 2^31 - 1 blocks in one pass), DWT_EUNSUPPORTED (types), DWT_ENOMEM.

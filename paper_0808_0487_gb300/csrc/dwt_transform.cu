@@ -16,6 +16,7 @@ int p2_interpolate(dwt_plan_s* Pl, const float* f, float* c, float* coef, int ba
 bool p2d_ok(int m);
 int p2d_transform(dwt_plan_s* Pl, const double* in, double* out, int batch, long long ld_in, long long ld_out,
                   int sgn, cudaStream_t st);
+int p2d_grouped(const std::vector<GroupJob>& jobs, int sgn, cudaStream_t st);
 bool p2_small_ok(int m);
 int p2_small_interpolate(dwt_plan_s* Pl, const float* f, float* c, float* coef, int batch, long long ld,
                          bool weighted, double thr, const EffOut& o, cudaStream_t st);
@@ -71,12 +72,13 @@ int run_transform_digits(dwt_plan_s* Pl, const void* in, void* out, int batch, l
 // Grouped transforms of jobs that share p and the element types (checked by
 // the caller).  p = 2 jobs that their own call sends to the register-tile
 // kernels go there too: m = 12 .. 14 as one grouped low pass per tile size,
-// larger ones one call each; all other jobs run the generic passes grouped.
+// larger ones one call each; FP64 ones of 2^12 points and more run their integer
+// passes grouped; all other jobs run the generic passes grouped.
 int run_transform_grouped(const std::vector<GroupJob>& jobs, dwt_dtype in_t, dwt_dtype out_t, int sgn,
                           cudaStream_t st) {
     if (jobs.empty()) return DWT_OK;
     const int p = jobs[0].plan->p;
-    std::vector<GroupJob> generic, lo[3];
+    std::vector<GroupJob> generic, wide, lo[3];
     for (const GroupJob& j : jobs) {
         if (j.batch <= 0) continue;
         if (p == 2 && (in_t == DWT_F32 || in_t == DWT_I32) && p2_fast_ok(j.plan->m) && aligned16(j.in, j.ld_in, 4) &&
@@ -90,8 +92,7 @@ int run_transform_grouped(const std::vector<GroupJob>& jobs, dwt_dtype in_t, dwt
             continue;
         }
         if (p == 2 && in_t == DWT_F64 && p2d_ok(j.plan->m)) {
-            const int rc = p2d_transform(j.plan, (const double*)j.in, (double*)j.out, j.batch, j.ld_in, j.ld_out, sgn, st);
-            if (rc) return rc;
+            wide.push_back(j);
             continue;
         }
         generic.push_back(j);
@@ -101,6 +102,10 @@ int run_transform_grouped(const std::vector<GroupJob>& jobs, dwt_dtype in_t, dwt
             const int rc = p2_lo_grouped(L, lo[L - 12], in_t, sgn, st);
             if (rc) return rc;
         }
+    if (!wide.empty()) {
+        const int rc = p2d_grouped(wide, sgn, st);
+        if (rc) return rc;
+    }
     if (generic.empty()) return DWT_OK;
 #define DWT_CASE(P) case P: return grouped_p<P>(generic, in_t, out_t, sgn, st);
     switch (p) {
