@@ -688,6 +688,21 @@ static void pass_scale(PassArgs& a, double scale) {
     a.scalef = (float)scale;
 }
 
+// L2 priorities of pass t of q: the first pass reads its input, the last pass its
+// intermediate for the last time and writes final results
+static void pass_ends(PassArgs& a, int t, int q) {
+    a.in_first = t == 0 || t == q - 1;
+    a.out_first = t == q - 1;
+}
+
+// the fused top pass of an interpolation: the only pass, or between two others
+// (its results are read again by the inverse passes)
+static PassArgs mid_pass_args(int p, int km, int elem, const PassPlan& pp, const void* in, void* out, long long ld) {
+    PassArgs a = pass_args(p, km, elem, pp.g[pp.q - 1], in, out, ld, ld);
+    if (pp.q == 1) pass_ends(a, 0, 1);
+    return a;
+}
+
 static const char* pass_family(int t, int q) { return t == 0 ? "pass_lo" : (t == q - 1 ? "pass_hi" : "pass_mid"); }
 
 // threads of a pass: one per task of its first (top) group, 32 .. 512
@@ -764,14 +779,13 @@ static int transform_pp(dwt_plan_s* Pl, const PassPlan& pp, double scale_by_n, c
                 PassArgs a = pass_args(P, KMax<P, T>::v, (int)sizeof(T), g, (const TI*)in + (long long)f0 * ld_in, (T*)out + (long long)f0 * ld_out,
                                        ld_in, ld_out);
                 if (scale && pp.q == 1) pass_scale(a, scale_by_n);
-                a.in_first = 1;
-                a.out_first = pp.q == 1;
+                pass_ends(a, t, pp.q);
                 rc = launch_pass<P, T, TI, SGN>(g, a, tw, nf, pass_family(t, pp.q), st);
             } else {
                 PassArgs a = pass_args(P, KMax<P, T>::v, (int)sizeof(T), g, (const T*)out + (long long)f0 * ld_out, (T*)out + (long long)f0 * ld_out,
                                        ld_out, ld_out);
                 if (scale && t == pp.q - 1) pass_scale(a, scale_by_n);
-                a.in_first = a.out_first = t == pp.q - 1;
+                pass_ends(a, t, pp.q);
                 rc = launch_pass<P, T, T, SGN>(g, a, tw, nf, pass_family(t, pp.q), st);
             }
             if (rc) return rc;
@@ -868,6 +882,37 @@ static int launch_grouped(const std::vector<GroupPass>& h, const Tw& tw, long lo
     return DWT_OK;
 }
 
+// pass t of the jobs (those that have one): the tiles of the launch, their number,
+// and the threads and shared memory of the largest
+struct GroupLaunch {
+    std::vector<GroupPass> h;
+    long long blocks = 0;
+    int threads = 32;
+    size_t smem = 0;
+};
+template <int P, typename T>
+static GroupLaunch group_launch(const std::vector<GroupJob>& js, const std::vector<const PassPlan*>& pps, int t, bool scale) {
+    constexpr int KM = KMax<P, T>::v;
+    GroupLaunch l;
+    for (size_t i = 0; i < js.size(); ++i) {
+        const PassPlan& pp = *pps[i];
+        const GroupJob& j = js[i];
+        if (t >= pp.q || j.batch <= 0) continue;
+        const PassGeom& g = pp.g[t];
+        GroupPass gp;
+        gp.a = pass_args(P, KM, (int)sizeof(T), g, t == 0 ? j.in : j.out, j.out, t == 0 ? j.ld_in : j.ld_out, j.ld_out);
+        if (scale && t == pp.q - 1) pass_scale(gp.a, 1.0 / (double)j.plan->N);
+        pass_ends(gp.a, t, pp.q);
+        gp.ntile = g.ntile;
+        gp.first = l.blocks;
+        l.blocks += g.ntile * (long long)j.batch;
+        l.h.push_back(gp);
+        l.threads = std::max(l.threads, pass_threads<P, KM>(g));
+        l.smem = std::max(l.smem, spad_bytes<T>(g.R << g.wlog));
+    }
+    return l;
+}
+
 // The jobs' transforms by their plans' pass plans, pass t of all jobs in one
 // launch; the same tile body, geometry and scaling as transform_pp, so every
 // element equals the one of the job's own call.
@@ -875,7 +920,6 @@ template <int P, typename T, typename TI, int SGN>
 static int grouped_t(const std::vector<GroupJob>& js, cudaStream_t st) {
     static const Tw tw = make_tw(P);
     const bool scale = SGN < 0 && !std::is_same<T, int>::value;
-    constexpr int KM = KMax<P, T>::v;
     std::vector<const PassPlan*> pps;
     int qmax = 0;
     for (const GroupJob& j : js) {
@@ -883,32 +927,9 @@ static int grouped_t(const std::vector<GroupJob>& js, cudaStream_t st) {
         qmax = std::max(qmax, pps.back()->q);
     }
     for (int t = 0; t < qmax; ++t) {
-        std::vector<GroupPass> h;
-        long long blocks = 0;
-        int threads = 32;
-        size_t smem = 0;
-        for (size_t i = 0; i < js.size(); ++i) {
-            const PassPlan& pp = *pps[i];
-            const GroupJob& j = js[i];
-            if (t >= pp.q || j.batch <= 0) continue;
-            const PassGeom& g = pp.g[t];
-            GroupPass gp;
-            if (t == 0) {
-                gp.a = pass_args(P, KMax<P, T>::v, (int)sizeof(T), g, j.in, j.out, j.ld_in, j.ld_out);
-                if (scale && pp.q == 1) pass_scale(gp.a, 1.0 / (double)j.plan->N);
-            } else {
-                gp.a = pass_args(P, KMax<P, T>::v, (int)sizeof(T), g, j.out, j.out, j.ld_out, j.ld_out);
-                if (scale && t == pp.q - 1) pass_scale(gp.a, 1.0 / (double)j.plan->N);
-            }
-            gp.ntile = g.ntile;
-            gp.first = blocks;
-            blocks += g.ntile * (long long)j.batch;
-            h.push_back(gp);
-            threads = std::max(threads, pass_threads<P, KM>(g));
-            smem = std::max(smem, spad_bytes<T>(g.R << g.wlog));
-        }
-        const int rc = t == 0 ? launch_grouped<P, T, TI, SGN>(h, tw, blocks, threads, smem, "grouped_pass", st)
-                              : launch_grouped<P, T, T, SGN>(h, tw, blocks, threads, smem, "grouped_pass", st);
+        const GroupLaunch l = group_launch<P, T>(js, pps, t, scale);
+        const int rc = t == 0 ? launch_grouped<P, T, TI, SGN>(l.h, tw, l.blocks, l.threads, l.smem, "grouped_pass", st)
+                              : launch_grouped<P, T, T, SGN>(l.h, tw, l.blocks, l.threads, l.smem, "grouped_pass", st);
         if (rc) return rc;
     }
     return DWT_OK;
@@ -993,8 +1014,8 @@ static int interpolate_t(dwt_plan_s* Pl, const void* f, void* c, void* coef, int
         }
         // fused top pass
         MidArgs m;
-        if (pp.q == 1) m.pa = pass_args(P, KM, (int)sizeof(T), gm, (const TI*)f + off, (T*)c + off, ld, ld);
-        else m.pa = pass_args(P, KM, (int)sizeof(T), gm, (const T*)c + off, (T*)c + off, ld, ld);
+        m.pa = mid_pass_args(P, KM, (int)sizeof(T), pp, pp.q == 1 ? (const void*)((const TI*)f + off) : (const T*)c + off,
+                             (T*)c + off, ld);
         m.pa.scale = 1.0 / (double)Pl->N;
         m.pa.scalef = (float)m.pa.scale;
         m.W = weight == DWT_WEIGHT_INV_SQ_WAVENUMBER ? Pl->d_W : nullptr;
