@@ -150,9 +150,13 @@ def _stream(s):
     if s is None:
         # torch's current stream of its current device; once torch has initialised CUDA
         # the raw handle costs a tenth of the Stream object that current_stream() makes
+        # (both functions are torch's own; a torch without them takes the way below)
         torch = sys.modules.get("torch")
         if torch is not None and torch.cuda.is_initialized():
-            return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+            try:
+                return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+            except AttributeError:
+                pass
         try:
             import torch
             if torch.cuda.is_available():
@@ -298,7 +302,19 @@ class _Job(ctypes.Structure):
     _fields_ = [("plan", _VP), ("in_", _VP), ("out", _VP), ("batch", _I), ("ld_in", _LL), ("ld_out", _LL)]
 
 
-_JOB = struct.Struct("@PPPi4xqq")   # the layout of _Job
+def _packer(cls):
+    """struct.Struct of a ctypes structure, its padding included (packing a list of
+    jobs with it costs a fifth of building an array of ctypes structures)."""
+    fmt, end = "=", 0
+    for name, kind in cls._fields_:
+        field = getattr(cls, name)
+        fmt += "%dx" % (field.offset - end) if field.offset > end else ""
+        fmt += {_VP: "Q", _I: "i", _LL: "q"}[kind]
+        end = field.offset + field.size
+    return struct.Struct(fmt + "%dx" % (ctypes.sizeof(cls) - end))
+
+
+_JOB = _packer(_Job)
 
 
 def _jobs(jobs):
