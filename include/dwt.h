@@ -85,9 +85,10 @@ typedef struct dwt_plan_s *dwt_plan_t;
  * points in the FP32 form (real in, complex out for p > 2), for
  * N (4 + element size) <= 1 GiB, and keeps the fastest of:
  *   - the grouping of the generic passes (used for p > 2, and for p = 2
- *     outside 12 <= m <= 14, 16 <= m <= 24) and the functions per group of
- *     those passes (16, 64 or 96 MB of functions kept in L2 between the
- *     passes of a group, or 1 GB: each pass over the whole batch at once);
+ *     outside 12 <= m <= 14, 16 <= m <= 24 in FP32 and int32 and below m = 12
+ *     in FP64) and the functions per group of those passes (16, 64 or 96 MB of
+ *     functions kept in L2 between the passes of a group, or 1 GB: each pass
+ *     over the whole batch at once);
  *   - p = 2, 16 <= m <= 19: the digits of the register-tile low pass;
  *   - p = 2, m = 14 or 18 <= m <= 24: whether DWT_ALGO_AUTO runs the
  *     split-BF16 tensor-core form (results then differ from the butterflies'
@@ -119,7 +120,11 @@ int dwt_plan_info(dwt_plan_t plan, int *p, int *m, int *s, long long *N, int *ta
 /* The digit split of the generic passes for elements of elem_bytes (4: FP32
  * or int32, 8: complex FP32 or FP64, 16: complex FP64): *q passes, digits[t]
  * digits and wc[t] columns (consecutive low indices per row) in pass t, from
- * the lowest digits up.  digits and wc: host int [32]. */
+ * the lowest digits up.  Some p = 2 calls run other passes whatever this says:
+ * FP32 and int32 ones the register tiles where their rules allow it, FP64
+ * transforms of 2^12 points and more their integer passes (the 12 low digits,
+ * then the others in passes of at most 9; dwt_forward_digits and
+ * dwt_inverse_digits run the generic ones).  digits and wc: host int [32]. */
 int dwt_plan_passes(dwt_plan_t plan, int elem_bytes, int *q, int *digits, int *wc);
 
 /* The measured choices of a DWT_PLAN_TUNE plan (0 where the heuristic stays):
