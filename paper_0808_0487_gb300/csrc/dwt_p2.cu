@@ -131,8 +131,10 @@ struct HiArgs {
 };
 
 // CTAs per SM: three of the plain pass (80 registers), but two where rows are 64
-// bytes (B = 10: m = 24, 32 functions 1462 us with two, 1538 us with three; B = 6:
-// m = 20 87 and 84 us; B = 9: m = 23 185 and 170 us).
+// bytes.  Two and three: B = 10 (m = 24, 4 functions) 182.5 and 193.0 us, B = 9
+// (m = 23, 8) 179.5 and 167.4, B = 8 (m = 22, 16) 174.3 and 172.7, B = 7 (m = 21, 32)
+// 172.4 and 166.7, B = 6 (m = 20, 32) 85.7 and 83.2, B = 5 (m = 19, 65) 88.6 and 88.6,
+// B = 4 (m = 18, 100) 61.8 and 61.7; int32 within 1% up to B = 9.
 template <typename T, int LT, int B, bool FUSED, bool HAS_COEF>
 __global__ void __launch_bounds__(1 << (LT - 6), FUSED ? 4 : B == 10 ? 2 : 3) k2_hi(HiArgs a) {
     static_assert(B >= 4 && B <= 10 && LT - B >= 2, "high-pass shape");
@@ -461,10 +463,13 @@ static int launch_hi_t(int B, const HiArgs& a, int nf, size_t bins_bytes, const 
 }
 
 // Bytes of functions per group: the passes of a group run back to back so that
-// the intermediate stays in L2 between them.  p = 2, m = 20, 32 functions,
-// 48 / 64 / 80 / 96 MB: forward 97 / 90 / 97 / 100 us, int32 88 / 80 / 84 / 92,
-// interpolation 185 / 176 / 182 / 188; m = 24 (64 MB per function): the same up
-// to 112 MB, slower from two functions on.
+// the intermediate stays in L2 between them; the last group may hold half as much
+// again (group_size).  Groups of 48 / 64 / 80 / 96 MB with a short last one, and
+// of 64 MB so: p = 2, m = 20, forward of 32 functions 93 / 83 / 87 / 89 and 83 us,
+// 17 52 / 51 / 46 / 46 and 46, 33 93 / 92 / 88 / 90 and 88, 50 146 / 134 / 135 / 137
+// and 131; interpolation of 32 172 / 167 / 176 / 181 and 168; m = 19, 33 forward
+// 44 / 46 / 39 / 39 and 39, interpolations 87 / 91 / 81 / 81 and 81; m = 22, 9
+// 105 / 100 / 97 / 100 and 97 (int32 alike).  m = 24 takes one function per group.
 static const long long kL2GroupP2 = 64ll << 20;
 
 // forward (sgn < 0, scaled by 2^-m for FP32) or inverse transform, FP32 or int32
@@ -477,9 +482,9 @@ static int p2_transform_t(dwt_plan_s* Pl, const T* in, T* out, int batch, long l
     const float sc = (float)(1.0 / (double)N);
     const long long fbytes = N * (long long)sizeof(T);
     int G = (int)std::max(1ll, kL2GroupP2 / fbytes);
-    G = std::min(G, 65535);
-    for (int f0 = 0; f0 < batch; f0 += G) {
-        const int nf = std::min(G, batch - f0);
+    G = std::min(G, 43690);   // a last group of G + G / 2 fits a grid
+    for (int f0 = 0, nf; f0 < batch; f0 += nf) {
+        nf = group_size(batch - f0, G);
         const T* src = in + (long long)f0 * ld_in;
         T* dst = out + (long long)f0 * ld_out;
         if (m <= 14) {
@@ -608,7 +613,7 @@ int p2_interpolate(dwt_plan_s* Pl, const float* f, float* c, float* coef, int ba
     double* part = (double*)Pl->d_ws;
     const long long fbytes = N * 4;
     int G = (int)std::max(1ll, kL2GroupP2 / fbytes);
-    G = std::min(G, 65535);
+    G = std::min(G, 43690);   // a last group of G + G / 2 fits a grid
     // low passes: FP32 register tiles, or (tc) the split-BF16 tensor-core tiles
     int* err = nullptr;
     if (tc) {
@@ -635,10 +640,10 @@ int p2_interpolate(dwt_plan_s* Pl, const float* f, float* c, float* coef, int ba
     };
     // forward low pass of the first group; then per group: fused top pass, and one
     // launch holding this group's inverse low pass and the next group's forward
-    rc = low(f, c, std::min(G, batch), false, nullptr, nullptr, 0, "interp_fwd");
+    rc = low(f, c, group_size(batch, G), false, nullptr, nullptr, 0, "interp_fwd");
     if (rc) return rc;
-    for (int f0 = 0; f0 < batch; f0 += G) {
-        const int nf = std::min(G, batch - f0);
+    for (int f0 = 0, nf; f0 < batch; f0 += nf) {
+        nf = group_size(batch - f0, G);
         const long long off = (long long)f0 * ld;
         HiArgs a{};
         a.in = c + off;
@@ -658,10 +663,10 @@ int p2_interpolate(dwt_plan_s* Pl, const float* f, float* c, float* coef, int ba
         rc = coef ? launch_hi_t<float, LT, true, true>(B, a, nf, bins_bytes, "interp_top", st)
                   : launch_hi_t<float, LT, true, false>(B, a, nf, bins_bytes, "interp_top", st);
         if (rc) return rc;
-        const int g1 = f0 + G;
+        const int g1 = f0 + nf;
         if (g1 < batch) {
             const long long off1 = (long long)g1 * ld;
-            rc = low(c + off, c + off, nf, true, f + off1, c + off1, std::min(G, batch - g1), "interp_inv_fwd");
+            rc = low(c + off, c + off, nf, true, f + off1, c + off1, group_size(batch - g1, G), "interp_inv_fwd");
         } else {
             rc = low(c + off, c + off, nf, true, nullptr, nullptr, 0, "interp_inv");
         }

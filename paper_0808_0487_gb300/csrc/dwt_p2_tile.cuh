@@ -210,4 +210,8 @@ __device__ __forceinline__ void bin_group(float* bt, float* bs, uint2 c, const f
     bin_pair(bt, bs, c.y, q[2], q[3]);
 }
 
+// functions of the next group when `left` are to be done in groups of G: up to half
+// a group more at the end, instead of a short one whose launches leave SMs idle
+static inline int group_size(int left, int G) { return left <= G + G / 2 ? left : G; }
+
 }  // namespace dwt

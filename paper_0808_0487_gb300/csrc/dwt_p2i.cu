@@ -684,7 +684,7 @@ int p2i_interpolate(dwt_plan_s* Pl, const float* f, float* c, float* coef, int b
     if (rc) return rc;
     double* part = (double*)Pl->d_ws;
     int G = (int)std::max(1ll, kL2GroupP2i / (N * 4));
-    G = std::min(G, 65535);
+    G = std::min(G, 43690);   // a last group of G + G / 2 fits a grid
     int* err = nullptr;
     if (tc) {
         if (!tc_ok(m)) {
@@ -706,10 +706,10 @@ int p2i_interpolate(dwt_plan_s* Pl, const float* f, float* c, float* coef, int b
         LoJobI b{i1, o1, ld, n1, 0};
         return launch_lo_i(a, i1 ? &b : nullptr, N, fam, st);
     };
-    rc = low(f, c, std::min(G, batch), false, nullptr, nullptr, 0, "interp_fwd");
+    rc = low(f, c, group_size(batch, G), false, nullptr, nullptr, 0, "interp_fwd");
     if (rc) return rc;
-    for (int f0 = 0; f0 < batch; f0 += G) {
-        const int nf = std::min(G, batch - f0);
+    for (int f0 = 0, nf; f0 < batch; f0 += nf) {
+        nf = group_size(batch - f0, G);
         const long long off = (long long)f0 * ld;
         TopArgs a{};
         a.scale = (float)(1.0 / (double)N);
@@ -727,10 +727,10 @@ int p2i_interpolate(dwt_plan_s* Pl, const float* f, float* c, float* coef, int b
         a.err = Pl->d_err;
         rc = launch_top(B, c + off, ld, nf, a, Pl->s, st);
         if (rc) return rc;
-        const int g1 = f0 + G;
+        const int g1 = f0 + nf;
         if (g1 < batch) {
             const long long off1 = (long long)g1 * ld;
-            rc = low(c + off, c + off, nf, true, f + off1, c + off1, std::min(G, batch - g1), "interp_inv_fwd");
+            rc = low(c + off, c + off, nf, true, f + off1, c + off1, group_size(batch - g1, G), "interp_inv_fwd");
         } else {
             rc = low(c + off, c + off, nf, true, nullptr, nullptr, 0, "interp_inv");
         }
