@@ -23,6 +23,7 @@
 // DWTs are real up to rounding).  dwt_spline then transforms each function,
 // multiplies by W_K, contracts |c~|^2 with the tables in a fixed summation
 // order, and transforms back.
+#include <cooperative_groups.h>
 #include <cuda_fp16.h>
 #include <math.h>
 #include <string.h>
@@ -136,9 +137,10 @@ __global__ void k_spline_scale(double* ft, int cplx, long long N, long long ld, 
 //
 // Integer instructions and the tensor cores bound it, a fifth goes to the sums
 // formed again.  p = 2, m = 20, s = 16, 32 functions: 2920 us on the FP64 pipe (one
-// CTA per function and 4096 labels) plus 95 us for the scaling; so 623 us
-// (535 without the sums formed again; with every warp forming its own again, in
-// tiles of 512 labels, 763).  Eight digits, 36 pairs and no second look took
+// CTA per function and 4096 labels) plus 95 us for the scaling; so 608 us,
+// 535 of them without the sums formed again (pair by pair instead of function by
+// function 623; the next block's numbers loaded before this one's sums are drained,
+// which takes 130 registers and spills, 708).  Eight digits, 36 pairs and no second look took
 // 364 us and were wrong by up to 2^-16 of a variance (random values, s = 2, m = 16).
 constexpr int kDotThreads = 256;
 constexpr int kDotRows = 32;                  // functions, and tables, per round
@@ -146,7 +148,7 @@ constexpr int kDotK = 64;                     // labels per block
 constexpr int kDotPlane = kDotRows * kDotK;   // halves of one digit's rows
 constexpr int kDotDigits = 12;
 constexpr int kDotOperand = kDotDigits * kDotPlane;   // halves of one operand
-constexpr size_t kDotSmem = (size_t)2 * kDotOperand * 2 + 6 * kDotRows * 4 + 16;
+constexpr size_t kDotSmem = (size_t)2 * kDotOperand * 2 + 7 * kDotRows * 4 + 16;
 constexpr int kDotKeep = 60;                  // log2 of the least sum per label that is kept
 
 __device__ __forceinline__ uint32_t abs_hi(double x) { return (uint32_t)__double2hiint(x) & 0x7fffffffu; }
@@ -230,34 +232,46 @@ __device__ __forceinline__ void mma_f16(float (&d)[4], const uint32_t (&a)[4], u
         : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
-// sum over [h0, h1) of |c~|^2 T in FP64 by one warp: four chains per lane (the
-// additions take 64 cycles), then trees; eight pairs of loads in flight
+// sums over [h0, h1) of |c~|^2 T_t in FP64 by one warp, for the tables t of a mask:
+// 256 labels at a time, their squares kept in registers for all tables; two chains
+// per lane, then a tree.  Lane t returns table t's sum.
 template <bool CPLX>
-__device__ __forceinline__ double warp_sum(const double* c, const double* T, long long h0, long long h1, int lane) {
-    double v[4] = {0.0, 0.0, 0.0, 0.0};
-    for (long long H = h0 + lane; H < h1; H += 256) {
-        double x[8], y[8];
+__device__ __forceinline__ double warp_sums(const double* c, const double* tab, long long N, unsigned mask, long long h0,
+                                            long long h1, int lane) {
+    double tot = 0.0;
+    for (long long H = h0 + lane; H - lane < h1; H += 256) {
+        double a[8];
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
             const long long h = H + 32 * i;
-            x[i] = y[i] = 0.0;
+            a[i] = 0.0;
             if (h >= h1) continue;
             if constexpr (CPLX) {
                 const double2 u = reinterpret_cast<const double2*>(c)[h];
-                x[i] = u.x * u.x + u.y * u.y;
+                a[i] = u.x * u.x + u.y * u.y;
             } else {
-                x[i] = c[h];
+                a[i] = c[h] * c[h];
             }
-            y[i] = T[h];
         }
+        for (unsigned m = mask; m; m &= m - 1) {
+            const int tr = __ffs((int)m) - 1;
+            const double* T = tab + (long long)tr * N;
+            double y[8];
 #pragma unroll
-        for (int i = 0; i < 8; ++i)
-            if (H + 32 * i < h1) v[i & 3] += (CPLX ? x[i] : x[i] * x[i]) * y[i];
+            for (int i = 0; i < 8; ++i) y[i] = H + 32 * i < h1 ? T[H + 32 * i] : 0.0;
+            double v0 = a[0] * y[0], v1 = a[1] * y[1];
+#pragma unroll
+            for (int i = 2; i < 8; i += 2) {
+                v0 += a[i] * y[i];
+                v1 += a[i + 1] * y[i + 1];
+            }
+            v0 += v1;
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) v0 += __shfl_xor_sync(0xffffffffu, v0, o);
+            if (lane == tr) tot += v0;
+        }
     }
-    double x = (v[0] + v[1]) + (v[2] + v[3]);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-    return x;
+    return tot;
 }
 
 // grid (tiles, groups of 32 functions); warp w converts rows 4 w .. 4 w + 3 of
@@ -268,13 +282,14 @@ __global__ void __launch_bounds__(kDotThreads, 2) k_spline_dots(double* ct, long
                                                                 const double* __restrict__ tab,
                                                                 const double* __restrict__ W, double* part, int ntile,
                                                                 int labels) {
-    extern __shared__ __align__(128) unsigned char smraw[];
+    extern __shared__ __align__(16) unsigned char smraw[];
     __half* A = reinterpret_cast<__half*>(smraw);
     __half* B = A + kDotOperand;
     int* grow = reinterpret_cast<int*>(B + kDotOperand);   // [2][32]: growth of the rows' exponents in this block
     int* bad = grow + 2 * kDotRows;                        // [2][32]: rows with an infinity or a NaN
     int* some = bad + 2 * kDotRows;                        // [2][32]: rows with a number other than zero
-    int* again = some + 2 * kDotRows;                      // sums to form again
+    unsigned* fails = reinterpret_cast<unsigned*>(some + 2 * kDotRows);   // [32]: a function's sums to form again
+    int* next = reinterpret_cast<int*>(fails + kDotRows);
     const int t = threadIdx.x, lane = t & 31, w = t >> 5;
     const int tile = blockIdx.x, f0 = blockIdx.y * kDotRows;
     const long long h0 = (long long)tile * labels, h1 = min(N, h0 + labels);
@@ -458,9 +473,9 @@ __global__ void __launch_bounds__(kDotThreads, 2) k_spline_dots(double* ct, long
             }
         }
         if (lane < 8) some[(lane >> 2) * kDotRows + 4 * w + (lane & 3)] = (any >> lane) & 1;
-        if (t == 0) *again = 0;
+        if (t < kDotRows) fails[t] = 0;
+        if (t == 0) *next = 0;
         __syncthreads();   // bad and some are complete, c~ of the tile is written
-        uint16_t* list = reinterpret_cast<uint16_t*>(smraw);   // pairs to form again, in the digits' place
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
             const int fr = fo + (lane >> 2) + 8 * (q >> 1), tr = to + 2 * (lane & 3) + (q & 1);
@@ -477,14 +492,20 @@ __global__ void __launch_bounds__(kDotThreads, 2) k_spline_dots(double* ct, long
                 if (!some[fr] || !some[kDotRows + tr]) v = 0.0;
                 else redo = sum < ((__int128)(h1 - h0) << kDotKeep);
             }
-            if (redo) list[atomicAdd(again, 1)] = (uint16_t)(fr * kDotRows + tr);
+            if (redo) atomicOr(fails + fr, 1u << tr);
             else part[((long long)f * nt + tb) * ntile + tile] = v;
         }
         __syncthreads();
-        for (int i = w; i < *again; i += kDotThreads / 32) {
-            const int f = f0 + list[i] / kDotRows, tb = t0 + list[i] % kDotRows;
-            const double v = warp_sum<CPLX>(ct + (long long)f * ld * (CPLX ? 2 : 1), tab + (long long)tb * N, h0, h1, lane);
-            if (lane == 0) part[((long long)f * nt + tb) * ntile + tile] = v;
+        for (;;) {   // the functions with sums to form again, one warp each
+            int fr = 0;
+            if (lane == 0) fr = atomicAdd(next, 1);
+            fr = __shfl_sync(0xffffffffu, fr, 0);
+            if (fr >= kDotRows) break;
+            const unsigned mask = fails[fr];
+            if (!mask) continue;
+            const long long f = f0 + fr;
+            const double v = warp_sums<CPLX>(ct + f * ld * (CPLX ? 2 : 1), tab + (long long)t0 * N, N, mask, h0, h1, lane);
+            if ((mask >> lane) & 1) part[(f * nt + t0 + lane) * ntile + tile] = v;
         }
     }
 }
@@ -538,19 +559,31 @@ __global__ void __launch_bounds__(kFewThreads) k_spline_dots_fp64(double* ct, lo
 }
 
 // sums over tiles, then the cumulative variances and dimensions (least d with
-// variance >= thr * total, 0 when the total is 0): one CTA per function.  The
-// FP64 additions of its 2 s ntile partials bound it (p = 2, m = 20, s = 16, 32
-// functions: 553 us with one thread per function, 9 us so).
+// variance >= thr * total, 0 when the total is 0): one CTA per function, or a
+// cluster whose sums meet in the first CTA's shared memory.  The FP64 additions of
+// the 2 s ntile partials bound it (p = 2, m = 20, s = 16, 32 functions, 4096 tiles:
+// 48 us with one CTA, 23 us in a cluster of eight).
 constexpr int kFinThreads = 512;
+template <int CL>
 __global__ void __launch_bounds__(kFinThreads) k_spline_finalize(const double* __restrict__ part, int ntile, int s,
                                                                  int lg, double N2, double thr, double* var_trc,
                                                                  double* var_sup, int* dim) {
+    namespace cg = cooperative_groups;
     __shared__ double x[2 * kSplineMaxS];
     __shared__ double v[2][kSplineMaxS + 1];
     __shared__ int first[2];
-    const long long b = blockIdx.x;
-    const int t = threadIdx.x;
-    sum_rows(part + b * 2 * s * ntile, 2 * s, ntile, lg, 0, 1, x);
+    const long long b = blockIdx.x / CL;
+    const int t = threadIdx.x, rank = blockIdx.x % CL;
+    double* dst = x;
+    if constexpr (CL > 1) {
+        dst = cg::this_cluster().map_shared_rank(x, 0);
+        cg::this_cluster().sync();   // the first CTA is running before its shared memory is written
+    }
+    sum_rows(part + b * 2 * s * ntile, 2 * s, ntile, lg, rank, CL, dst);
+    if constexpr (CL > 1) {
+        cg::this_cluster().sync();
+        if (rank != 0) return;
+    }
     if (t < 2) first[t] = s;
     __syncthreads();
     if (t == 0) {
@@ -1026,6 +1059,30 @@ int run_spline_eval(dwt_plan_s* P, const void* c, int batch, long long ld, const
     return DWT_OK;
 }
 
+template <int CL>
+static int launch_finalize_cl(const double* part, int nb, int ntile, int s, double N2, double thr, double* vt, double* vs,
+                              int* dim, cudaStream_t st) {
+    LaunchScope ls("spline_finalize", st);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)nb * CL);
+    cfg.blockDim = dim3(kFinThreads);
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim = {CL, 1, 1};
+    cfg.attrs = at;
+    cfg.numAttrs = CL > 1 ? 1 : 0;
+    const int lg = sum_rows_lanes((2 * s + CL - 1) / CL, ntile, kFinThreads);
+    DWT_CK(cudaLaunchKernelEx(&cfg, k_spline_finalize<CL>, part, ntile, s, lg, N2, thr, vt, vs, dim));
+    return DWT_OK;
+}
+// a cluster from 2049 partials per function, as in effdim_reduce
+static int launch_finalize(const double* part, int nb, int ntile, int s, double N2, double thr, double* vt, double* vs,
+                           int* dim, cudaStream_t st) {
+    return 2ll * s * ntile <= 2048 ? launch_finalize_cl<1>(part, nb, ntile, s, N2, thr, vt, vs, dim, st)
+                                   : launch_finalize_cl<8>(part, nb, ntile, s, N2, thr, vt, vs, dim, st);
+}
+
 int run_spline(dwt_plan_s* P, const double* f, void* c, int batch, long long ld, double* var_trc, double* var_sup,
                int* dim, double thr, cudaStream_t st) {
     if (!P->d_splW) {
@@ -1055,8 +1112,8 @@ int run_spline(dwt_plan_s* P, const double* f, void* c, int batch, long long ld,
     // labels per tile, from the net alone: a function's sums do not depend on the
     // others of its call.  Tiles for two CTAs per SM of one group; in digits at most
     // 256 labels (the sums that are formed again in FP64 find the tile in L2, fewer
-    // fail and no SM is left with a long list: p = 2, 32 functions of s = 16,
-    // contraction of smooth functions, 2048 / 1024 / 512 / 256 labels: m = 20
+    // fail and no SM is left with a long list: p = 2, 32 functions of s = 16, pair by
+    // pair, contraction of smooth functions, 2048 / 1024 / 512 / 256 labels: m = 20
     // 880 / 744 / 651 / 623 us, m = 18 - / 286 / 221 / 174, random values 1418 / 878 /
     // 707 / 638 and - / 509 / 368 / 267) or 16 s, so that the tiles' sums take a byte
     // per point at most; in FP64 between 256 and 2048
@@ -1082,7 +1139,6 @@ int run_spline(dwt_plan_s* P, const double* f, void* c, int batch, long long ld,
         auto kern = cplx ? k_spline_dots<true> : k_spline_dots<false>;
         auto kern64 = cplx ? k_spline_dots_fp64<true> : k_spline_dots_fp64<false>;
         if ((rc = smem_limit_max(kern))) { cleanup(); return rc; }
-        const int lg = sum_rows_lanes(2 * s, ntile, kFinThreads);
         for (long long b0 = 0; b0 < batch; b0 += chunk) {
             const int nb = (int)std::min<long long>(chunk, batch - b0);
             double* rows0 = ft + b0 * ldt * (cplx ? 2 : 1);
@@ -1096,13 +1152,11 @@ int run_spline(dwt_plan_s* P, const double* f, void* c, int batch, long long ld,
                     rows0, N, ldt, nb, 2 * s, P->d_splT, P->d_splW, part, ntile, (int)labels);
             }
             DWT_CK_LAUNCH("k_spline_dots");
-            LaunchScope ls("spline_finalize", st);
-            k_spline_finalize<<<nb, kFinThreads, 0, st>>>(part, ntile, s, lg, (double)N * (double)N, thr,
-                                                          var_trc ? var_trc + b0 * (s + 1) : nullptr,
-                                                          var_sup ? var_sup + b0 * (s + 1) : nullptr,
-                                                          dim ? dim + 2 * b0 : nullptr);
+            double* vt = var_trc ? var_trc + b0 * (s + 1) : nullptr;
+            double* vs = var_sup ? var_sup + b0 * (s + 1) : nullptr;
+            rc = launch_finalize(part, nb, ntile, s, (double)N * (double)N, thr, vt, vs, dim ? dim + 2 * b0 : nullptr, st);
+            if (rc) { cleanup(); return rc; }
         }
-        DWT_CK_LAUNCH("k_spline_finalize");
     } else {
         LaunchScope ls("spline_scale", st);
         k_spline_scale<<<grid_sp((long long)batch * N), 256, 0, st>>>(ft, cplx ? 1 : 0, N, ldt, (long long)batch * N,
