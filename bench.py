@@ -296,9 +296,9 @@ def accuracy_vs_oracle(acc_in, f):
 # that source makes the figures stale: they are then reported as null.
 MEASURED_TRAFFIC = {
     "source": "paper_0808_0487_gb300/csrc/dwt_p2i.cu",
-    "sha256": "ce189fa2289c2e643514c309a17258d9b1e6232015091b8b5cf3fbe5312cd07d",
-    # top pass: mean of two launches (80.2 and 104.8 MB); paired low pass: one launch
-    "bytes_per_launch": {"interp_top": 92.5e6, "interp_inv_fwd": 140.2e6},
+    "sha256": "e7d4219058f18be3cf723b5442fe129f43091cd8a3c0e37dc408ff42901bd740",
+    # top pass: mean of two launches (84.3 and 101.4 MB); paired low pass: one launch
+    "bytes_per_launch": {"interp_top": 92.8e6, "interp_inv_fwd": 138.0e6},
 }
 
 

@@ -513,9 +513,10 @@ long long dwt_alloc_count(void);
  * Families: p = 2 register tiles "p2_lo_fwd", "p2_lo_inv", "p2_hi_fwd",
  * "p2_hi_inv"; p = 2 interpolation "interp_fwd", "interp_top", "interp_inv",
  * "interp_inv_fwd" (two low passes in one launch), "interp_small" (2^8 .. 2^14
- * points in one launch); tensor-core tiles
- * "tc_lo14"; generic passes "pass_lo", "pass_mid", "pass_hi"; variance classes
- * "effdim_bins", "effdim_reduce"; index maps "points",
+ * points in one launch); tensor-core tiles "tc_lo14"; generic and FP64 passes
+ * "pass_lo", "pass_mid", "pass_hi"; grouped calls "grouped_lo", "grouped_pass";
+ * variance classes "effdim_bins", "effdim_reduce"; kernel spline "spline_dots",
+ * "spline_dots_fp64", "spline_scale", "spline_finalize"; index maps "points",
  * "k_to_h", "h2k_recon", "h2k_copy"; plan build "dp_init", "dp_step",
  * "dp_check", "dp_prefix", "dp_recon", "dp_weights", "dp_small",
  * "tile_tables", "tree_maps", "tree_one", "tree_sweep", "tree_reps",

@@ -317,7 +317,8 @@ __device__ __noinline__ void tile_levels(const double* src, double* dst, long lo
 // of the additions, about 50 of the conversions and exchanges.  32 functions of
 // 2^20 points: 1660 us on the FP64 pipe; so, with the
 // short conversions 306 us, without groups of functions 270, with one vote per
-// four results 256 (random values) and 274 (coefficients of a smooth function).
+// four results 256 (random values) and 274 (coefficients of a smooth function);
+// with the votes on cut bits 255 .. 259 (m = 24, 2 functions 369 -> 374).
 template <int B> __device__ __forceinline__ void pass_tile(const DArgs& a, long long tile, long long fn) {
     constexpr int LC = kLT - B;          // column bits
     extern __shared__ __align__(16) unsigned char smraw[];
